@@ -70,7 +70,13 @@ typedef enum {
 } fbcorr_status_t;
 
 /* Arithmetic of the forward pass; tensors are FP32 in every mode.
- *  F32    : FP32 products, FP32 accumulation (CUDA cores).
+ *  F32    : FP32 products and accumulation: FP32 FMAs on the CUDA cores, or, where
+ *           it is faster and the caller passes scratch (fbcorr_plan_scratch_size),
+ *           the tensor cores on an exact three-way split v = v1 + v2 + v3 into BF16
+ *           (24 bits; six of the nine products, the rest below 2^-26 of x w; short
+ *           sums in the tensor core added up in FP32).  Its error against 64 bits
+ *           is at or below the FMA kernels'; non-finite and out-of-range values give
+ *           what the FMA kernels give.
  *  BF16   : x and w rounded to BF16 (round-to-nearest-even), BF16 x BF16
  *           products with FP32 accumulation on the tcgen05 tensor cores.
  *  BF16X3 : "split BF16": v = hi + lo with hi = bf16(v), lo = bf16(v - hi);
@@ -133,6 +139,14 @@ fbcorr_status_t fbcorr_plan_out_shape(fbcorr_plan_t plan, int64_t out[3]);
  * may be NULL).  Zero means the call accepts ws = NULL. */
 fbcorr_status_t fbcorr_plan_workspace_size(fbcorr_plan_t plan, size_t* fwd_bytes,
                                            size_t* bwd_bytes);
+
+/* Bytes of device workspace with which forward and backward run their fastest
+ * kernels (either pointer may be NULL): at least the sizes above.  FP32 plans
+ * need none for the forward, but given this much they may run it -- and, in
+ * every plan, dL/dx -- on the tensor cores (each FP32 value split exactly into
+ * three BF16 values); with less they run FP32 FMA kernels.  The size may change
+ * with fbcorr_autotune and fbcorr_plan_set_variant. */
+fbcorr_status_t fbcorr_plan_scratch_size(fbcorr_plan_t plan, size_t* fwd_bytes, size_t* bwd_bytes);
 
 /* y = epi(corr(x, w)).  x, w, y: device pointers as above; ws: device
  * workspace of at least the forward size (NULL allowed when it is zero).

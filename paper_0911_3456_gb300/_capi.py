@@ -53,6 +53,7 @@ PROTOTYPES = {
     "fbcorr_plan_destroy": (_st, [_vp]),
     "fbcorr_plan_out_shape": (_st, [_vp, I64_3]),
     "fbcorr_plan_workspace_size": (_st, [_vp, ctypes.POINTER(_sz), ctypes.POINTER(_sz)]),
+    "fbcorr_plan_scratch_size": (_st, [_vp, ctypes.POINTER(_sz), ctypes.POINTER(_sz)]),
     "fbcorr_forward": (_st, [_vp, _vp, _vp, _vp, _vp, _sz, _vp]),
     "fbcorr_forward_host": (_st, [_vp, _vp, _vp, _vp, ctypes.c_int, _vp]),
     "fbcorr_plan_create_snippet": (_st, [ctypes.POINTER(_vp), I64_3, I64_4, ctypes.c_int, Epilogue, ctypes.c_char_p]),

@@ -87,6 +87,7 @@ class Plan:
         C.call("fbcorr_plan_workspace_size", h, ctypes.byref(fwd), ctypes.byref(bwd))
         self.ws_fwd, self.ws_bwd = fwd.value, bwd.value
         self._ws = {}
+        self._scratch = {}
 
     # -- lifetime
     def close(self) -> None:
@@ -115,6 +116,25 @@ class Plan:
             self._ws[key] = ws
         return ws
 
+    # -- optional scratch of the FP32 tensor-core kernels: from PyTorch's allocator on
+    # the call's stream, call by call, so that FP32 calls of one plan may overlap on
+    # several streams and threads
+    def _scratch_size(self, backward: bool) -> int:
+        n = self._scratch.get(backward)
+        if n is None:
+            out = ctypes.c_size_t()
+            fwd, bwd = (None, ctypes.byref(out)) if backward else (ctypes.byref(out), None)
+            C.call("fbcorr_plan_scratch_size", self._h, fwd, bwd)
+            n = self._scratch[backward] = out.value
+        return n
+
+    @staticmethod
+    def _scratch_tensor(nbytes: int, device, stream) -> torch.Tensor:
+        if stream is None:
+            return torch.empty(nbytes, dtype=torch.uint8, device=device)
+        with torch.cuda.stream(stream):
+            return torch.empty(nbytes, dtype=torch.uint8, device=device)
+
     # -- calls
     def forward(self, x: torch.Tensor, w: torch.Tensor, y: Optional[torch.Tensor] = None,
                 ws: Optional[torch.Tensor] = None, stream=None) -> torch.Tensor:
@@ -124,7 +144,10 @@ class Plan:
             y = torch.empty(self.out_shape, dtype=torch.float32, device=x.device)
         _check_tensor(y, "y", self.out_shape)
         if ws is None:
-            ws = self.workspace(self.ws_fwd, x.device)
+            if self.ws_fwd:
+                ws = self.workspace(self.ws_fwd, x.device)
+            elif self._scratch_size(False):
+                ws = self._scratch_tensor(self._scratch[False], x.device, stream)
         nbytes = ws.numel() * ws.element_size() if ws is not None else 0
         C.call("fbcorr_forward", self._h, _vp(x), _vp(w), _vp(y), _vp(ws), nbytes,
                _stream_handle(stream))
@@ -157,8 +180,12 @@ class Plan:
         dev = g.device
         dx = torch.empty(self.in_shape, dtype=torch.float32, device=dev) if need_dx else None
         dw = torch.empty(self.filt_shape, dtype=torch.float32, device=dev) if need_dw else None
-        if ws is None and need_dw:
-            ws = self.workspace(self.ws_bwd, dev)
+        if ws is None and (need_dx or need_dw):
+            scratch = self._scratch_size(True)
+            if need_dx and scratch > self.ws_bwd:
+                ws = self._scratch_tensor(scratch, dev, stream)
+            elif need_dw:
+                ws = self.workspace(self.ws_bwd, dev)
         nbytes = ws.numel() * ws.element_size() if ws is not None else 0
         C.call("fbcorr_backward", self._h, _vp(x if need_dw else None), _vp(w if need_dx else None),
                _vp(g), _vp(y), _vp(dx), _vp(dw), _vp(ws), nbytes, _stream_handle(stream))
@@ -166,6 +193,7 @@ class Plan:
 
     def autotune(self, stream=None) -> None:
         C.call("fbcorr_autotune", self._h, _stream_handle(stream))
+        self._scratch = {}
 
     def candidates(self):
         """The forward variants the auto-tuner times for this plan (spec strings)."""
@@ -175,6 +203,7 @@ class Plan:
 
     def set_variant(self, spec: str) -> None:
         C.call("fbcorr_plan_set_variant", self._h, spec.encode())
+        self._scratch = {}
 
     def info(self) -> dict:
         buf = ctypes.create_string_buffer(8192)

@@ -80,6 +80,7 @@ const char* kind_name(VarKind k) {
         case VarKind::Default: return "default";
         case VarKind::Direct: return "direct";
         case VarKind::Tensor: return "tcgen05";
+        case VarKind::F32tc: return "f32tc";
     }
     return "?";
 }
@@ -89,6 +90,14 @@ std::string shape_key(const fbcorr_plan* p, const char* what) {
     o << what << "|x" << p->H << "x" << p->W << "x" << p->D << "|w" << p->N << "x" << p->fh << "x"
       << p->fw << "|dt" << (int)p->dtype << "|epi" << p->epi.kind;
     return o.str();
+}
+
+// The spec of the variant an untuned FP32 problem takes: the tensor-core kernel
+// where the model expects it to win over the FMA kernels.
+std::string heuristic_spec(const DirectProblem& pr, const DeviceInfo& dev) {
+    F3Tile f3;
+    if (f3_wins(pr, dev.sm_count, &f3)) return f3_spec(f3);
+    return direct_tile_spec(direct_heuristic(pr, smem_limit(dev), dev.sm_count));
 }
 
 // Select the forward variant of an F32 plan from a spec string.
@@ -101,10 +110,25 @@ fbcorr_status_t set_fwd_spec(fbcorr_plan* p, const std::string& spec, const char
         p->fwd_source = source;
         return FBCORR_OK;
     }
+    const DirectProblem pr = fwd_problem(p);
+    F3Tile f3;
+    if (f3_parse_spec(spec, &f3)) {
+        F3Launch l;
+        FBC_TRY(f3_build(pr, f3, p->dev.sm_count, &l));
+        // and the FMA kernel that calls without scratch run
+        const DirectTile dt = direct_heuristic(pr, smem_limit(p->dev), p->dev.sm_count);
+        Kernel k;
+        FBC_TRY(build_direct(pr, dt, &k));
+        p->fwd_kind = VarKind::F32tc;
+        p->fwd_f3 = l;
+        p->fwd_tile = dt;
+        p->fwd_kernel = k;
+        p->fwd_source = source;
+        return FBCORR_OK;
+    }
     DirectTile t;
     if (!parse_direct_spec(spec, &t))
         return set_error(FBCORR_ERR_INVALID_ARG, "unknown variant spec '%s'", spec.c_str());
-    const DirectProblem pr = fwd_problem(p);
     if (direct_smem_bytes(t, pr.fh, pr.fw, pr.c) > smem_limit(p->dev))
         return set_error(FBCORR_ERR_UNSUPPORTED, "variant %s needs too much shared memory",
                          spec.c_str());
@@ -129,9 +153,7 @@ fbcorr_status_t choose_fwd_f32(fbcorr_plan* p) {
         if (set_fwd_spec(p, cached, "cache") == FBCORR_OK) return FBCORR_OK;
         logf("tune-cache entry '%s' not usable; ignoring it", cached.c_str());
     }
-    const DirectProblem pr = fwd_problem(p);
-    const DirectTile t = direct_heuristic(pr, smem_limit(p->dev), p->dev.sm_count);
-    fbcorr_status_t s = set_fwd_spec(p, direct_tile_spec(t), "heuristic");
+    fbcorr_status_t s = set_fwd_spec(p, heuristic_spec(fwd_problem(p), p->dev), "heuristic");
     if (s == FBCORR_ERR_NVRTC && p->snippet.empty()) {
         logf("code generation failed, falling back to the prebuilt default kernel: %s",
              last_error_message());
@@ -165,28 +187,37 @@ void replan_dw_chunks(fbcorr_plan* p, int resident) {
     p->dw_chunks = (int)((p->Ho + best_rows - 1) / best_rows);
 }
 
+// The dL/dx variant: forced (tests, profiling), tuned, or the model's.
+std::string dx_spec(const fbcorr_plan* p) {
+    std::string spec = env_str("FBCORR_DX_VARIANT", "");
+    if (!spec.empty() || tune_lookup(tune_key(p->dev, shape_key(p, "dx")), &spec)) return spec;
+    return heuristic_spec(dx_problem(p), p->dev);
+}
+
+// Where the dL/dx scratch begins in a backward workspace: after the dL/dw partial sums.
+size_t dx_scratch_offset(const fbcorr_plan* p) { return (p->ws_bwd + 255) / 256 * 256; }
+
 fbcorr_status_t prepare_backward(fbcorr_plan* p) {
     if (p->bwd_ready) return FBCORR_OK;
     const DirectProblem pr = dx_problem(p);
     DirectTile t = direct_heuristic(pr, smem_limit(p->dev), p->dev.sm_count);
-    std::string cached;
-    bool use_default = false;
-    const std::string forced = env_str("FBCORR_DX_VARIANT", "");   // a dL/dx spec (tests, profiling)
-    if (!forced.empty() || tune_lookup(tune_key(p->dev, shape_key(p, "dx")), &cached)) {
-        if (!forced.empty()) cached = forced;
-        DirectTile ct;
-        if (cached == "default")
-            use_default = true;
-        else if (parse_direct_spec(cached, &ct) &&
-                 direct_smem_bytes(ct, pr.fh, pr.fw, pr.c) <= smem_limit(p->dev))
-            t = ct;
-    }
+    const std::string spec = dx_spec(p);
+    const bool use_default = spec == "default";
+    DirectTile ct;
+    if (parse_direct_spec(spec, &ct) && direct_smem_bytes(ct, pr.fh, pr.fw, pr.c) <= smem_limit(p->dev)) t = ct;
     Kernel k;
     fbcorr_status_t s = use_default ? FBCORR_ERR_NVRTC : build_direct(pr, t, &k);
     if (s == FBCORR_OK) {
         p->dx_kind = VarKind::Direct;
         p->dx_tile = t;
         p->dx_kernel = k;
+        F3Tile f3;
+        F3Launch l;
+        // with scratch the tensor-core kernel runs, without it the FMA kernel
+        if (f3_parse_spec(spec, &f3) && f3_build(pr, f3, p->dev.sm_count, &l) == FBCORR_OK) {
+            p->dx_kind = VarKind::F32tc;
+            p->dx_f3 = l;
+        }
     } else if (s == FBCORR_ERR_NVRTC) {
         p->dx_kind = VarKind::Default;
     } else {
@@ -509,7 +540,7 @@ fbcorr_status_t fbcorr_plan_profile_read(fbcorr_plan_t p, float* ms, int cap, in
 }
 
 int plan_launches_per_forward(const fbcorr_plan* p) {
-    return p->fwd_kind == VarKind::Tensor ? tc_launches(p->tc) : 1;
+    return p->fwd_kind == VarKind::Tensor ? tc_launches(p->tc) : p->fwd_kind == VarKind::F32tc ? 2 : 1;
 }
 
 fbcorr_status_t fbcorr_plan_destroy(fbcorr_plan_t p) {
@@ -544,6 +575,20 @@ fbcorr_status_t fbcorr_plan_workspace_size(fbcorr_plan_t p, size_t* fwd, size_t*
     return FBCORR_OK;
 }
 
+fbcorr_status_t fbcorr_plan_scratch_size(fbcorr_plan_t p, size_t* fwd, size_t* bwd) {
+    clear_error();
+    if (!p) return set_error(FBCORR_ERR_INVALID_ARG, "NULL plan");
+    if (fwd) *fwd = p->fwd_kind == VarKind::F32tc ? p->fwd_f3.ws_bytes : p->ws_fwd;
+    if (bwd) {
+        *bwd = p->ws_bwd;
+        if (p->epi.kind != FBCORR_EPI_SNIPPET) {
+            FBC_TRY(prepare_backward(p));
+            if (p->dx_kind == VarKind::F32tc) *bwd = dx_scratch_offset(p) + p->dx_f3.ws_bytes;
+        }
+    }
+    return FBCORR_OK;
+}
+
 fbcorr_status_t fbcorr_forward(fbcorr_plan_t p, const float* x, const float* w, float* y, void* ws,
                                size_t ws_bytes, fbcorr_stream_t stream) {
     clear_error();
@@ -571,6 +616,13 @@ fbcorr_status_t fbcorr_forward(fbcorr_plan_t p, const float* x, const float* w, 
         case VarKind::Default:
             if (e0) FBC_CUDA(cudaEventRecord(e0, s));
             st = run_default(fwd_problem(p), x, nullptr, w, y, p->epi.lo, p->epi.hi, s);
+            if (e1 && st == FBCORR_OK) FBC_CUDA(cudaEventRecord(e1, s));
+            return st;
+        case VarKind::F32tc:
+            if (e0) FBC_CUDA(cudaEventRecord(e0, s));
+            st = ws && aligned16(ws) && ws_bytes >= p->fwd_f3.ws_bytes
+                     ? f3_run(p->fwd_f3, fwd_problem(p), x, nullptr, w, y, ws, p->epi.lo, p->epi.hi, p->err_dev, s)
+                     : run_direct(p->fwd_kernel, fwd_problem(p), p->fwd_tile, x, nullptr, w, y, p->epi.lo, p->epi.hi, s);
             if (e1 && st == FBCORR_OK) FBC_CUDA(cudaEventRecord(e1, s));
             return st;
         case VarKind::Tensor:
@@ -629,7 +681,10 @@ fbcorr_status_t fbcorr_backward(fbcorr_plan_t p, const float* x, const float* w,
     fbcorr_status_t st = FBCORR_OK;
     if (dx) {
         const DirectProblem pr = dx_problem(p);
-        st = p->dx_kind == VarKind::Direct
+        const size_t off = dx_scratch_offset(p);
+        const bool f3 = p->dx_kind == VarKind::F32tc && ws && aligned16(ws) && ws_bytes >= off + p->dx_f3.ws_bytes;
+        st = f3 ? f3_run(p->dx_f3, pr, g, m, w, dx, (uint8_t*)ws + off, p->epi.lo, p->epi.hi, p->err_dev, s)
+             : p->dx_kind != VarKind::Default
                  ? run_direct(p->dx_kernel, pr, p->dx_tile, g, m, w, dx, p->epi.lo, p->epi.hi, s)
                  : run_default(pr, g, m, w, dx, p->epi.lo, p->epi.hi, s);
     }
@@ -652,10 +707,7 @@ fbcorr_status_t fbcorr_plan_set_variant(fbcorr_plan_t p, const char* spec) {
         p->fwd_source = s == "heuristic" ? "heuristic" : "forced";
         return FBCORR_OK;
     }
-    if (s == "heuristic") {
-        const DirectTile t = direct_heuristic(fwd_problem(p), smem_limit(p->dev), p->dev.sm_count);
-        return set_fwd_spec(p, direct_tile_spec(t), "heuristic");
-    }
+    if (s == "heuristic") return set_fwd_spec(p, heuristic_spec(fwd_problem(p), p->dev), "heuristic");
     if (s == "tuned") return fbcorr_autotune(p, nullptr);
     return set_fwd_spec(p, s, "forced");
 }
@@ -678,12 +730,24 @@ fbcorr_status_t fbcorr_autotune(fbcorr_plan_t p, fbcorr_stream_t stream) {
     std::string best;
     float ms = 0.f;
     FBC_TRY(tune_direct(p, fwd_problem(p), s, "fwd", &best, &ms));
+    float f3_ms = 0.f;
+    std::string f3;
+    FBC_TRY(f3_tune(p->dev, fwd_problem(p), s, p->err_dev, &f3_ms, &f3));
+    if (!f3.empty() && f3_ms < ms) {
+        best = f3;
+        ms = f3_ms;
+    }
     FBC_TRY(set_fwd_spec(p, best, "tuned"));
     tune_store(tune_key(p->dev, shape_key(p, "fwd")), best);
     logf("autotune fwd picked %s (%.4f ms)", best.c_str(), ms);
     // dL/dx: the same generated kernel family on the flipped problem
     std::string best_dx;
     FBC_TRY(tune_direct(p, dx_problem(p), s, "dx", &best_dx, &ms));
+    FBC_TRY(f3_tune(p->dev, dx_problem(p), s, p->err_dev, &f3_ms, &f3));
+    if (!f3.empty() && f3_ms < ms) {
+        best_dx = f3;
+        ms = f3_ms;
+    }
     tune_store(tune_key(p->dev, shape_key(p, "dx")), best_dx);
     logf("autotune dx picked %s (%.4f ms)", best_dx.c_str(), ms);
     p->bwd_ready = false;   // rebuilt from the cache entry on the next backward call
@@ -821,6 +885,11 @@ fbcorr_status_t fbcorr_plan_info(fbcorr_plan_t p, char* buf, size_t cap) {
         o << ",\"spec\":\"" << direct_tile_spec(p->fwd_tile) << "\",\"smem\":" << p->fwd_kernel.smem
           << ",\"threads\":" << p->fwd_kernel.threads << ",\"kernel\":\"" << p->fwd_kernel.name
           << "\",\"source_hash\":\"" << hex64(p->fwd_kernel.src_hash) << "\"";
+    } else if (p->fwd_kind == VarKind::F32tc) {
+        o << ",\"spec\":\"" << f3_spec(p->fwd_f3.tile) << "\",\"smem\":" << p->fwd_f3.kernel.smem << ",\"threads\":"
+          << p->fwd_f3.kernel.threads << ",\"grid\":" << p->fwd_f3.grid << ",\"slots\":[" << p->fwd_f3.na << ","
+          << p->fwd_f3.nb << "],\"kernel\":\"" << p->fwd_f3.kernel.name << "\",\"source_hash\":\""
+          << hex64(p->fwd_f3.kernel.src_hash) << "\"";
     } else if (p->fwd_kind == VarKind::Default) {
         o << ",\"spec\":\"default\"";
     } else if (p->tc) {
@@ -830,6 +899,7 @@ fbcorr_status_t fbcorr_plan_info(fbcorr_plan_t p, char* buf, size_t cap) {
     if (p->bwd_ready) {
         o << ",\"dx\":{\"kind\":\"" << kind_name(p->dx_kind) << "\"";
         if (p->dx_kind == VarKind::Direct) o << ",\"spec\":\"" << direct_tile_spec(p->dx_tile) << "\"";
+        if (p->dx_kind == VarKind::F32tc) o << ",\"spec\":\"" << f3_spec(p->dx_f3.tile) << "\"";
         o << "},\"dw\":{\"kind\":\"" << kind_name(p->dw_kind) << "\",\"threads\":" << p->D * p->dw_ng
           << ",\"filters_per_cta\":" << p->dw_tn * p->dw_ng << ",\"packed_pairs\":" << p->dw_pk << ",\"min_blocks\":" << p->dw_mb
           << ",\"registers\":" << p->dw_regs << ",\"tile\":[" << p->dw_tn << "," << p->dw_ng << "," << p->dw_qb << "]"
@@ -922,6 +992,23 @@ fbcorr_status_t fbcorr_rtcg_check(const int64_t in_shape[3], const int64_t filt_
     }
     const size_t lim = 200 * 1024;
     const DirectProblem fp = fwd_problem(&tmp), bp = dx_problem(&tmp);
+    F3Tile f3;
+    if (f3_parse_spec(sp, &f3) || sp == "f32tc") {
+        // the FP32 tensor-core kernels of the forward (this tile, or the heuristic's) and of dL/dx
+        for (const DirectProblem* pr : {&fp, &bp}) {
+            const std::vector<F3Tile> ranked = f3_ranked(*pr, 152, nullptr);
+            if (ranked.empty())
+                return set_error(FBCORR_ERR_UNSUPPORTED, "the FP32 tensor-core kernel does not take this shape");
+            const F3Tile ft = pr == &fp && sp != "f32tc" ? f3 : ranked.front();
+            std::string lg;
+            const fbcorr_status_t st = rtcg_compile_only(f3_kernel_source(*pr, ft, f3_kernel_name(*pr, ft)), &lg);
+            if (st != FBCORR_OK) {
+                if (log && cap) snprintf(log, cap, "%s", lg.c_str());
+                return st;
+            }
+        }
+        return FBCORR_OK;
+    }
     DirectTile t;
     if (sp == "heuristic")
         t = direct_heuristic(fp, lim, 148);

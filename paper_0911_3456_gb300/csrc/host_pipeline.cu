@@ -71,7 +71,7 @@ fbcorr_status_t setup(fbcorr_plan_t p, int bands, cudaStream_t s) {
         // a tuned plan gets tuned band plans (first call only; cached by shape)
         if (p->fwd_source == "tuned" && bp->fwd_source != "cache") FBC_TRY(fbcorr_autotune(bp, s));
         size_t need = 0;
-        FBC_TRY(fbcorr_plan_workspace_size(bp, &need, nullptr));
+        FBC_TRY(fbcorr_plan_scratch_size(bp, &need, nullptr));
         hp->ws_bytes = std::max(hp->ws_bytes, need);
     }
     if (hp->ws_bytes) FBC_CUDA(cudaMalloc(&hp->ws, hp->ws_bytes));

@@ -63,6 +63,8 @@ std::string hex64(unsigned long long v);
 // on-disk cubin cache, load it into the current context and return a handle.
 fbcorr_status_t rtcg_kernel(const std::string& src, const std::string& name, size_t smem,
                             int threads, Kernel* out);
+// Another kernel (of at most 48 KB of shared memory) of the source that `first` came from.
+fbcorr_status_t rtcg_second_kernel(const Kernel& first, const std::string& name, size_t smem, int threads, Kernel* out);
 // Compile many sources on host threads into the on-disk cubin cache.
 fbcorr_status_t rtcg_precompile(const std::vector<std::string>& sources);
 // Compile only (no GPU needed); returns the NVRTC log on failure.
@@ -90,11 +92,13 @@ const char* rtcg_header_source();     // contents of rtcg_direct.cuh
 const char* rtcg_tc_params_source();  // contents of tc_params.h
 const char* rtcg_ptx_source();        // contents of rtcg_ptx.cuh
 const char* rtcg_tc_source();         // contents of rtcg_tc.cuh
+const char* rtcg_f32tc_params_source();   // contents of f32tc_params.h
+const char* rtcg_f32tc_source();      // contents of rtcg_f32tc.cuh
 const char* rtcg_nn_params_source();  // contents of nn_params.h
 const char* rtcg_nn_source();         // contents of rtcg_nn.cuh
 
 // ---- variants ------------------------------------------------------------------
-enum class VarKind { Default = 0, Direct = 1, Tensor = 2 };
+enum class VarKind { Default = 0, Direct = 1, Tensor = 2, F32tc = 3 };
 
 struct DirectTile {
     int tr = 8, tf = 8, wr = 1, wf = 2;
@@ -225,6 +229,38 @@ fbcorr_status_t tc_rtcg_check(int D, int fw, const std::string& spec, std::strin
 // Compile-only check of the generated kernel with a snippet epilogue (default configuration).
 fbcorr_status_t tc_snippet_check(int D, int fw, int split, const std::string& snippet, std::string* log);
 
+// ---- FP32 on the tensor cores (f32tc_kernel.cu) --------------------------------------
+// One direct-correlation problem (forward or dL/dx) by a three-way BF16 split.
+struct F3Tile {
+    int nt = 64;   // columns of B per tile (a multiple of 16, at most 80)
+    int r = 1;     // output rows folded into the columns (narrow banks)
+    int gc = 16;   // channels per unit: 8 (packed), 16 or 32
+    int jt = 1;    // filter taps per unit
+    int ru = 1;    // slab rows per unit (a unit is one accumulation chunk)
+};
+struct F3Launch {
+    F3Tile tile;
+    Kernel kernel, bank;       // the correlation, and the split of the bank before it
+    int grid = 0, bank_blocks = 0, filter_tiles = 0;
+    int na = 0, nb = 0;
+    size_t ws_bytes = 0;       // scratch of one call: the split bank and its flags
+};
+std::string f3_spec(const F3Tile& t);
+bool f3_parse_spec(const std::string& s, F3Tile* t);
+// Every tile the kernel takes the problem with (none: it does not), by the cost model, best first.
+std::vector<F3Tile> f3_ranked(const DirectProblem& pr, int sm_count, double* best_cycles);
+// Time the model's first tiles on patterned buffers; *spec is empty when there are none.
+fbcorr_status_t f3_tune(const DeviceInfo& dev, const DirectProblem& pr, cudaStream_t s, int* err_word, float* ms,
+                        std::string* spec);
+// The best rated tile, and whether the model expects it to be faster than the FP32 FMA kernels.
+bool f3_wins(const DirectProblem& pr, int sm_count, F3Tile* t);
+size_t f3_ws_bytes(const DirectProblem& pr, const F3Tile& t);
+std::string f3_kernel_source(const DirectProblem& pr, const F3Tile& t, const std::string& name);   // + name "_bank"
+std::string f3_kernel_name(const DirectProblem& pr, const F3Tile& t);
+fbcorr_status_t f3_build(const DirectProblem& pr, const F3Tile& t, int sm_count, F3Launch* out);
+fbcorr_status_t f3_run(const F3Launch& l, const DirectProblem& pr, const float* x, const float* m, const float* w,
+                       float* y, void* ws, float lo, float hi, int* err_word, cudaStream_t s);
+
 // ---- argument validation (api.cu) -------------------------------------------------------
 fbcorr_status_t validate_shapes(const int64_t* in, const int64_t* fs, fbcorr_dtype_t dtype,
                                 const fbcorr_epilogue_t& epi);
@@ -249,6 +285,7 @@ struct fbcorr_plan {
     fbc::Kernel fwd_kernel;
     std::string fwd_source;        // "heuristic", "tuned", "cache", "env", "forced"
     fbc::TcPlan* tc = nullptr;
+    fbc::F3Launch fwd_f3;
     std::string snippet;           // user epilogue expression (epi.kind == FBCORR_EPI_SNIPPET)
 
     // backward (F32 always)
@@ -256,6 +293,7 @@ struct fbcorr_plan {
     fbc::VarKind dx_kind = fbc::VarKind::Direct;
     fbc::DirectTile dx_tile;
     fbc::Kernel dx_kernel;
+    fbc::F3Launch dx_f3;
     fbc::VarKind dw_kind = fbc::VarKind::Direct;
     fbc::Kernel dw_kernel;
     int dw_tn = 4, dw_ng = 1, dw_qb = 64, dw_nblocks = 1;

@@ -75,5 +75,7 @@ extern "C" fbcorr_status_t fbcorr_forward_noalloc(fbcorr_plan_t plan, const floa
     // kernel reads (zero padding included) before the kernel runs.
     void* ws = nullptr;
     FBC_TRY(scratch_address(plan->dev.device, &ws));
+    // FP32 plans leave it alone: their calls may overlap
+    if (plan->dtype == FBCORR_F32) return fbcorr_forward(plan, x, w, y, nullptr, 0, stream);
     return fbcorr_forward(plan, x, w, y, ws, kNoAllocScratchBytes, stream);
 }

@@ -314,6 +314,29 @@ fbcorr_status_t rtcg_kernel(const std::string& src, const std::string& name, siz
     return FBCORR_OK;
 }
 
+fbcorr_status_t rtcg_second_kernel(const Kernel& first, const std::string& name, size_t smem, int threads, Kernel* out) {
+    DriverApi* drv = nullptr;
+    FBC_TRY(driver_api(&drv));
+    CUcontext ctx = nullptr;
+    CUmodule mod = nullptr;
+    if (drv->ctxGetCurrent(&ctx) == CUDA_SUCCESS && ctx) {
+        std::lock_guard<std::mutex> lk(g_mu);
+        auto it = g_modules.find(ModKey{ctx, first.src_hash});
+        if (it != g_modules.end()) mod = it->second;
+    }
+    if (!mod) return set_error(FBCORR_ERR_INTERNAL, "the module of %s is not loaded", first.name.c_str());
+    CUfunction fn = nullptr;
+    const CUresult r = drv->moduleGetFunction(&fn, mod, name.c_str());
+    if (r != CUDA_SUCCESS)
+        return set_error(FBCORR_ERR_CUDA, "cuModuleGetFunction(%s): %s", name.c_str(), cu_err(r));
+    out->fn = fn;
+    out->threads = threads;
+    out->smem = smem;
+    out->name = name;
+    out->src_hash = first.src_hash;
+    return FBCORR_OK;
+}
+
 std::string hex64(unsigned long long v) {
     char b[32];
     snprintf(b, sizeof b, "%016llx", v);

@@ -1,0 +1,657 @@
+// rtcg_f32tc.cuh -- the FP32 correlation on the tensor cores, compiled at plan
+// time by NVRTC for sm_103a.  Embedded as a string into libfbcorr and prefixed
+// with f32tc_params.h and rtcg_ptx.cuh; self-contained (no system headers).
+//
+// Arithmetic.  Every FP32 operand is split exactly into three BF16 values,
+// v = v1 + v2 + v3 with v1 = bf16_rn(v), v2 = bf16_rn(v - v1), v3 = v - v1 - v2
+// (24 significand bits in three 8-bit ones), and the product x w is taken as the
+// six largest of the nine BF16 products, each exact in FP32:
+//   order 0: x1 w1      order 1: x1 w2 + x2 w1      order 2: x1 w3 + x2 w2 + x3 w1
+// The three that are left out are below 2^-26 |x w|.  The tensor core truncates
+// its FP32 accumulator at every K = 16 step, so a sum is only left there for a
+// chunk of a few steps: each order has its own accumulator (a truncation of
+// order 1 and 2 is then 2^-8 and 2^-16 below one of the result), and the chunk
+// sums are added to FP32 registers with ordinary rounding.  Measured error
+// against 64 bits: at or below that of the FP32 FMA kernels it stands in for.
+//
+// Layout.  As in the BF16 kernels, an A tile is 128 consecutive pixels of the
+// image laid out with the virtual row width vw = out_w + FW - 1 (columns past
+// out_w are computed and dropped), and one slab of pixels serves every filter
+// tap of a row: tap j is the slab started j pixels later.  The three orders of B
+// lie side by side as 3 NT rows of one operand, so a K = 16 step is three MMAs,
+//   x1 x [w1 w2 w3] (N = 3 NT) -> columns [0, 3 NT)
+//   x2 x [w1 w2]    (N = 2 NT) -> columns [NT, 3 NT)
+//   x3 x [w1]       (N =   NT) -> columns [2 NT, 3 NT)
+// which read each A tile three times instead of six: at NT = 64 the operand
+// reads of shared memory (24 KB per step) take as long as the MMAs (192 cycles).
+//
+// Depth.  GC = 16 or 32: the step takes 16 channels of one tap (two chunk
+// planes of 8 channels, LBO = one plane).  GC = 8: one plane whose 16-byte chunk
+// at pixel q holds PP = 8 / CP pixels q .. q + PP - 1 of CP channels, and the
+// second half of the step is the same plane PP pixels later (LBO = 16 PP bytes):
+// a step covers 2 PP taps, so depths of 1, 2, 4 and 8 waste none of K = 16.
+//
+// Rows.  R > 1 (narrow banks): the columns of B are R output rows x NF filters,
+// column (r, n) of slab row u holding filter row u - r (zero outside the
+// filter), so one slab row feeds R output rows and FH + R - 1 rows of MMAs do the
+// work of R FH.
+//
+// Units.  A unit is RU slab rows of one channel and tap group; its RU S steps are
+// one accumulation chunk, its A slot holds RU slabs and its B stage all filters of
+// the tile.  The bank is split once per call (fbc_f32tc_bank_body) into the images
+// of the B stages, so that a stage is one bulk copy.
+//
+// Roles per CTA (persistent, one per SM): warps 0..7 add the chunk sums up and
+// store; warps 8..12 read x from global memory (prefetched in registers), split it
+// and write the A slots; a thread of warp 13 copies the B stages; a thread of
+// warp 14 issues the MMAs of every other unit, one of warp 15 the rest, each into
+// its own accumulator set, so chunk sums are drained while the next chunk runs.
+//
+// Values the split cannot carry.  Non-finite inputs or overflow give a
+// non-finite sum, and a non-zero |v| < 2^-100 (whose third part could fall below
+// the BF16 range) raises a flag for its work item; the epilogue warps then
+// recompute their outputs with FP32 FMAs straight from global memory.
+//
+// Every mbarrier wait is bounded in time; on expiry the kernel records an error
+// code in host-mapped memory, stops every role, waits (bounded) for its MMAs in
+// flight, frees TMEM and returns.
+
+#define FBC_F3_ERR_WAIT 5
+
+// tcgen05.mma with the descriptors as low and high words.
+__device__ __forceinline__ void fbc_umma_lo(fbc_u32 d, fbc_u32 alo, fbc_u32 ahi, fbc_u32 blo, fbc_u32 bhi, fbc_u32 idesc,
+                                            fbc_u32 accumulate) {
+    asm volatile(
+        "{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %6, 0;\n mov.b64 a, {%1, %2};\n mov.b64 b, {%3, %4};\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, p;\n}\n" ::"r"(d),
+        "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(accumulate));
+}
+
+// Snippet epilogue (EPI = 2): defined by the generated source after this file.
+__device__ float fbc_user_epi(float y, int n, float lo, float hi);
+
+template <int FH_, int FW_, int C_, int NF_, int FLIP_, int EPI_, int MASK_, int NT_, int R_, int GC_,
+          int JT_, int RU_>
+struct FbcF3Cfg {
+    static constexpr int FH = FH_, FW = FW_, C = C_, NF = NF_, FLIP = FLIP_, EPI = EPI_, MASK = MASK_;
+    static constexpr int NT = NT_, R = R_, GC = GC_, JT = JT_, RU = RU_;
+    static constexpr bool PACK = GC == 8;
+    static constexpr int PP = !PACK ? 1 : C <= 1 ? 8 : C <= 2 ? 4 : C <= 4 ? 2 : 1;   // pixels per chunk
+    static constexpr int CP = 8 / PP;                                                // channels per pixel in it
+    static constexpr int PL = PACK ? 1 : GC / 8;                                     // chunk planes of a slab
+    static constexpr int S = PACK ? (JT + 2 * PP - 1) / (2 * PP) : JT * (GC / 16);   // K = 16 steps per slab
+    static constexpr int NCG = (C + GC - 1) / GC;                                    // channel groups
+    static constexpr int NTG = (FW + JT - 1) / JT;                                   // tap groups
+    static constexpr int ROWS = FH + R - 1;                                          // slab rows per pixel tile
+    static constexpr int NU = (ROWS + RU - 1) / RU * NCG * NTG;                      // units per pixel tile
+    static constexpr int LS = PACK ? 128 + (2 * S - 1) * PP : 128 + JT - 1;          // slab pixels
+    // plane pitch in pixels: planes 32 (four planes) or 64 (two) bytes apart modulo
+    // 128, so that the writes of neighbouring quads of a pixel hit other banks
+    static constexpr int LP = PL == 4 ? (LS + 5) / 8 * 8 + 2 : PL == 2 ? (LS + 3) / 8 * 8 + 4 : LS;
+    static constexpr unsigned PLANE = LP * 16;
+    static constexpr unsigned AORD = PL * PLANE;                                     // bytes of one order of a slab
+    static constexpr unsigned SLAB = 3 * AORD;
+    static constexpr unsigned ASLOT = (RU * SLAB + 127) / 128 * 128;
+    static constexpr unsigned BCH = 3 * NT * 16;             // bytes per chunk of B
+    static constexpr unsigned BSTEP = 2 * BCH;
+    static constexpr int STEPS = RU * S;                     // steps of a unit
+    // a B stage holds BS steps, about 12 KB (one copy at the copy unit's full rate):
+    // refills start, and are waited for, in small pieces
+    static constexpr int BS = NT >= 48 ? 2 : NT >= 32 ? 4 : 8;
+    static constexpr int NST = (STEPS + BS - 1) / BS;        // stages of a unit
+    static constexpr unsigned BSTAGE = BS * BSTEP;
+    static constexpr unsigned BUNIT = STEPS * BSTEP;         // the unit's image in the split bank
+    static constexpr int NCT = 32 * FBC_F3_CONV_WARPS;
+    // Items of the converters: quads of 4 channels read with one 16-byte load, lanes
+    // along the channels, or (depths that are no multiple of 4) chunks of 8 single
+    // loads, lanes along the pixels.
+    static constexpr bool VA = C % 4 == 0;
+    static constexpr int WA = VA ? 4 : 8;                    // floats per item
+    static constexpr int QA = !VA ? PL : PP == 2 ? 1 : GC / 4;      // items per pixel
+    static constexpr int NPX = VA && PP == 2 ? LS + 1 : LS;         // pixels read per slab
+    static constexpr int NIT = RU * NPX * QA;                // items per unit
+    static constexpr int KA = (NIT + NCT - 1) / NCT;
+    static constexpr int PA = KA * WA <= 18 ? 4 : KA * WA <= 24 ? 3 : KA * WA <= 36 ? 2 : 1;   // units in registers
+    static constexpr int NBC = RU * S * 2 * NT;              // bank chunks per unit
+    __device__ static __forceinline__ int tap_group(int u) { return NTG > 1 ? u % NTG : 0; }
+    __device__ static __forceinline__ int channel_group(int u) { return NCG > 1 ? (u / NTG) % NCG : 0; }
+    __device__ static __forceinline__ int row0(int u) { return u / (NTG * NCG) * RU; }
+    static constexpr unsigned TMEM = 6 * NT <= 32 ? 32 : 6 * NT <= 64 ? 64 : 6 * NT <= 128 ? 128 : 6 * NT <= 256 ? 256 : 512;
+};
+
+// v = h + m + l exactly (finite v in the BF16 range); tiny takes the least of
+// 2|v| - 1 as integers over the values (zeros: the largest integer).
+__device__ __forceinline__ void fbc_f3_split2(float v0, float v1, fbc_u32& h, fbc_u32& m, fbc_u32& l, fbc_u32& tiny) {
+    h = fbc_pack_bf16x2(v0, v1);
+    const float r0 = v0 - __uint_as_float(h << 16), r1 = v1 - __uint_as_float(h & 0xFFFF0000u);
+    m = fbc_pack_bf16x2(r0, r1);
+    l = fbc_pack_bf16x2(r0 - __uint_as_float(m << 16), r1 - __uint_as_float(m & 0xFFFF0000u));
+    tiny = min(tiny, min(__float_as_uint(v0) * 2u - 1u, __float_as_uint(v1) * 2u - 1u));
+}
+
+__device__ __forceinline__ void fbc_f3_split4(const float (&v)[4], fbc_u32 (&h)[2], fbc_u32 (&m)[2], fbc_u32 (&l)[2],
+                                              fbc_u32& tiny) {
+    fbc_f3_split2(v[0], v[1], h[0], m[0], l[0], tiny);
+    fbc_f3_split2(v[2], v[3], h[1], m[1], l[1], tiny);
+}
+
+// The three orders of one chunk (8 values) to shared memory, `ord` bytes apart.
+__device__ __forceinline__ void fbc_f3_put(const float (&v)[8], fbc_u32 dst, fbc_u32 ord, fbc_u32& tiny) {
+    fbc_u32 h[4], m[4], l[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) fbc_f3_split2(v[2 * k], v[2 * k + 1], h[k], m[k], l[k], tiny);
+    fbc_st_shared_v4(dst, h[0], h[1], h[2], h[3]);
+    fbc_st_shared_v4(dst + ord, m[0], m[1], m[2], m[3]);
+    fbc_st_shared_v4(dst + 2 * ord, l[0], l[1], l[2], l[3]);
+}
+
+__device__ __forceinline__ void fbc_f3_put(const float (&v)[4], fbc_u32 dst, fbc_u32 ord, fbc_u32& tiny) {
+    fbc_u32 h[2], m[2], l[2];
+    fbc_f3_split4(v, h, m, l, tiny);
+    fbc_st_shared_v2(dst, h[0], h[1]);
+    fbc_st_shared_v2(dst + ord, m[0], m[1]);
+    fbc_st_shared_v2(dst + 2 * ord, l[0], l[1]);
+}
+
+#define FBC_F3_TINY ((27u << 24) - 1u)   // 2 * bits(2^-100) - 1
+
+__device__ __forceinline__ int fbc_f3_row(int v, const FbcF3Params& P) {
+    return P.vw == 1 ? v : (int)(__umulhi((unsigned)v, P.vw_mul) >> P.vw_shift);
+}
+
+template <class G>
+__device__ __forceinline__ float fbc_f3_masked(float v, const float* m, const FbcF3Params& P) {
+    if constexpr (G::MASK) {
+        const float t = __ldg(m);
+        return (t > P.lo && t < P.hi) ? v : 0.f;
+    }
+    return v;
+}
+
+// The epilogue and store of 8 consecutive columns col0 .. col0 + 7 of the tile
+// at output pixel (row group pg, column q); n0 = first filter of the tile.
+template <class G>
+__device__ __forceinline__ void fbc_f3_store8(const FbcF3Params& P, int pg, int q, int n0, int col0, float (&v)[8]) {
+    if constexpr (G::EPI == 1) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = fminf(fmaxf(v[k], P.lo), P.hi);
+    }
+    if constexpr (G::EPI == 2) {
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            v[k] = fbc_user_epi(v[k], G::R > 1 ? (col0 + k) % G::NF : n0 + col0 + k, P.lo, P.hi);
+    }
+    // group size of contiguous, equally aligned filters of one output row
+    constexpr int GS = G::NF % 8 == 0 ? 8 : G::NF % 4 == 0 ? 4 : 1;
+#pragma unroll
+    for (int g = 0; g < 8; g += GS) {
+        const int col = col0 + g;
+        const int r = G::R > 1 ? col / G::NF : 0;
+        const int n = G::R > 1 ? col - r * G::NF : n0 + col;
+        const int p = pg * G::R + r;
+        if (r >= G::R || p >= P.out_h || n >= G::NF) continue;
+        float* dst = P.y + ((long long)p * P.out_w + q) * G::NF + n;
+        if constexpr (GS == 8) {
+            if ((reinterpret_cast<unsigned long long>(P.y) & 31) == 0) {
+                asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "f"(v[0]),
+                             "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7])
+                             : "memory");
+            } else {
+                *reinterpret_cast<float4*>(dst) = make_float4(v[0], v[1], v[2], v[3]);
+                *reinterpret_cast<float4*>(dst + 4) = make_float4(v[4], v[5], v[6], v[7]);
+            }
+        } else if constexpr (GS == 4) {
+            *reinterpret_cast<float4*>(dst) = make_float4(v[g], v[g + 1], v[g + 2], v[g + 3]);
+        } else {
+            dst[0] = v[g];
+        }
+    }
+}
+
+// Columns [c0, c1) of one pixel recomputed with FP32 FMAs from global memory.
+template <class G>
+__device__ __noinline__ void fbc_f3_recompute(const FbcF3Params& P, int pg, int q, int n0, int c0, int c1) {
+    for (int col0 = c0; col0 < c1; col0 += 8) {
+        float acc[8];
+        int rr[8], nn[8];
+        bool on[8];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            acc[k] = 0.f;
+            rr[k] = G::R > 1 ? (col0 + k) / G::NF : 0;
+            nn[k] = G::R > 1 ? (col0 + k) % G::NF : n0 + col0 + k;
+            on[k] = rr[k] < G::R && pg * G::R + rr[k] < P.out_h && nn[k] < G::NF;
+        }
+        for (int i = 0; i < G::FH; ++i)
+            for (int j = 0; j < G::FW; ++j) {
+                const int xc = q + j - P.pad_x;
+                if (xc < 0 || xc >= P.in_w) continue;
+                for (int c = 0; c < G::C; ++c) {
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const int xr = pg * G::R + rr[k] + i - P.pad_y;
+                        if (!on[k] || xr < 0 || xr >= P.in_h) continue;
+                        const long long xo = ((long long)xr * P.in_w + xc) * G::C + c;
+                        const long long wo =
+                            G::FLIP ? (((long long)c * G::FH + (G::FH - 1 - i)) * G::FW + (G::FW - 1 - j)) * G::NF + nn[k]
+                                    : (((long long)nn[k] * G::FH + i) * G::FW + j) * G::C + c;
+                        acc[k] = fmaf(fbc_f3_masked<G>(__ldg(P.x + xo), P.m + xo, P), __ldg(P.w + wo), acc[k]);
+                    }
+                }
+            }
+        fbc_f3_store8<G>(P, pg, q, n0, col0, acc);
+    }
+}
+
+// Position in a CTA's sequence of (work item, unit); item = filter tile * mtiles + pixel tile.
+template <class G>
+struct FbcF3Pos {
+    int item, u;
+    __device__ __forceinline__ void start() {
+        item = blockIdx.x;
+        u = 0;
+    }
+    __device__ __forceinline__ bool valid(const FbcF3Params& P) const { return item < P.nitems; }
+    __device__ __forceinline__ void next() {
+        if (++u < G::NU) return;
+        u = 0;
+        item += gridDim.x;
+    }
+};
+
+// Item `it` of unit j: slab row it / (NPX QA) of the unit, a quad (VA) or a chunk
+// of 8 of one of its pixels.
+template <class G>
+__device__ __forceinline__ void fbc_f3_a_item(int it, int& k, int& px, int& sub) {
+    k = G::RU > 1 ? it / (G::NPX * G::QA) : 0;
+    const int r = it - k * (G::NPX * G::QA);
+    px = G::VA ? r / G::QA : r % G::NPX;
+    sub = G::VA ? r % G::QA : r / G::NPX;
+}
+
+template <class G>
+__device__ __forceinline__ void fbc_f3_load_a(const FbcF3Params& P, const FbcF3Pos<G>& j, int it, float (&v)[G::WA]) {
+    const int cg = G::channel_group(j.u);
+    int k, px, sub;
+    fbc_f3_a_item<G>(it, k, px, sub);
+    const int ri = G::row0(j.u) + k;
+    const int vp = (j.item % P.mtiles) * 128 + G::tap_group(j.u) * G::JT + px;
+    const int pg = fbc_f3_row(vp, P);
+    const int col = vp - pg * P.vw - P.pad_x;
+    const int row = pg * G::R + ri - P.pad_y;
+#pragma unroll
+    for (int e = 0; e < G::WA; ++e) v[e] = 0.f;
+    if (it >= G::NIT || ri >= G::ROWS || row < 0 || row >= P.in_h) return;
+    if constexpr (G::VA) {
+        const int ch = cg * G::GC + sub * 4;
+        if (col < 0 || col >= P.in_w || (G::PP == 1 && ch >= G::C)) return;
+        const unsigned o = (unsigned)((row * P.in_w + col) * G::C + (G::PP == 1 ? ch : 0));
+        const float4 f = __ldg(reinterpret_cast<const float4*>(P.x + o));
+        v[0] = f.x;
+        v[1] = f.y;
+        v[2] = f.z;
+        v[3] = f.w;
+        if constexpr (G::MASK) {
+            const float4 g = __ldg(reinterpret_cast<const float4*>(P.m + o));
+            if (!(g.x > P.lo && g.x < P.hi)) v[0] = 0.f;
+            if (!(g.y > P.lo && g.y < P.hi)) v[1] = 0.f;
+            if (!(g.z > P.lo && g.z < P.hi)) v[2] = 0.f;
+            if (!(g.w > P.lo && g.w < P.hi)) v[3] = 0.f;
+        }
+    } else {
+        const int ch = G::PP == 1 ? cg * G::GC + sub * 8 : 0;
+#pragma unroll
+        for (int e = 0; e < G::WA; ++e) {
+            const int cc = col + e / G::CP, c = ch + e % G::CP;
+            if (cc < 0 || cc >= P.in_w || c >= G::C) continue;
+            const unsigned o = (unsigned)((row * P.in_w + cc) * G::C + c);
+            v[e] = fbc_f3_masked<G>(__ldg(P.x + o), P.m + o, P);
+        }
+    }
+}
+
+// Item `it` of a unit into the A slot at dst.
+template <class G>
+__device__ __forceinline__ void fbc_f3_put_a(int it, const float (&v)[G::WA], fbc_u32 dst, fbc_u32& tiny) {
+    if (it >= G::NIT) return;
+    int k, px, sub;
+    fbc_f3_a_item<G>(it, k, px, sub);
+    const fbc_u32 d = dst + (fbc_u32)k * G::SLAB + (fbc_u32)px * 16u;
+    if constexpr (!G::VA) {
+        fbc_f3_put(v, d + (fbc_u32)sub * G::PLANE, G::AORD, tiny);
+    } else if constexpr (G::PP == 2) {
+        // a pixel of 4 channels: first half of chunk px and second half of chunk px - 1
+        fbc_u32 h[2], m[2], l[2];
+        fbc_f3_split4(v, h, m, l, tiny);
+        if (px < G::LS) {
+            fbc_st_shared_v2(d, h[0], h[1]);
+            fbc_st_shared_v2(d + G::AORD, m[0], m[1]);
+            fbc_st_shared_v2(d + 2 * G::AORD, l[0], l[1]);
+        }
+        if (px > 0) {
+            fbc_st_shared_v2(d - 8u, h[0], h[1]);
+            fbc_st_shared_v2(d - 8u + G::AORD, m[0], m[1]);
+            fbc_st_shared_v2(d - 8u + 2 * G::AORD, l[0], l[1]);
+        }
+    } else {
+        fbc_f3_put(v, d + (fbc_u32)(sub >> 1) * G::PLANE + (fbc_u32)(sub & 1) * 8u, G::AORD, tiny);
+    }
+}
+
+// The bank split: block (b, filter tile) splits chunks 256 b .. of the tile's
+// NU x NBC chunks (unit, slab row, step, half, column), one per thread, columns
+// fastest, into the B stage images; flags say where a tiny value was met.
+template <class G>
+__device__ __forceinline__ void fbc_f32tc_bank_body(const FbcF3Params& P) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int id = blockIdx.x * FBC_F3_BANK_THREADS + threadIdx.x;
+    fbc_u32 tiny = 0xFFFFFFFFu;
+    if (id < G::NU * G::NBC) {
+        const int u = id / G::NBC, it = id % G::NBC;
+        const int col = it % G::NT, kq = (it / G::NT) % (2 * G::S), ri = G::row0(u) + it / (G::NT * 2 * G::S);
+        const int r = G::R > 1 ? col / G::NF : 0;
+        const int n = G::R > 1 ? col - r * G::NF : (int)blockIdx.y * G::NT + col;
+        const int i = ri - r;
+        float v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) v[e] = 0.f;
+        if (r < G::R && n < G::NF && i >= 0 && i < G::FH) {
+            const int jl = G::PACK ? kq * G::PP : kq / G::PL;     // first tap of the chunk in its group
+            const int ch = G::PP > 1 ? 0 : G::PACK ? G::channel_group(u) * 8 : G::channel_group(u) * G::GC + (kq % G::PL) * 8;
+            const int tap = G::tap_group(u) * G::JT + jl;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int dt = e / G::CP, c = ch + e % G::CP;
+                if (jl + dt >= G::JT || tap + dt >= G::FW || c >= G::C) continue;
+                const unsigned o =
+                    G::FLIP ? (unsigned)(((c * G::FH + (G::FH - 1 - i)) * G::FW + (G::FW - 1 - tap - dt)) * G::NF + n)
+                            : (unsigned)(((n * G::FH + i) * G::FW + tap + dt) * G::C + c);
+                v[e] = __ldg(P.w + o);
+            }
+        }
+        fbc_u32 h[4], m[4], l[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) fbc_f3_split2(v[2 * k], v[2 * k + 1], h[k], m[k], l[k], tiny);
+        unsigned char* dst = P.bank + ((long long)blockIdx.y * G::NU + u) * G::BUNIT + (it / G::NT) * G::BCH + col * 16;
+        *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<uint4*>(dst + G::NT * 16) = make_uint4(m[0], m[1], m[2], m[3]);
+        *reinterpret_cast<uint4*>(dst + 2 * G::NT * 16) = make_uint4(l[0], l[1], l[2], l[3]);
+    }
+    const int any = __syncthreads_or(tiny < FBC_F3_TINY);
+    if (threadIdx.x == 0) P.flags[blockIdx.y * P.bank_blocks + blockIdx.x] = any;
+}
+
+template <class G>
+__device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
+    __shared__ int s_abort;
+    __shared__ fbc_u32 s_tmem;
+    __shared__ int s_tiny[16];       // item + 1 whose inputs need the FP32 path, by item ordinal % 16
+    const int warp = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31;
+    const fbc_u32 sbase = fbc_smem_addr(fbc_tc_smem);
+    // barrier table: a_full[na] a_empty[na] b_full[nb] b_empty[nb] acc_full[2] acc_empty[2] drain[2]
+    const fbc_u32 a_full0 = sbase + P.bar_off;
+    const fbc_u32 a_empty0 = a_full0 + 8u * P.na;
+    const fbc_u32 b_full0 = a_empty0 + 8u * P.na;
+    const fbc_u32 b_empty0 = b_full0 + 8u * P.nb;
+    const fbc_u32 acc_full0 = b_empty0 + 8u * P.nb;
+    const fbc_u32 acc_empty0 = acc_full0 + 16u;
+    const fbc_u32 drain_bar = acc_empty0 + 16u;
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < P.na; ++s) {
+            fbc_mbar_init(a_full0 + 8u * s, FBC_F3_CONV_WARPS);
+            fbc_mbar_init(a_empty0 + 8u * s, 1);
+        }
+        for (int s = 0; s < P.nb; ++s) {
+            fbc_mbar_init(b_full0 + 8u * s, 1);
+            fbc_mbar_init(b_empty0 + 8u * s, 1);
+        }
+        for (int s = 0; s < 2; ++s) {
+            fbc_mbar_init(acc_full0 + 8u * s, 2);    // the MMA commit, and the issuing thread itself
+            fbc_mbar_init(acc_empty0 + 8u * s, FBC_F3_EPI_WARPS);
+        }
+        fbc_mbar_init(drain_bar, 1);
+        fbc_mbar_init(drain_bar + 8u, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        s_abort = 0;
+    }
+    if (threadIdx.x < 16) s_tiny[threadIdx.x] = 0;
+    if (warp == 15) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(fbc_smem_addr(&s_tmem)),
+                     "n"(G::TMEM));
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    fbc_tc_fence_before();
+    __syncthreads();
+    fbc_tc_fence_after();
+    const fbc_u32 tmem = s_tmem;
+    volatile int* abort_flag = &s_abort;
+    // launched as a programmatic dependent: the previous kernel of the stream is
+    // complete and visible before anything below touches global memory
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+
+    if (warp >= 8 && warp < 8 + FBC_F3_CONV_WARPS) {
+        // ------------------------------------------------------------ converters
+        const int ct = threadIdx.x - 8 * 32;
+        FbcF3Pos<G> ja, jn;      // unit being written, unit being loaded
+        ja.start();
+        jn = ja;
+        float abuf[G::PA][G::KA][G::WA];
+        auto load_a = [&](float (&buf)[G::KA][G::WA]) {
+            if (!jn.valid(P)) return;
+#pragma unroll
+            for (int k = 0; k < G::KA; ++k) fbc_f3_load_a<G>(P, jn, ct + k * G::NCT, buf[k]);
+            jn.next();
+        };
+#pragma unroll
+        for (int s = 0; s < G::PA; ++s) load_a(abuf[s]);
+        int as = 0, ord = 0, item = ja.item;
+        fbc_u32 aph = 0;
+        bool ok = true;
+        while (ok && ja.valid(P)) {
+#pragma unroll
+            for (int s = 0; s < G::PA; ++s) {
+                if (!ok || !ja.valid(P)) break;
+                if (ja.item != item) {
+                    item = ja.item;
+                    ++ord;
+                }
+                if (!(ok = fbc_wait(a_empty0 + 8u * as, aph ^ 1, P, abort_flag, FBC_F3_ERR_WAIT))) break;
+                const fbc_u32 dst = sbase + (fbc_u32)as * G::ASLOT;
+                fbc_u32 tiny = 0xFFFFFFFFu;
+#pragma unroll
+                for (int k = 0; k < G::KA; ++k) fbc_f3_put_a<G>(ct + k * G::NCT, abuf[s][k], dst, tiny);
+                if (tiny < FBC_F3_TINY) *(volatile int*)&s_tiny[ord & 15] = ja.item + 1;
+                fbc_fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) fbc_mbar_arrive(a_full0 + 8u * as);
+                if (++as == P.na) { as = 0; aph ^= 1; }
+                load_a(abuf[s]);
+                ja.next();
+            }
+        }
+    } else if (warp == 13) {
+        if (lane == 0) {
+            // -------------------------------------------------------- bank producer
+            int bs = 0;
+            fbc_u32 bph = 0, it = 0;
+            bool ok = true;
+            FbcF3Pos<G> j;
+            for (j.start(); j.valid(P); j.next()) {
+                const unsigned char* src = P.bank + ((long long)(j.item / P.mtiles) * G::NU + j.u) * G::BUNIT;
+#pragma unroll 1
+                for (int st = 0; st < G::NST; ++st) {
+                    if (!(ok = fbc_wait(b_empty0 + 8u * bs, bph ^ 1, P, abort_flag, FBC_F3_ERR_WAIT))) break;
+                    const fbc_u32 bytes = min(G::BSTAGE, G::BUNIT - st * G::BSTAGE);
+                    fbc_mbar_expect_tx(b_full0 + 8u * bs, bytes);
+                    fbc_bulk_g2s(sbase + P.b_off + (fbc_u32)bs * G::BSTAGE, src + st * G::BSTAGE, bytes, b_full0 + 8u * bs);
+                    ++it;
+                    if (++bs == P.nb) { bs = 0; bph ^= 1; }
+                }
+                if (!ok) break;
+            }
+            if (!ok) {
+                // wait (bounded) for the copies still in flight into the ring
+                const fbc_u32 k0 = it > (fbc_u32)P.nb ? it - P.nb : 0;
+                for (fbc_u32 k = k0; k < it; ++k) fbc_wait_drain(b_full0 + 8u * (k % P.nb), (k / P.nb) & 1, P);
+            }
+        }
+    } else if (warp >= 14) {
+        if (lane == 0) {
+            // -------------------------------------------------------- MMA issuers
+            // Issuing one MMA takes a thread 40 to 60 cycles, a barrier wait or a commit
+            // about 70; at 32 to 96 cycles per MMA one thread alone left the tensor core
+            // idle a third of the time (dense 512 x 512 x 32 * 256 x 5 x 5: 0.43 ms).
+            const fbc_u32 idesc0 = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);   // FP32 += BF16 x BF16, M = 128
+            const fbc_u32 id3 = idesc0 | ((3u * G::NT >> 3) << 17);
+            const fbc_u32 id2 = idesc0 | ((2u * G::NT >> 3) << 17);
+            const fbc_u32 id1 = idesc0 | ((1u * G::NT >> 3) << 17);
+            // descriptors: the start address (16-byte units) sits in the low bits of the
+            // low word and never carries out of its field; the high word is constant
+            const fbc_u64 adesc0 = fbc_smem_desc(sbase, G::PACK ? 16u * G::PP : G::PLANE, 128);
+            const fbc_u64 bdesc0 = fbc_smem_desc(sbase + P.b_off, G::BCH, 128);
+            const fbc_u32 ahi = (fbc_u32)(adesc0 >> 32), bhi = (fbc_u32)(bdesc0 >> 32);
+            const int acc = warp - 14;         // this thread's accumulator set
+            const fbc_u32 d = tmem + (fbc_u32)(acc * 3 * G::NT);
+            int as = 0, bs = 0;
+            fbc_u32 aph = 0, bph = 0, accph = 0;
+            int turn = 0;
+            bool ok = true, issued = false;
+            FbcF3Pos<G> j;
+            for (j.start(); j.valid(P); j.next(), turn ^= 1) {
+                if (turn == acc) {
+                    if (!(ok = fbc_wait(acc_empty0 + 8u * acc, accph ^ 1, P, abort_flag, FBC_F3_ERR_WAIT))) break;
+                    if (!(ok = fbc_wait(a_full0 + 8u * as, aph, P, abort_flag, FBC_F3_ERR_WAIT))) break;
+                    accph ^= 1;
+                    const fbc_u32 alo = (fbc_u32)adesc0 + ((fbc_u32)as * G::ASLOT >> 4);
+                    const int steps = min(G::RU, G::ROWS - G::row0(j.u)) * G::S;   // the last unit may hold fewer rows
+                    int sb = bs;
+                    fbc_u32 sph = bph;
+#pragma unroll
+                    for (int st = 0; st < G::NST; ++st) {
+                        if (!(ok = fbc_wait(b_full0 + 8u * sb, sph, P, abort_flag, FBC_F3_ERR_WAIT))) break;
+                        fbc_tc_fence_after();
+                        issued = true;
+                        const fbc_u32 blo = (fbc_u32)bdesc0 + ((fbc_u32)sb * G::BSTAGE >> 4);
+#pragma unroll
+                        for (int q = 0; q < G::BS; ++q) {
+                            const int e = st * G::BS + q, k = e / G::S, s = e % G::S;
+                            if (e >= G::STEPS || (G::ROWS % G::RU != 0 && k > 0 && e >= steps)) break;
+                            const fbc_u32 ao = k * G::SLAB + (G::PACK ? 2u * s * G::PP * 16u
+                                                                      : (s % (G::GC / 16)) * 2u * G::PLANE + (s / (G::GC / 16)) * 16u);
+                            const fbc_u32 a1 = alo + (ao >> 4), b = blo + (q * G::BSTEP >> 4);
+                            fbc_umma_lo(d, a1, ahi, b, bhi, id3, e > 0 ? 1u : 0u);
+                            fbc_umma_lo(d + G::NT, a1 + (G::AORD >> 4), ahi, b, bhi, id2, 1u);
+                            fbc_umma_lo(d + 2 * G::NT, a1 + (2 * G::AORD >> 4), ahi, b, bhi, id1, 1u);
+                        }
+                        fbc_umma_commit<1>(b_empty0 + 8u * sb);
+                        if (++sb == P.nb) { sb = 0; sph ^= 1; }
+                    }
+                    if (!ok) break;
+                    fbc_umma_commit<1>(a_empty0 + 8u * as);
+                    fbc_umma_commit<1>(acc_full0 + 8u * acc);
+                    fbc_mbar_arrive(acc_full0 + 8u * acc);   // this thread has seen the converters' writes
+                }
+                if (++as == P.na) { as = 0; aph ^= 1; }
+                bs += G::NST;
+                while (bs >= P.nb) { bs -= P.nb; bph ^= 1; }
+            }
+            if (!ok && issued) {
+                fbc_umma_commit<1>(drain_bar + 8u * acc);
+                fbc_wait_drain(drain_bar + 8u * acc, 0, P);
+            }
+        }
+    } else {
+        // ------------------------------------------------------------ accumulate and store
+        constexpr int HC = G::NT / 2;          // columns of this warp
+        const int lq = warp & 3, half = warp >> 2;
+        const fbc_u32 trow = tmem + ((fbc_u32)(lq * 32) << 16) + (fbc_u32)(half * HC);
+        int acc = 0, ord = 0, ftile = -1;
+        bool tiny_bank = false;
+        fbc_u32 accph = 0;
+        bool ok = true;
+        // A finished tile is stored in pieces between the drains of the next one: storing
+        // it at once held both accumulator sets, and with them the tensor core, for a
+        // tenth of the time.
+        constexpr int NG = HC / 8, PER = (NG + G::NU - 1) / G::NU;    // groups of 8 columns, groups per drain
+        float out[HC];
+        int o_pg = 0, o_q = 0, o_n0 = 0, o_next = NG;
+        auto store_some = [&](int count) {
+#pragma unroll
+            for (int g = 0; g < NG; ++g)
+                if (g >= o_next && g < o_next + count) {
+                    float v8[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) v8[e] = out[8 * g + e];
+                    fbc_f3_store8<G>(P, o_pg, o_q, o_n0, half * HC + 8 * g, v8);
+                }
+            o_next += count;
+        };
+        for (int item = blockIdx.x; item < P.nitems && ok; item += gridDim.x, ++ord) {
+            const int mt = item % P.mtiles;
+            const int n0 = G::R > 1 ? 0 : (item / P.mtiles) * G::NT;
+            if (item / P.mtiles != ftile) {
+                ftile = item / P.mtiles;
+                int f = 0;
+                for (int b = lane; b < P.bank_blocks; b += 32) f |= P.flags[ftile * P.bank_blocks + b];
+                tiny_bank = __any_sync(0xFFFFFFFFu, f != 0);
+            }
+            float sum[HC];
+#pragma unroll
+            for (int k = 0; k < HC; ++k) sum[k] = 0.f;
+            for (int u = 0; u < G::NU; ++u) {
+                if (!(ok = fbc_wait(acc_full0 + 8u * acc, accph, P, abort_flag, FBC_F3_ERR_WAIT))) break;
+                fbc_tc_fence_after();
+                const fbc_u32 ta = trow + (fbc_u32)(acc * 3 * G::NT);
+#pragma unroll
+                for (int k = 0; k < HC; k += 8) {
+                    fbc_u32 r0[8], r1[8], r2[8];
+                    fbc_tmem_ld32x32b_x8_async(ta + k, r0);
+                    fbc_tmem_ld32x32b_x8_async(ta + G::NT + k, r1);
+                    fbc_tmem_ld32x32b_x8_async(ta + 2 * G::NT + k, r2);
+                    fbc_tmem_ld_wait();
+                    fbc_reg_fence8(r0);
+                    fbc_reg_fence8(r1);
+                    fbc_reg_fence8(r2);
+#pragma unroll
+                    for (int e = 0; e < 8; ++e)
+                        sum[k + e] += __uint_as_float(r0[e]) + (__uint_as_float(r1[e]) + __uint_as_float(r2[e]));
+                }
+                fbc_tc_fence_before();
+                __syncwarp();
+                if (lane == 0) fbc_mbar_arrive(acc_empty0 + 8u * acc);
+                acc ^= 1;
+                if (acc == 0) accph ^= 1;
+                if (o_next < NG) store_some(PER);
+            }
+            if (!ok) break;
+            // the tile is complete
+            const int v = mt * 128 + lq * 32 + lane;
+            o_pg = fbc_f3_row(v, P);
+            o_q = v - o_pg * P.vw;
+            o_n0 = n0;
+            const bool inside = o_q < P.out_w && o_pg * G::R < P.out_h;
+            // a sum is finite unless its difference with itself is not zero
+            float z = 0.f;
+#pragma unroll
+            for (int k = 0; k < HC; ++k) {
+                z += sum[k] - sum[k];
+                out[k] = sum[k];
+            }
+            const bool redo = tiny_bank || *(volatile int*)&s_tiny[ord & 15] == item + 1 ||
+                              __any_sync(0xFFFFFFFFu, inside && !(z == 0.f));
+            if (redo && inside) fbc_f3_recompute<G>(P, o_pg, o_q, n0, half * HC, half * HC + HC);
+            o_next = inside && !redo ? 0 : NG;
+            __syncwarp();
+        }
+        if (o_next < NG) store_some(NG);
+    }
+    __syncwarp();
+    fbc_tc_fence_before();
+    __syncthreads();
+    fbc_tc_fence_after();
+    if (warp == 15)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(G::TMEM));
+}

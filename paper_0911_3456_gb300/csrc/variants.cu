@@ -22,6 +22,8 @@ const char* rtcg_header_source() { return kRtcgDirectSrc; }
 const char* rtcg_tc_params_source() { return kRtcgTcParamsSrc; }
 const char* rtcg_ptx_source() { return kRtcgPtxSrc; }
 const char* rtcg_tc_source() { return kRtcgTcSrc; }
+const char* rtcg_f32tc_params_source() { return kRtcgF32tcParamsSrc; }
+const char* rtcg_f32tc_source() { return kRtcgF32tcSrc; }
 const char* rtcg_nn_params_source() { return kRtcgNnParamsSrc; }
 const char* rtcg_nn_source() { return kRtcgNnSrc; }
 

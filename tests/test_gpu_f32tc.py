@@ -1,0 +1,180 @@
+"""FP32 on the tensor cores (three-way BF16 split) against the FP64 oracle.
+
+Tolerance, derived from the arithmetic: a chunk of at most 16 steps truncates its
+FP32 accumulator by at most one unit (2^-23) of the magnitude summed so far at each
+step, the chunk sums are added with ordinary rounding, and the products left out are
+below 2^-26: |error| <= (16 * 2^-23 + (chunks + 4) * 2^-24) * sum |x| |w|.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_0911_3456_gb300 import inputs
+from helpers import dev, host, torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+# (H, W, D, N, fh, fw), forced tile: every depth layout (packed 1, 2, 4 and 8
+# channels, 16 and 32 per unit, odd depths), tap groups, folded rows with a ragged
+# last fold, several slab rows per unit with a ragged last unit, one and several
+# filter tiles, filters past the tile, pixel tiles with a ragged end, one pixel
+CASES = [
+    ((20, 37, 1, 5, 3, 4), "f32tc:nt=16,r=1,gc=8,jt=4,ru=2"),
+    ((19, 30, 2, 9, 4, 5), "f32tc:nt=32,r=3,gc=8,jt=5,ru=4"),
+    ((21, 33, 3, 7, 2, 3), "f32tc:nt=16,r=2,gc=8,jt=3,ru=1"),
+    ((33, 40, 4, 4, 8, 8), "f32tc:nt=32,r=8,gc=8,jt=8,ru=4"),
+    ((25, 31, 5, 6, 3, 3), "f32tc:nt=16,r=1,gc=8,jt=3,ru=3"),
+    ((30, 47, 8, 16, 9, 9), "f32tc:nt=64,r=4,gc=8,jt=5,ru=2"),
+    ((17, 140, 12, 40, 5, 3), "f32tc:nt=48,r=1,gc=16,jt=3,ru=3"),
+    ((18, 29, 20, 33, 2, 6), "f32tc:nt=48,r=1,gc=8,jt=4,ru=2"),
+    ((23, 26, 16, 64, 7, 7), "f32tc:nt=64,r=1,gc=16,jt=7,ru=2"),
+    ((15, 300, 32, 90, 3, 5), "f32tc:nt=48,r=1,gc=32,jt=5,ru=1"),
+    ((16, 21, 33, 17, 5, 11), "f32tc:nt=32,r=1,gc=16,jt=6,ru=1"),
+    ((12, 13, 64, 160, 1, 1), "f32tc:nt=80,r=1,gc=32,jt=1,ru=1"),
+    ((6, 7, 8, 3, 6, 7), "f32tc:nt=16,r=1,gc=8,jt=7,ru=3"),
+    ((4, 1, 4, 1, 2, 1), "f32tc:nt=16,r=3,gc=8,jt=1,ru=1"),
+]
+
+
+def _within(got, ref, mag, chunks):
+    assert np.all(np.abs(got - ref) <= (16 * 2.0 ** -23 + (chunks + 4) * 2.0 ** -24) * mag + 1e-30)
+
+
+@pytest.mark.parametrize("shape,spec", CASES)
+def test_forward_against_oracle_and_integers(shape, spec):
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    for kind in ("real", "int"):
+        wl = inputs.random_case(7100, *shape, kind=kind)
+        p = Plan(wl.x.shape, wl.w.shape)
+        p.set_variant(spec)
+        assert p.info()["fwd"]["spec"] == spec
+        y = host(p.forward(dev(wl.x, torch), dev(wl.w, torch)))
+        assert p.device_status() == 0
+        ref = oracle.fwd(wl.x, wl.w)
+        if kind == "int":
+            assert np.array_equal(y, ref)
+        else:
+            _within(y, ref, oracle.fwd(np.abs(wl.x), np.abs(wl.w)), shape[2] * shape[4] * shape[5])
+
+
+@pytest.mark.parametrize("clamp", [None, (-0.5, 0.5)])
+@pytest.mark.parametrize("shape,spec", [
+    ((20, 23, 16, 64, 7, 7), "f32tc:nt=64,r=4,gc=32,jt=7,ru=1"),
+    ((19, 26, 12, 40, 5, 3), "f32tc:nt=48,r=3,gc=8,jt=3,ru=4"),
+    ((24, 31, 5, 7, 3, 4), "f32tc:nt=16,r=1,gc=8,jt=4,ru=2"),
+    ((17, 40, 33, 3, 2, 5), "f32tc:nt=48,r=1,gc=8,jt=3,ru=1"),
+])
+def test_dx_against_oracle(shape, spec, clamp, monkeypatch):
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    monkeypatch.setenv("FBCORR_DX_VARIANT", spec)
+    wl = inputs.random_case(7200, *shape, with_g=True)
+    p = Plan(wl.x.shape, wl.w.shape, "f32", clamp)
+    y64 = oracle.fwd(wl.x, wl.w, epilogue=clamp)
+    y = y64.astype(np.float32)
+    dx, _ = p.backward(dev(wl.x, torch), dev(wl.w, torch), dev(wl.g, torch), dev(y, torch), need_dw=False)
+    assert p.info()["dx"]["spec"] == spec
+    assert p.device_status() == 0
+    ref = oracle.bwd_input(wl.g, wl.w, wl.x.shape, y=y.astype(np.float64), epilogue=clamp)
+    mag = oracle.bwd_input(np.abs(wl.g), np.abs(wl.w), wl.x.shape)
+    _within(host(dx), ref, mag, shape[3] * shape[4] * shape[5])
+
+
+def _special(shape):
+    """Inputs the BF16 split cannot carry: non-finite, at the range's ends, denormal."""
+    wl = inputs.random_case(7300, *shape)
+    x = wl.x.copy()
+    x[3, 4, 0] = np.inf
+    x[9, 20, 1] = np.nan
+    x[14, 7, 0] = -3.3e38
+    x[18, 25, 2] = 1e-39
+    return x, wl.w
+
+
+def test_values_outside_the_split_match_the_fma_kernel():
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    x, w = _special((24, 30, 8, 20, 3, 3))
+    xd, wd = dev(x, torch), dev(w, torch)
+    p = Plan(x.shape, w.shape)
+    p.set_variant("f32tc:nt=32,r=1,gc=8,jt=3,ru=3")
+    y = p.forward(xd, wd).cpu().numpy()
+    p.set_variant("default")
+    ref = p.forward(xd, wd).cpu().numpy()
+    assert np.array_equal(np.isnan(y), np.isnan(ref))
+    assert np.array_equal(np.isinf(y), np.isinf(ref)) and np.array_equal(y[np.isinf(y)], ref[np.isinf(ref)])
+    fin = np.isfinite(ref)
+    with np.errstate(all="ignore"):
+        exact, mag = oracle.fwd(x, w), oracle.fwd(np.abs(x), np.abs(w))
+    _within(y[fin].astype(np.float64), exact[fin], mag[fin], 72)
+
+
+@pytest.mark.parametrize("scale_x,scale_w", [(1e-33, 1.0), (1.0, 1e-34), (1e-38, 1e20), (1e19, 1e18)])
+def test_extreme_scales_keep_fp32_accuracy(scale_x, scale_w):
+    """Tiny images and banks (the third part of the split would underflow) and large ones."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    wl = inputs.random_case(7400, 20, 40, 8, 18, 3, 3)
+    x, w = (wl.x * np.float32(scale_x)), (wl.w * np.float32(scale_w))
+    p = Plan(x.shape, w.shape)
+    p.set_variant("f32tc:nt=32,r=1,gc=8,jt=3,ru=3")
+    y = host(p.forward(dev(x, torch), dev(w, torch)))
+    ref = oracle.fwd(x, w)
+    mag = oracle.fwd(np.abs(x), np.abs(w))
+    assert np.all(np.abs(y - ref) <= 2.0 ** -18 * mag + 1e-44)
+
+
+def test_scratch_too_small_runs_the_fma_kernel():
+    """Any workspace is accepted: none, or less than the kernel wants, gives the FMA result."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    wl = inputs.random_case(7500, 40, 50, 8, 32, 5, 5)
+    x, w = dev(wl.x, torch), dev(wl.w, torch)
+    p = Plan(wl.x.shape, wl.w.shape)
+    p.set_variant("f32tc:nt=32,r=1,gc=8,jt=5,ru=2")
+    y3 = p.forward(x, w)
+    small = p.forward(x, w, ws=torch.empty(64, dtype=torch.uint8, device="cuda"))
+    assert p.ws_fwd == 0
+    ref = oracle.fwd(wl.x, wl.w)
+    scale = np.abs(ref).max()
+    assert np.abs(host(y3) - ref).max() <= 1e-6 * scale and np.abs(host(small) - ref).max() <= 1e-6 * scale
+    from paper_0911_3456_gb300 import _capi as C
+    import ctypes
+    y = torch.empty_like(small)
+    C.call("fbcorr_forward", p.handle, *[ctypes.c_void_p(t.data_ptr()) for t in (x, w, y)], None, 0, None)
+    torch.cuda.synchronize()
+    assert torch.equal(y, small)
+
+
+def test_streams_and_capture():
+    """Overlapping calls of one plan on two streams, and a call captured in a graph."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    wl = inputs.random_case(7600, 64, 80, 16, 48, 5, 5)
+    p = Plan(wl.x.shape, wl.w.shape)
+    p.set_variant("f32tc:nt=48,r=1,gc=16,jt=5,ru=2")
+    x, w = dev(wl.x, torch), dev(wl.w, torch)
+    x2, w2 = x * 2, w * 3
+    y = p.forward(x, w)
+    y2 = p.forward(x2, w2)
+    torch.cuda.synchronize()
+    s1, s2 = torch.cuda.Stream(), torch.cuda.Stream()
+    for _ in range(5):
+        a = p.forward(x, w, torch.empty_like(y), stream=s1)
+        b = p.forward(x2, w2, torch.empty_like(y), stream=s2)
+        torch.cuda.synchronize()
+        assert torch.equal(a, y) and torch.equal(b, y2)
+    g = torch.cuda.CUDAGraph()
+    out = torch.empty_like(y)
+    with torch.cuda.graph(g):
+        p.forward(x, w, out)
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, y)
+    x.copy_(x2)
+    w.copy_(w2)
+    g.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(out, y2)
