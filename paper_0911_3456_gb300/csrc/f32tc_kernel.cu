@@ -57,8 +57,8 @@ long long pixel_tiles(const DirectProblem& pr, const F3Tile& t) {
     return ((pr.out_h + t.r - 1) / t.r * virtual_width(pr) + 127) / 128;
 }
 
-// Ring depths: three to six A slots, and the B stages that then fit, up to 16 (at
-// least 5: a copy takes about 1 us).
+// Ring depths: three to six A slots, and two B rings of the stages that then fit, up
+// to 8 each (at least 3: a copy takes about 1 us).
 bool layout(const DirectProblem& pr, const F3Tile& t, int* na, int* nb, size_t* smem) {
     if (t.nt < 16 || t.nt > 80 || t.nt % 16 || t.r < 1 || t.ru < 1 || t.jt < 1 || t.jt > pr.fw)
         return false;
@@ -69,14 +69,14 @@ bool layout(const DirectProblem& pr, const F3Tile& t, int* na, int* nb, size_t* 
     if ((pixel_tiles(pr, t) + 1) * 128 + 4096 >= (1ll << 31)) return false;
     const Geometry g = geometry(pr, t);
     if (t.ru > g.rows || g.ka > 18 || g.bank_chunks >= (1ll << 30)) return false;
-    for (int want : {8, 5})
+    for (int want : {4, 3})
         for (int a = 6; a >= 3; --a) {
             const long room = (long)kSmemMax - kBarBytes - (long)(a * g.aslot);
-            const int b = room < 0 ? 0 : (int)std::min<long>(16, room / (long)g.bstage);
+            const int b = room < 0 ? 0 : (int)std::min<long>(8, room / (long)(2 * g.bstage));
             if (b < want) continue;
             *na = a;
             *nb = b;
-            *smem = a * g.aslot + b * g.bstage + kBarBytes;
+            *smem = a * g.aslot + 2 * b * g.bstage + kBarBytes;
             return true;
         }
     return false;
@@ -86,11 +86,12 @@ bool layout(const DirectProblem& pr, const F3Tile& t, int* na, int* nb, size_t* 
 // core, or longer at narrow tiles (measured alone: 123, 144, 168, 204, 244 cycles
 // at NT = 16 .. 80); a unit measured 600 to 900 cycles more (barriers, commits, the
 // drain that is not hidden).
-double model_cycles(const DirectProblem& pr, const F3Tile& t, int sm_count) {
+// shared: the launch runs beside others that fill the SMs its last round leaves idle.
+double model_cycles(const DirectProblem& pr, const F3Tile& t, int sm_count, bool shared) {
     const Geometry g = geometry(pr, t);
     const double step = std::max(102.0 + 1.2 * t.nt, 3.06 * t.nt);
     const long long items = pixel_tiles(pr, t) * filter_tiles(pr, t);
-    const double rounds = (double)((items + sm_count - 1) / sm_count);
+    const double rounds = shared ? (double)items / sm_count : (double)((items + sm_count - 1) / sm_count);
     const double mma = t.ru * g.s * step + 700, conv = 90.0 * g.ka + 300, drain = 400.0 + 8 * t.nt;
     return rounds * g.nu * std::max(std::max(mma, conv), drain) + 4000;
 }
@@ -118,7 +119,7 @@ bool f3_parse_spec(const std::string& s, F3Tile* t) {
     return true;
 }
 
-std::vector<F3Tile> f3_ranked(const DirectProblem& pr, int sm_count, double* best_cycles) {
+std::vector<F3Tile> f3_ranked(const DirectProblem& pr, int sm_count, double* best_cycles, bool shared) {
     std::vector<std::pair<double, F3Tile>> all;
     const int npad = (pr.nf + 15) / 16 * 16;
     for (int fold = 1; fold <= std::min(16, pr.out_h); ++fold) {
@@ -147,7 +148,7 @@ std::vector<F3Tile> f3_ranked(const DirectProblem& pr, int sm_count, double* bes
                     size_t smem;
                     if (!layout(pr, t, &na, &nb, &smem)) continue;
                     // three A slots measured 5 % behind four or more
-                    all.push_back({model_cycles(pr, t, sm_count) * (na < 4 ? 1.06 : 1.0), t});
+                    all.push_back({model_cycles(pr, t, sm_count, shared) * (na < 4 ? 1.06 : 1.0), t});
                 }
                 if (g.s <= 4) break;   // splitting the taps further only adds slabs
             }
@@ -166,15 +167,16 @@ std::vector<F3Tile> f3_ranked(const DirectProblem& pr, int sm_count, double* bes
 // 16x9x9 (0.3 GFLOP) 11 / 19, 187x233x12 * 40x5x3 (0.6) 20 / 20, 256x256x8 *
 // 64x9x9 (5.1) 115 / 35, 2048x2048x4 * 4x8x8 (8.5) 180 / 100, 512x512x32 *
 // 256x5x5 (106) 1937 / 394.
-bool f3_wins(const DirectProblem& pr, int sm_count, F3Tile* t) {
+// Beside other launches (shared) neither the launch nor the last round counts.
+bool f3_wins(const DirectProblem& pr, int sm_count, F3Tile* t, bool shared) {
     const std::string sw = env_str("FBCORR_F32TC", "1");
     if (sw == "0") return false;
     double cycles = 0;
-    const std::vector<F3Tile> r = f3_ranked(pr, sm_count, &cycles);
+    const std::vector<F3Tile> r = f3_ranked(pr, sm_count, &cycles, shared);
     if (r.empty()) return false;
     *t = r.front();
     const double flops = 2.0 * pr.out_h * pr.out_w * pr.nf * pr.fh * pr.fw * pr.c;
-    return sw == "force" || cycles + 9000 < 0.9 * (flops / (sm_count * 256 * 0.65) + 4000);
+    return sw == "force" || cycles + (shared ? 0 : 9000) < 0.9 * (flops / (sm_count * 256 * 0.65) + (shared ? 0 : 4000));
 }
 
 size_t f3_ws_bytes(const DirectProblem& pr, const F3Tile& t) {
@@ -232,8 +234,8 @@ fbcorr_status_t f3_build(const DirectProblem& pr, const F3Tile& t, int sm_count,
     return FBCORR_OK;
 }
 
-fbcorr_status_t f3_run(const F3Launch& l, const DirectProblem& pr, const float* x, const float* m, const float* w,
-                       float* y, void* ws, float lo, float hi, int* err_word, cudaStream_t s) {
+FbcF3Params f3_params(const F3Launch& l, const DirectProblem& pr, const float* x, const float* m, const float* w,
+                      float* y, void* ws, float lo, float hi, int* err_word) {
     const Geometry g = geometry(pr, l.tile);
     FbcF3Params k;
     memset(&k, 0, sizeof k);
@@ -260,17 +262,24 @@ fbcorr_status_t f3_run(const F3Launch& l, const DirectProblem& pr, const float* 
     k.nitems = k.mtiles * l.filter_tiles;
     k.na = l.na; k.nb = l.nb;
     k.b_off = (unsigned)(l.na * g.aslot);
-    k.bar_off = (unsigned)(k.b_off + l.nb * g.bstage);
-    void* args[] = {&k};
-    FBC_TRY(launch_dependent(l.bank, dim3(l.bank_blocks, l.filter_tiles), args, s));
-    return launch_dependent(l.kernel, dim3(l.grid), args, s);
+    k.bar_off = (unsigned)(k.b_off + 2 * l.nb * g.bstage);
+    return k;
 }
 
+dim3 f3_bank_grid(const F3Launch& l) { return dim3((unsigned)l.bank_blocks, (unsigned)l.filter_tiles); }
+
+fbcorr_status_t f3_run(const F3Launch& l, const DirectProblem& pr, const float* x, const float* m, const float* w,
+                       float* y, void* ws, float lo, float hi, int* err_word, cudaStream_t s) {
+    FbcF3Params k = f3_params(l, pr, x, m, w, y, ws, lo, hi, err_word);
+    void* args[] = {&k};
+    FBC_TRY(launch_dependent(l.bank, f3_bank_grid(l), args, s));
+    return launch_dependent(l.kernel, dim3(l.grid), args, s);
+}
 
 fbcorr_status_t f3_tune(const DeviceInfo& dev, const DirectProblem& pr, cudaStream_t s, int* err_word, float* ms,
                         std::string* spec) {
     spec->clear();
-    std::vector<F3Tile> tiles = f3_ranked(pr, dev.sm_count, nullptr);
+    std::vector<F3Tile> tiles = f3_ranked(pr, dev.sm_count, nullptr, false);
     if (env_str("FBCORR_F32TC", "1") == "0" || tiles.empty()) return FBCORR_OK;
     tiles.resize(std::min<size_t>(tiles.size(), 8));
     std::vector<std::string> srcs;

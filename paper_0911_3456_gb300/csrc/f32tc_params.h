@@ -28,7 +28,7 @@ struct FbcF3Params {
     int mtiles;                 // 128-pixel tiles over ceil(out_h / R) * vw virtual pixels
     int nitems;                 // mtiles x filter tiles
     int bank_blocks;            // blocks of the bank split per filter tile
-    int na, nb;                 // A slots, B stages
+    int na, nb;                 // A slots, B stages per issuer
     unsigned int b_off, bar_off;    // B ring and barrier table in shared memory (A ring at 0)
 };
 

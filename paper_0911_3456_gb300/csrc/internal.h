@@ -248,18 +248,26 @@ struct F3Launch {
 std::string f3_spec(const F3Tile& t);
 bool f3_parse_spec(const std::string& s, F3Tile* t);
 // Every tile the kernel takes the problem with (none: it does not), by the cost model, best first.
-std::vector<F3Tile> f3_ranked(const DirectProblem& pr, int sm_count, double* best_cycles);
+std::vector<F3Tile> f3_ranked(const DirectProblem& pr, int sm_count, double* best_cycles, bool shared = false);
 // Time the model's first tiles on patterned buffers; *spec is empty when there are none.
 fbcorr_status_t f3_tune(const DeviceInfo& dev, const DirectProblem& pr, cudaStream_t s, int* err_word, float* ms,
                         std::string* spec);
 // The best rated tile, and whether the model expects it to be faster than the FP32 FMA kernels.
-bool f3_wins(const DirectProblem& pr, int sm_count, F3Tile* t);
+bool f3_wins(const DirectProblem& pr, int sm_count, F3Tile* t, bool shared = false);
 size_t f3_ws_bytes(const DirectProblem& pr, const F3Tile& t);
 std::string f3_kernel_source(const DirectProblem& pr, const F3Tile& t, const std::string& name);   // + name "_bank"
 std::string f3_kernel_name(const DirectProblem& pr, const F3Tile& t);
 fbcorr_status_t f3_build(const DirectProblem& pr, const F3Tile& t, int sm_count, F3Launch* out);
+dim3 f3_bank_grid(const F3Launch& l);
 fbcorr_status_t f3_run(const F3Launch& l, const DirectProblem& pr, const float* x, const float* m, const float* w,
                        float* y, void* ws, float lo, float hi, int* err_word, cudaStream_t s);
+
+}  // namespace fbc
+struct FbcF3Params;   // f32tc_params.h
+namespace fbc {
+// The parameters of both kernels of a call (graph nodes).
+FbcF3Params f3_params(const F3Launch& l, const DirectProblem& pr, const float* x, const float* m, const float* w,
+                      float* y, void* ws, float lo, float hi, int* err_word);
 
 // ---- argument validation (api.cu) -------------------------------------------------------
 fbcorr_status_t validate_shapes(const int64_t* in, const int64_t* fs, fbcorr_dtype_t dtype,

@@ -44,8 +44,12 @@
 // Roles per CTA (persistent, one per SM): warps 0..7 add the chunk sums up and
 // store; warps 8..12 read x from global memory (prefetched in registers), split it
 // and write the A slots; a thread of warp 13 copies the B stages; a thread of
-// warp 14 issues the MMAs of every other unit, one of warp 15 the rest, each into
-// its own accumulator set, so chunk sums are drained while the next chunk runs.
+// warp 14 issues the MMAs of every other unit, one of warp 15 the rest, each from
+// its own B ring into its own accumulator set, so chunk sums are drained while the
+// next chunk runs.  (A barrier is only ever waited for by threads that have seen its
+// phase before: the parity does not tell phase k from k - 2.  B stages therefore
+// have one ring per issuer; A slots, which the converters fill in order, do not need
+// it: an issuer that has seen unit u - 2 filled knows that every earlier one was.)
 //
 // Values the split cannot carry.  Non-finite inputs or overflow give a
 // non-finite sum, and a non-zero |v| < 2^-100 (whose third part could fall below
@@ -390,12 +394,12 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const fbc_u32 sbase = fbc_smem_addr(fbc_tc_smem);
-    // barrier table: a_full[na] a_empty[na] b_full[nb] b_empty[nb] acc_full[2] acc_empty[2] drain[2]
+    // barrier table: a_full[na] a_empty[na] b_full[2][nb] b_empty[2][nb] acc_full[2] acc_empty[2] drain[2]
     const fbc_u32 a_full0 = sbase + P.bar_off;
     const fbc_u32 a_empty0 = a_full0 + 8u * P.na;
     const fbc_u32 b_full0 = a_empty0 + 8u * P.na;
-    const fbc_u32 b_empty0 = b_full0 + 8u * P.nb;
-    const fbc_u32 acc_full0 = b_empty0 + 8u * P.nb;
+    const fbc_u32 b_empty0 = b_full0 + 16u * P.nb;
+    const fbc_u32 acc_full0 = b_empty0 + 16u * P.nb;
     const fbc_u32 acc_empty0 = acc_full0 + 16u;
     const fbc_u32 drain_bar = acc_empty0 + 16u;
     if (threadIdx.x == 0) {
@@ -403,7 +407,7 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
             fbc_mbar_init(a_full0 + 8u * s, FBC_F3_CONV_WARPS);
             fbc_mbar_init(a_empty0 + 8u * s, 1);
         }
-        for (int s = 0; s < P.nb; ++s) {
+        for (int s = 0; s < 2 * P.nb; ++s) {
             fbc_mbar_init(b_full0 + 8u * s, 1);
             fbc_mbar_init(b_empty0 + 8u * s, 1);
         }
@@ -475,27 +479,66 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
     } else if (warp == 13) {
         if (lane == 0) {
             // -------------------------------------------------------- bank producer
-            int bs = 0;
-            fbc_u32 bph = 0, it = 0;
+            // both rings in turn, whichever has a free stage
+            struct {
+                FbcF3Pos<G> j;
+                int st, bs;
+                fbc_u32 ph, it;
+            } q[2];
+#pragma unroll
+            for (int r = 0; r < 2; ++r) {
+                q[r].j.start();
+                if (r == 1) q[r].j.next();
+                q[r].st = q[r].bs = 0;
+                q[r].ph = q[r].it = 0;
+            }
+            fbc_u64 t0 = fbc_globaltimer();
+            fbc_u32 idle = 0;
             bool ok = true;
-            FbcF3Pos<G> j;
-            for (j.start(); j.valid(P); j.next()) {
-                const unsigned char* src = P.bank + ((long long)(j.item / P.mtiles) * G::NU + j.u) * G::BUNIT;
-#pragma unroll 1
-                for (int st = 0; st < G::NST; ++st) {
-                    if (!(ok = fbc_wait(b_empty0 + 8u * bs, bph ^ 1, P, abort_flag, FBC_F3_ERR_WAIT))) break;
-                    const fbc_u32 bytes = min(G::BSTAGE, G::BUNIT - st * G::BSTAGE);
-                    fbc_mbar_expect_tx(b_full0 + 8u * bs, bytes);
-                    fbc_bulk_g2s(sbase + P.b_off + (fbc_u32)bs * G::BSTAGE, src + st * G::BSTAGE, bytes, b_full0 + 8u * bs);
-                    ++it;
-                    if (++bs == P.nb) { bs = 0; bph ^= 1; }
+            while (ok && (q[0].j.valid(P) || q[1].j.valid(P))) {
+                bool moved = false;
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    if (!q[r].j.valid(P)) continue;
+                    const int slot = r * P.nb + q[r].bs;
+                    if (!fbc_mbar_test(b_empty0 + 8u * slot, q[r].ph ^ 1)) continue;
+                    moved = true;
+                    const fbc_u32 off = (fbc_u32)q[r].st * G::BSTAGE;
+                    const fbc_u32 bytes = min(G::BSTAGE, G::BUNIT - off);
+                    fbc_mbar_expect_tx(b_full0 + 8u * slot, bytes);
+                    fbc_bulk_g2s(sbase + P.b_off + (fbc_u32)slot * G::BSTAGE,
+                                 P.bank + ((long long)(q[r].j.item / P.mtiles) * G::NU + q[r].j.u) * G::BUNIT + off, bytes,
+                                 b_full0 + 8u * slot);
+                    ++q[r].it;
+                    if (++q[r].bs == P.nb) { q[r].bs = 0; q[r].ph ^= 1; }
+                    if (++q[r].st == G::NST) {
+                        q[r].st = 0;
+                        q[r].j.next();
+                        q[r].j.next();
+                    }
                 }
-                if (!ok) break;
+                if (moved) {
+                    idle = 0;
+                } else if ((++idle & 63u) == 0) {
+                    // nothing freed for a while: stop with the CTA, or after the bound
+                    if (idle == 64u) t0 = fbc_globaltimer();
+                    if (*abort_flag) ok = false;
+                    if (fbc_globaltimer() - t0 > P.wait_ns) {
+                        *abort_flag = 1;
+                        *(volatile int*)P.err = FBC_F3_ERR_WAIT;
+                        __threadfence_system();
+                        ok = false;
+                    }
+                }
             }
             if (!ok) {
-                // wait (bounded) for the copies still in flight into the ring
-                const fbc_u32 k0 = it > (fbc_u32)P.nb ? it - P.nb : 0;
-                for (fbc_u32 k = k0; k < it; ++k) fbc_wait_drain(b_full0 + 8u * (k % P.nb), (k / P.nb) & 1, P);
+                // wait (bounded) for the copies still in flight into the rings
+#pragma unroll
+                for (int r = 0; r < 2; ++r) {
+                    const fbc_u32 k0 = q[r].it > (fbc_u32)P.nb ? q[r].it - P.nb : 0;
+                    for (fbc_u32 k = k0; k < q[r].it; ++k)
+                        fbc_wait_drain(b_full0 + 8u * (r * P.nb + k % P.nb), (k / P.nb) & 1, P);
+                }
             }
         }
     } else if (warp >= 14) {
@@ -511,7 +554,8 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
             // descriptors: the start address (16-byte units) sits in the low bits of the
             // low word and never carries out of its field; the high word is constant
             const fbc_u64 adesc0 = fbc_smem_desc(sbase, G::PACK ? 16u * G::PP : G::PLANE, 128);
-            const fbc_u64 bdesc0 = fbc_smem_desc(sbase + P.b_off, G::BCH, 128);
+            const fbc_u32 ring = (fbc_u32)(warp - 14) * P.nb;      // this thread's B stages
+            const fbc_u64 bdesc0 = fbc_smem_desc(sbase + P.b_off + ring * G::BSTAGE, G::BCH, 128);
             const fbc_u32 ahi = (fbc_u32)(adesc0 >> 32), bhi = (fbc_u32)(bdesc0 >> 32);
             const int acc = warp - 14;         // this thread's accumulator set
             const fbc_u32 d = tmem + (fbc_u32)(acc * 3 * G::NT);
@@ -527,14 +571,12 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
                     accph ^= 1;
                     const fbc_u32 alo = (fbc_u32)adesc0 + ((fbc_u32)as * G::ASLOT >> 4);
                     const int steps = min(G::RU, G::ROWS - G::row0(j.u)) * G::S;   // the last unit may hold fewer rows
-                    int sb = bs;
-                    fbc_u32 sph = bph;
 #pragma unroll
                     for (int st = 0; st < G::NST; ++st) {
-                        if (!(ok = fbc_wait(b_full0 + 8u * sb, sph, P, abort_flag, FBC_F3_ERR_WAIT))) break;
+                        if (!(ok = fbc_wait(b_full0 + 8u * (ring + bs), bph, P, abort_flag, FBC_F3_ERR_WAIT))) break;
                         fbc_tc_fence_after();
                         issued = true;
-                        const fbc_u32 blo = (fbc_u32)bdesc0 + ((fbc_u32)sb * G::BSTAGE >> 4);
+                        const fbc_u32 blo = (fbc_u32)bdesc0 + ((fbc_u32)bs * G::BSTAGE >> 4);
 #pragma unroll
                         for (int q = 0; q < G::BS; ++q) {
                             const int e = st * G::BS + q, k = e / G::S, s = e % G::S;
@@ -546,8 +588,8 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
                             fbc_umma_lo(d + G::NT, a1 + (G::AORD >> 4), ahi, b, bhi, id2, 1u);
                             fbc_umma_lo(d + 2 * G::NT, a1 + (2 * G::AORD >> 4), ahi, b, bhi, id1, 1u);
                         }
-                        fbc_umma_commit<1>(b_empty0 + 8u * sb);
-                        if (++sb == P.nb) { sb = 0; sph ^= 1; }
+                        fbc_umma_commit<1>(b_empty0 + 8u * (ring + bs));
+                        if (++bs == P.nb) { bs = 0; bph ^= 1; }
                     }
                     if (!ok) break;
                     fbc_umma_commit<1>(a_empty0 + 8u * as);
@@ -555,8 +597,6 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
                     fbc_mbar_arrive(acc_full0 + 8u * acc);   // this thread has seen the converters' writes
                 }
                 if (++as == P.na) { as = 0; aph ^= 1; }
-                bs += G::NST;
-                while (bs >= P.nb) { bs -= P.nb; bph ^= 1; }
             }
             if (!ok && issued) {
                 fbc_umma_commit<1>(drain_bar + 8u * acc);

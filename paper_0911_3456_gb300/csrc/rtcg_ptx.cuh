@@ -44,6 +44,18 @@ __device__ __forceinline__ bool fbc_mbar_try_wait(fbc_u32 bar, fbc_u32 parity) {
     return ok != 0;
 }
 
+// The same test without a wait.
+__device__ __forceinline__ bool fbc_mbar_test(fbc_u32 bar, fbc_u32 parity) {
+    fbc_u32 ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.b32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 __device__ __forceinline__ void fbc_mbar_arrive(fbc_u32 bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
