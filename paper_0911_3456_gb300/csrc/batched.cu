@@ -15,6 +15,12 @@
 //     Image pointers are kernel parameters; when a call passes different
 //     pointers the instantiated graph's kernel node is updated in place
 //     (launches already enqueued keep their old parameters).
+// Images that the FP32 tensor-core kernel computes faster (rtcg_f32tc.cuh, by
+// the cost model) are branches of the same graph instead: each image's bank split
+// and its correlation, all independent, so that the CTAs of one image fill the SMs
+// that another leaves idle.  The persistent kernel takes the rest.  Measured on 24
+// images (205 GFLOP, GB300): 3752 us with the persistent kernel alone (0.68 of the
+// FP32 FMA peak), 1085 us with every image on the tensor cores.
 #include <algorithm>
 #include <array>
 #include <cstdio>
@@ -24,6 +30,7 @@
 #include <sstream>
 #include <tuple>
 
+#include "f32tc_params.h"
 #include "internal.h"
 
 using namespace fbc;
@@ -42,6 +49,15 @@ constexpr int kMetaInts = 6;
 constexpr int kArgsHeader = 40;                   // bytes before the pointer table
 constexpr int kPtrEntry = 24;
 constexpr int kBatchMaxBlock = 32;                // accumulators per thread (85 registers at 3 CTAs/SM)
+
+// An image on the tensor cores: its launch, its part of the plan's scratch and its graph nodes.
+struct BatchF3 {
+    int image = 0;
+    DirectProblem pr;
+    F3Launch l;
+    size_t ws_off = 0;
+    cudaGraphNode_t bank_node = nullptr, node = nullptr;
+};
 
 struct BatchVariant {
     int fh, fw, d, nclass;
@@ -70,7 +86,11 @@ struct fbcorr_batch_plan {
     std::vector<unsigned char> args;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
-    cudaGraphNode_t knode = nullptr;
+    cudaGraphNode_t knode = nullptr;      // of the persistent kernel (null: no image left for it)
+    std::vector<BatchF3> f3;
+    unsigned char* f3_ws = nullptr;       // scratch of every tensor-core image
+    int* err_host = nullptr;              // bounded-wait failure flag (host-mapped)
+    int* err_dev = nullptr;
     long long flops = 0;
 };
 
@@ -138,6 +158,8 @@ void destroy(fbcorr_batch_plan* b) {
     if (b->work) cudaFree(b->work);
     if (b->meta) cudaFree(b->meta);
     if (b->counter) cudaFree(b->counter);
+    if (b->f3_ws) cudaFree(b->f3_ws);
+    if (b->err_host) cudaFreeHost(b->err_host);
     delete b;
 }
 
@@ -149,9 +171,10 @@ void destroy(fbcorr_batch_plan* b) {
 fbcorr_status_t select_variants(fbcorr_batch_plan* b, bool allow_tuning) {
     std::map<std::tuple<int, int, int, int>, int> key_to_var;
     std::vector<int> rep_image;   // per variant: its largest image
-    b->var_of.resize(b->n);
+    b->var_of.assign(b->n, -1);
     b->variants.clear();
     for (int k = 0; k < b->n; ++k) {
+        if (std::any_of(b->f3.begin(), b->f3.end(), [k](const BatchF3& f) { return f.image == k; })) continue;
         const auto& s = b->shp[k];
         const auto key = std::make_tuple((int)s[4], (int)s[5], (int)s[2], filter_class(s[3]));
         auto it = key_to_var.find(key);
@@ -243,14 +266,63 @@ size_t batch_smem(const fbcorr_batch_plan* b) {
     return smem;
 }
 
+// The images that run on the tensor cores, their kernels (compiled in parallel)
+// and scratch, largest first.
+fbcorr_status_t build_f3(fbcorr_batch_plan* b) {
+    if (env_str("FBCORR_BATCH_KS", "0") == "1") return FBCORR_OK;   // the K-split tiles are asked for
+    const int epi = b->epi.kind == FBCORR_EPI_CLAMP ? 1 : 0;
+    std::vector<std::string> srcs;
+    for (int k = 0; k < b->n; ++k) {
+        const auto& s = b->shp[k];
+        BatchF3 f;
+        f.image = k;
+        f.pr = DirectProblem{(int)s[0], (int)s[1], (int)s[2], (int)(s[0] - s[4] + 1), (int)(s[1] - s[5] + 1), (int)s[3],
+                             (int)s[4], (int)s[5], 0, 0, 0, epi, 0, ""};
+        if (!f3_wins(f.pr, b->dev.sm_count, &f.l.tile, true)) continue;
+        srcs.push_back(f3_kernel_source(f.pr, f.l.tile, f3_kernel_name(f.pr, f.l.tile)));
+        b->f3.push_back(f);
+    }
+    if (b->f3.empty()) return FBCORR_OK;
+    rtcg_precompile(srcs);
+    size_t bytes = 0;
+    for (BatchF3& f : b->f3) {
+        const fbcorr_status_t s = f3_build(f.pr, f.l.tile, b->dev.sm_count, &f.l);
+        if (s == FBCORR_ERR_NVRTC) {     // no code generation: the persistent kernel reports it
+            b->f3.clear();
+            return FBCORR_OK;
+        }
+        FBC_TRY(s);
+        f.ws_off = bytes;
+        bytes += (f.l.ws_bytes + 255) / 256 * 256;
+    }
+    std::stable_sort(b->f3.begin(), b->f3.end(), [](const BatchF3& a, const BatchF3& c) {
+        auto work = [](const DirectProblem& p) { return (double)p.out_h * p.out_w * p.nf * p.fh * p.fw * p.c; };
+        return work(a.pr) > work(c.pr);
+    });
+    FBC_CUDA(cudaMalloc(&b->f3_ws, bytes));
+    FBC_CUDA(cudaHostAlloc((void**)&b->err_host, sizeof(int), cudaHostAllocMapped));
+    FBC_CUDA(cudaHostGetDevicePointer((void**)&b->err_dev, b->err_host, 0));
+    *b->err_host = 0;
+    return FBCORR_OK;
+}
+
+FbcF3Params image_params(const fbcorr_batch_plan* b, const BatchF3& f) {
+    const unsigned char* e = b->args.data() + kArgsHeader + (size_t)f.image * kPtrEntry;
+    const void* p[3];
+    memcpy(p, e, 24);
+    return f3_params(f.l, f.pr, (const float*)p[0], nullptr, (const float*)p[1], (float*)p[2], b->f3_ws + f.ws_off,
+                     b->epi.lo, b->epi.hi, b->err_dev);
+}
+
 fbcorr_status_t build(fbcorr_batch_plan* b) {
+    FBC_TRY(build_f3(b));
     FBC_TRY(select_variants(b, true));
     const size_t smem = batch_smem(b);
 
-    // ---- one generated kernel for the whole batch
+    // ---- one generated kernel for the rest of the batch
     char name[64];
     snprintf(name, sizeof name, "fbc_batch");
-    FBC_TRY(rtcg_kernel(batch_source(b), name, smem, kBatchThreads, &b->kern));
+    if (!b->variants.empty()) FBC_TRY(rtcg_kernel(batch_source(b), name, smem, kBatchThreads, &b->kern));
 
     // ---- work list, largest tiles first
     struct Item {
@@ -263,6 +335,8 @@ fbcorr_status_t build(fbcorr_batch_plan* b) {
     for (int k = 0; k < b->n; ++k) {
         const auto& s = b->shp[k];
         const int Ho = (int)(s[0] - s[4] + 1), Wo = (int)(s[1] - s[5] + 1), N = (int)s[3];
+        b->flops += 2LL * Ho * Wo * N * s[4] * s[5] * s[2];
+        if (b->var_of[k] < 0) continue;
         const BatchVariant& bv = b->variants[b->var_of[k]];
         const DirectTile& t = bv.tile;
         const int gx = (Wo + t.bw() - 1) / t.bw(), gy = (Ho + t.bh() - 1) / t.bh(), gz = (N + t.bn() - 1) / t.bn();
@@ -276,7 +350,6 @@ fbcorr_status_t build(fbcorr_batch_plan* b) {
         meta[kMetaInts * k + 3] = Wo;
         meta[kMetaInts * k + 4] = N;
         meta[kMetaInts * k + 5] = b->var_of[k];
-        b->flops += 2LL * Ho * Wo * N * s[4] * s[5] * s[2];
     }
     std::stable_sort(items.begin(), items.end(),
                      [](const Item& a, const Item& c) { return a.cost > c.cost; });
@@ -284,16 +357,18 @@ fbcorr_status_t build(fbcorr_batch_plan* b) {
     std::vector<int4> work(items.size());
     for (size_t i = 0; i < items.size(); ++i) work[i] = items[i].w;
 
-    FBC_CUDA(cudaMalloc(&b->work, sizeof(int4) * work.size()));
     FBC_CUDA(cudaMalloc(&b->meta, sizeof(int) * meta.size()));
     FBC_CUDA(cudaMalloc(&b->counter, sizeof(int)));
-    FBC_CUDA(cudaMemcpy(b->work, work.data(), sizeof(int4) * work.size(), cudaMemcpyHostToDevice));
+    if (!work.empty()) {
+        FBC_CUDA(cudaMalloc(&b->work, sizeof(int4) * work.size()));
+        FBC_CUDA(cudaMemcpy(b->work, work.data(), sizeof(int4) * work.size(), cudaMemcpyHostToDevice));
+    }
     FBC_CUDA(cudaMemcpy(b->meta, meta.data(), sizeof(int) * meta.size(), cudaMemcpyHostToDevice));
     FBC_CUDA(cudaMemset(b->counter, 0, sizeof(int)));
 
     // ---- persistent grid: every co-resident CTA, at most one per work item
-    FBC_TRY(kernel_occupancy(b->kern, &b->blocks_per_sm));
-    if (b->blocks_per_sm < 1)
+    if (b->nwork > 0) FBC_TRY(kernel_occupancy(b->kern, &b->blocks_per_sm));
+    if (b->nwork > 0 && b->blocks_per_sm < 1)
         return set_error(FBCORR_ERR_UNSUPPORTED, "batched kernel cannot be resident (smem %zu)", smem);
     b->grid = std::min(b->nwork, b->blocks_per_sm * std::max(1, b->dev.sm_count));
 
@@ -311,8 +386,19 @@ fbcorr_status_t build(fbcorr_batch_plan* b) {
     memcpy(a + 28, &lo, 4);
     memcpy(a + 32, &hi, 4);
 
-    // ---- the graph: zero the counter, then the persistent kernel
+    // ---- the graph: per tensor-core image the split of its bank and its
+    // correlation; zero the counter, then the persistent kernel
     FBC_CUDA(cudaGraphCreate(&b->graph, 0));
+    for (BatchF3& f : b->f3) {
+        FbcF3Params k = image_params(b, f);
+        void* kargs[] = {&k};
+        FBC_TRY(graph_add_kernel(b->graph, nullptr, 0, f.l.bank, f3_bank_grid(f.l), kargs, &f.bank_node));
+        FBC_TRY(graph_add_kernel(b->graph, &f.bank_node, 1, f.l.kernel, dim3(f.l.grid), kargs, &f.node));
+    }
+    if (b->nwork == 0) {
+        FBC_CUDA(cudaGraphInstantiate(&b->exec, b->graph, 0));
+        return FBCORR_OK;
+    }
     cudaMemsetParams ms;
     memset(&ms, 0, sizeof ms);
     ms.dst = b->counter;
@@ -417,6 +503,7 @@ fbcorr_status_t fbcorr_batch_plan_info(fbcorr_batch_plan_t b, char* buf, size_t 
     o << "{\"images\":" << b->n << ",\"work_items\":" << b->nwork << ",\"grid\":" << b->grid
       << ",\"blocks_per_sm\":" << b->blocks_per_sm << ",\"threads\":" << kBatchThreads
       << ",\"smem\":" << b->kern.smem << ",\"flops\":" << b->flops << ",\"launches\":1"
+      << ",\"tensor_images\":" << b->f3.size() << ",\"kernels\":" << 2 * b->f3.size() + (b->nwork > 0 ? 1 : 0)
       << ",\"variants\":[";
     for (size_t v = 0; v < b->variants.size(); ++v) {
         const auto& bv = b->variants[v];
@@ -435,7 +522,12 @@ fbcorr_status_t fbcorr_forward_batched(fbcorr_batch_plan_t b, const float* const
     (void)ws;
     (void)ws_bytes;
     if (!b || !x || !w || !y) return set_error(FBCORR_ERR_INVALID_ARG, "NULL argument");
-    bool changed = false;
+    if (b->err_host && *(volatile int*)b->err_host != 0) {
+        *(volatile int*)b->err_host = 0;
+        return set_error(FBCORR_ERR_TIMEOUT, "a kernel of an earlier call gave up a bounded wait");
+    }
+    std::vector<char> changed(b->n, 0);
+    bool any = false;
     for (int k = 0; k < b->n; ++k) {
         if (!x[k] || !w[k] || !y[k]) return set_error(FBCORR_ERR_INVALID_ARG, "NULL pointer for image %d", k);
         if ((((uintptr_t)x[k]) | ((uintptr_t)w[k]) | ((uintptr_t)y[k])) & 15u)
@@ -445,10 +537,18 @@ fbcorr_status_t fbcorr_forward_batched(fbcorr_batch_plan_t b, const float* const
         memcpy(old, e, 24);
         if (old[0] != x[k] || old[1] != w[k] || old[2] != y[k]) {
             write_ptr_entry(b->args, k, x[k], w[k], y[k]);
-            changed = true;
+            changed[k] = old[1] != w[k] ? 2 : 1;
+            any = any || b->var_of[k] >= 0;
         }
     }
-    if (changed) {
+    for (const BatchF3& f : b->f3) {
+        if (!changed[f.image]) continue;
+        FbcF3Params p = image_params(b, f);
+        void* kargs[] = {&p};
+        if (changed[f.image] == 2) FBC_TRY(graph_set_kernel(b->exec, f.bank_node, f.l.bank, f3_bank_grid(f.l), kargs));
+        FBC_TRY(graph_set_kernel(b->exec, f.node, f.l.kernel, dim3(f.l.grid), kargs));
+    }
+    if (any) {
         void* kargs[] = {b->args.data()};
         FBC_TRY(graph_set_kernel(b->exec, b->knode, b->kern, dim3(b->grid), kargs));
     }
