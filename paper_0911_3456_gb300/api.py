@@ -182,7 +182,7 @@ class Plan:
         dw = torch.empty(self.filt_shape, dtype=torch.float32, device=dev) if need_dw else None
         if ws is None and (need_dx or need_dw):
             scratch = self._scratch_size(True)
-            if need_dx and scratch > self.ws_bwd:
+            if scratch > self.ws_bwd:
                 ws = self._scratch_tensor(scratch, dev, stream)
             elif need_dw:
                 ws = self.workspace(self.ws_bwd, dev)

@@ -1,7 +1,7 @@
 """Build libfbcorr.so in-tree with nvcc for sm_103a.
 
 Steps: embed the NVRTC kernel templates (rtcg_direct.cuh, rtcg_ptx.cuh,
-rtcg_tc.cuh, rtcg_f32tc.cuh, rtcg_nn.cuh and their parameter headers) as strings, compile
+rtcg_tc.cuh, rtcg_f32tc.cuh, rtcg_f32dw.cuh, rtcg_nn.cuh and their parameter headers) as strings, compile
 every csrc/*.cu translation unit in parallel, link one shared library that
 statically links the CUDA runtime and dynamically links NVRTC.  Usage:
 ``python -m paper_0911_3456_gb300.build`` or ``build()`` from Python.
@@ -42,6 +42,7 @@ def _embed():
     for fname, var in (("rtcg_direct.cuh", "kRtcgDirectSrc"), ("tc_params.h", "kRtcgTcParamsSrc"),
                        ("rtcg_ptx.cuh", "kRtcgPtxSrc"), ("rtcg_tc.cuh", "kRtcgTcSrc"),
                        ("f32tc_params.h", "kRtcgF32tcParamsSrc"), ("rtcg_f32tc.cuh", "kRtcgF32tcSrc"),
+                       ("f32dw_params.h", "kRtcgF32dwParamsSrc"), ("rtcg_f32dw.cuh", "kRtcgF32dwSrc"),
                        ("nn_params.h", "kRtcgNnParamsSrc"), ("rtcg_nn.cuh", "kRtcgNnSrc")):
         text = open(os.path.join(CSRC, fname)).read()
         assert ')FBCSRC"' not in text

@@ -32,6 +32,8 @@ struct DwArgsK {
     int H, W, Ho, Wo, N;
     int rows_per_chunk;
     float lo, hi;
+    const int* flags;
+    int nflags;
 };
 
 const int64_t kMaxElems = (int64_t)1 << 31;
@@ -194,8 +196,20 @@ std::string dx_spec(const fbcorr_plan* p) {
     return heuristic_spec(dx_problem(p), p->dev);
 }
 
-// Where the dL/dx scratch begins in a backward workspace: after the dL/dw partial sums.
+// The forward problem with the mask of dL/dw.
+DirectProblem dw_problem(const fbcorr_plan* p) {
+    DirectProblem pr = fwd_problem(p);
+    pr.epi = 0;
+    pr.mask = p->epi.kind == FBCORR_EPI_CLAMP ? 1 : 0;
+    return pr;
+}
+
+// A backward workspace with scratch: the FMA kernel's dL/dw partial sums, the dL/dx
+// scratch, the tensor-core kernel's dL/dw partial sums.
 size_t dx_scratch_offset(const fbcorr_plan* p) { return (p->ws_bwd + 255) / 256 * 256; }
+size_t dw_scratch_offset(const fbcorr_plan* p) {
+    return (dx_scratch_offset(p) + (p->dx_kind == VarKind::F32tc ? p->dx_f3.ws_bytes : 0) + 255) / 256 * 256;
+}
 
 fbcorr_status_t prepare_backward(fbcorr_plan* p) {
     if (p->bwd_ready) return FBCORR_OK;
@@ -258,6 +272,11 @@ fbcorr_status_t prepare_backward(fbcorr_plan* p) {
         }
         if (s == FBCORR_OK) {
             p->dw_kind = VarKind::Direct;
+            F3DwTile dt;
+            F3DwLaunch dl;
+            p->dw_f3 = F3DwLaunch{};
+            if (f3dw_wins(dw_problem(p), p->dev.sm_count, &dt) && f3dw_build(dw_problem(p), dt, &dl) == FBCORR_OK)
+                p->dw_f3 = dl;
             if (kernel_resources(p->dw_kernel, &regs, &local) == FBCORR_OK) p->dw_regs = regs;
             int resident = 0;
             if (kernel_occupancy(p->dw_kernel, &resident) == FBCORR_OK && resident > 0)
@@ -584,6 +603,7 @@ fbcorr_status_t fbcorr_plan_scratch_size(fbcorr_plan_t p, size_t* fwd, size_t* b
         if (p->epi.kind != FBCORR_EPI_SNIPPET) {
             FBC_TRY(prepare_backward(p));
             if (p->dx_kind == VarKind::F32tc) *bwd = dx_scratch_offset(p) + p->dx_f3.ws_bytes;
+            if (p->dw_f3.parts) *bwd = dw_scratch_offset(p) + p->dw_f3.ws_bytes;
         }
     }
     return FBCORR_OK;
@@ -663,9 +683,16 @@ fbcorr_status_t fbcorr_backward(fbcorr_plan_t p, const float* x, const float* w,
     }
     if (dw) {
         float* part = (float*)ws;
+        // with scratch: the tensor-core kernel; the FMA kernel behind it then runs only
+        // for inputs that it flags (non-finite or tiny values)
+        const float* part3 = nullptr;
+        const int* flags = nullptr;
+        if (p->dw_f3.parts && ws_bytes >= dw_scratch_offset(p) + p->dw_f3.ws_bytes)
+            FBC_TRY(f3dw_run(p->dw_f3, dw_problem(p), x, g, m ? m : g, (uint8_t*)ws + dw_scratch_offset(p), p->epi.lo,
+                             p->epi.hi, p->err_dev, &part3, &flags, sw));
         if (p->dw_kind == VarKind::Direct) {
             DwArgsK a{x, g, m ? m : g, part, (int)p->H, (int)p->W, (int)p->Ho, (int)p->Wo, (int)p->N,
-                      p->dw_rows_per_chunk, p->epi.lo, p->epi.hi};
+                      p->dw_rows_per_chunk, p->epi.lo, p->epi.hi, flags, p->dw_f3.grid};
             void* args[] = {&a};
             dim3 grid((unsigned)p->dw_chunks, (unsigned)p->fh, (unsigned)p->dw_nblocks);
             FBC_TRY(launch(p->dw_kernel, grid, args, sw));
@@ -675,7 +702,9 @@ fbcorr_status_t fbcorr_backward(fbcorr_plan_t p, const float* x, const float* w,
                                        p->dw_chunks, p->dw_rows_per_chunk, clamp ? 1 : 0, p->epi.lo,
                                        p->epi.hi, sw));
         }
-        FBC_CUDA(launch_dw_reduce(part, dw, p->dw_chunks, (long long)p->N * p->fh * p->fw * p->D, sw));
+        const long long elems = (long long)p->N * p->fh * p->fw * p->D;
+        FBC_CUDA(part3 ? launch_dw_reduce(part3, dw, p->dw_f3.parts, elems, sw, flags, p->dw_f3.grid, part, p->dw_chunks)
+                       : launch_dw_reduce(part, dw, p->dw_chunks, elems, sw));
     }
     if (fork) FBC_CUDA(cudaEventRecord(p->bwd_join, sw));
     fbcorr_status_t st = FBCORR_OK;
@@ -904,7 +933,11 @@ fbcorr_status_t fbcorr_plan_info(fbcorr_plan_t p, char* buf, size_t cap) {
           << ",\"filters_per_cta\":" << p->dw_tn * p->dw_ng << ",\"packed_pairs\":" << p->dw_pk << ",\"min_blocks\":" << p->dw_mb
           << ",\"registers\":" << p->dw_regs << ",\"tile\":[" << p->dw_tn << "," << p->dw_ng << "," << p->dw_qb << "]"
           << ",\"chunks\":" << p->dw_chunks
-          << ",\"rows_per_chunk\":" << p->dw_rows_per_chunk << "}";
+          << ",\"rows_per_chunk\":" << p->dw_rows_per_chunk;
+        if (p->dw_f3.parts)
+            o << ",\"f32tc\":{\"kernel\":\"" << p->dw_f3.kernel.name << "\",\"grid\":" << p->dw_f3.grid
+              << ",\"splits\":" << p->dw_f3.tile.splits << "}";
+        o << "}";
     }
     o << ",\"ws_fwd\":" << p->ws_fwd << ",\"ws_bwd\":" << p->ws_bwd << ",\"sm_count\":"
       << p->dev.sm_count << "}";

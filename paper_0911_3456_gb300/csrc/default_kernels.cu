@@ -133,11 +133,20 @@ constexpr int kMaxChunks = 256;   // the plan keeps the chunk count at or below 
 // the groups.  No dynamically indexed register arrays.
 __global__ void __launch_bounds__(kRedElems * kRedSlices) fbc_dw_reduce(const float* __restrict__ part,
                                                                         float* __restrict__ dw, int S,
-                                                                        long long E) {
+                                                                        long long E, const int* flags, int nflags,
+                                                                        const float* part2, int S2) {
     extern __shared__ float gsum[];   // [ceil(S / 8)][kRedElems]
     // launched as the programmatic dependent of the partial-sum kernel: wait for
     // that grid to complete and its partials to be visible before reading them
     asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (flags) {
+        int any = 0;
+        for (int k = threadIdx.x; k < nflags; k += blockDim.x) any |= flags[k];
+        if (__syncthreads_or(any)) {
+            part = part2;
+            S = S2;
+        }
+    }
     const int el = threadIdx.x % kRedElems;
     const int slice = threadIdx.x / kRedElems;
     const long long e = (long long)blockIdx.x * kRedElems + el;
@@ -178,9 +187,10 @@ cudaError_t launch_default_dw(const float* x, const float* g, const float* m, fl
     return cudaGetLastError();
 }
 
-cudaError_t launch_dw_reduce(const float* part, float* dw, int S, long long E, cudaStream_t s) {
-    if (S < 1 || S > kMaxChunks) return cudaErrorInvalidValue;
-    const size_t smem = (size_t)((S + 7) / 8) * kRedElems * sizeof(float);
+cudaError_t launch_dw_reduce(const float* part, float* dw, int S, long long E, cudaStream_t s, const int* flags,
+                             int nflags, const float* part2, int S2) {
+    if (S < 1 || S > kMaxChunks || S2 > kMaxChunks) return cudaErrorInvalidValue;
+    const size_t smem = (size_t)((std::max(S, S2) + 7) / 8) * kRedElems * sizeof(float);
     // programmatic dependent launch: the reduction's launch and CTA set-up overlap
     // the tail of the partial-sum kernel (which triggers it once its sums are done)
     cudaLaunchConfig_t cfg = {};
@@ -193,7 +203,7 @@ cudaError_t launch_dw_reduce(const float* part, float* dw, int S, long long E, c
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, fbc_dw_reduce, part, dw, S, E);
+    return cudaLaunchKernelEx(&cfg, fbc_dw_reduce, part, dw, S, E, flags, nflags, part2, S2);
 }
 
 }  // namespace fbc

@@ -94,6 +94,8 @@ const char* rtcg_ptx_source();        // contents of rtcg_ptx.cuh
 const char* rtcg_tc_source();         // contents of rtcg_tc.cuh
 const char* rtcg_f32tc_params_source();   // contents of f32tc_params.h
 const char* rtcg_f32tc_source();      // contents of rtcg_f32tc.cuh
+const char* rtcg_f32dw_params_source();   // contents of f32dw_params.h
+const char* rtcg_f32dw_source();      // contents of rtcg_f32dw.cuh
 const char* rtcg_nn_params_source();  // contents of nn_params.h
 const char* rtcg_nn_source();         // contents of rtcg_nn.cuh
 
@@ -197,7 +199,10 @@ cudaError_t launch_default_dw(const float* x, const float* g, const float* m, fl
                               int H, int W, int C, int Ho, int Wo, int N, int fh, int fw,
                               int chunks, int rows_per_chunk, int mask, float lo, float hi,
                               cudaStream_t s);
-cudaError_t launch_dw_reduce(const float* part, float* dw, int S, long long E, cudaStream_t s);
+// Sums S partials per element; with flags, S of `part` where all `nflags` flags are
+// zero, else S2 of `part2`.
+cudaError_t launch_dw_reduce(const float* part, float* dw, int S, long long E, cudaStream_t s,
+                             const int* flags = nullptr, int nflags = 0, const float* part2 = nullptr, int S2 = 0);
 
 // Fill p[0..n) with values in [-scale, scale) from an integer hash (timing runs only).
 cudaError_t launch_fill_pattern(float* p, size_t n, float scale, unsigned seed, cudaStream_t s);
@@ -262,6 +267,26 @@ dim3 f3_bank_grid(const F3Launch& l);
 fbcorr_status_t f3_run(const F3Launch& l, const DirectProblem& pr, const float* x, const float* m, const float* w,
                        float* y, void* ws, float lo, float hi, int* err_word, cudaStream_t s);
 
+// dL/dw by the same split (f32dw_kernel.cu); the problem is the forward's, with the mask of dL/dw.
+struct F3DwTile {
+    int nb = 64, ncomb = 1, jt = 1, kpx = 96, splits = 1;
+};
+struct F3DwLaunch {
+    F3DwTile tile;
+    Kernel kernel;
+    int grid = 0;
+    int parts = 0;             // partial sums per element
+    size_t ws_bytes = 0;       // partial sums and the CTAs' flags
+};
+bool f3dw_wins(const DirectProblem& pr, int sm_count, F3DwTile* t);
+size_t f3dw_ws_bytes(const DirectProblem& pr, const F3DwTile& t);
+fbcorr_status_t f3dw_build(const DirectProblem& pr, const F3DwTile& t, F3DwLaunch* out);
+// *part: l.parts partial sums per element; *flags: l.grid flags, any set where the
+// result has to come from the FMA kernel.
+fbcorr_status_t f3dw_run(const F3DwLaunch& l, const DirectProblem& pr, const float* x, const float* g, const float* m,
+                         void* ws, float lo, float hi, int* err_word, const float** part, const int** flags,
+                         cudaStream_t s);
+
 }  // namespace fbc
 struct FbcF3Params;   // f32tc_params.h
 namespace fbc {
@@ -302,6 +327,7 @@ struct fbcorr_plan {
     fbc::DirectTile dx_tile;
     fbc::Kernel dx_kernel;
     fbc::F3Launch dx_f3;
+    fbc::F3DwLaunch dw_f3;         // parts = 0: dL/dw always runs the FMA kernel
     fbc::VarKind dw_kind = fbc::VarKind::Direct;
     fbc::Kernel dw_kernel;
     int dw_tn = 4, dw_ng = 1, dw_qb = 64, dw_nblocks = 1;

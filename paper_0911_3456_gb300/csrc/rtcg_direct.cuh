@@ -761,7 +761,17 @@ struct FbcDwArgs {
     int H, W, Ho, Wo, N;
     int rows_per_chunk;
     float lo, hi;
+    const int* flags;              // not null: run only where one of the nflags flags is set
+    int nflags;
 };
+
+// Launched behind the tensor-core dL/dw kernel, for the inputs it leaves to FMAs.
+__device__ __forceinline__ bool fbc_dw_not_needed(const FbcDwArgs& a) {
+    if (!a.flags) return false;
+    int any = 0;
+    for (int k = threadIdx.x; k < a.nflags; k += blockDim.x) any |= a.flags[k];
+    return !__syncthreads_or(any);
+}
 
 // 16-byte asynchronous copy global -> shared (cp.async, L2 only); bytes = 0
 // fills the destination with zeros and reads nothing.

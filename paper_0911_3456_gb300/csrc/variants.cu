@@ -24,6 +24,8 @@ const char* rtcg_ptx_source() { return kRtcgPtxSrc; }
 const char* rtcg_tc_source() { return kRtcgTcSrc; }
 const char* rtcg_f32tc_params_source() { return kRtcgF32tcParamsSrc; }
 const char* rtcg_f32tc_source() { return kRtcgF32tcSrc; }
+const char* rtcg_f32dw_params_source() { return kRtcgF32dwParamsSrc; }
+const char* rtcg_f32dw_source() { return kRtcgF32dwSrc; }
 const char* rtcg_nn_params_source() { return kRtcgNnParamsSrc; }
 const char* rtcg_nn_source() { return kRtcgNnSrc; }
 
@@ -200,6 +202,7 @@ std::string dw_kernel_source(int fh, int fw, int c, int tn, int ng, int qb, int 
     o << ") " << kname
       << "(FbcDwArgs a) {\n"
       << "  extern __shared__ __align__(16) float fbc_smem[];\n"
+      << "  if (fbc_dw_not_needed(a)) return;\n"
       << "  FbcDwThis::run(a, fbc_smem, blockIdx.x, blockIdx.y, blockIdx.z);\n"
       << "}\n";
     return o.str();

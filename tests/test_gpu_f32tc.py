@@ -81,6 +81,60 @@ def test_dx_against_oracle(shape, spec, clamp, monkeypatch):
     _within(host(dx), ref, mag, shape[3] * shape[4] * shape[5])
 
 
+# one and several filter tiles, 32- and 64-row blocks, one and two planes of x per CTA
+# with a half-empty and an empty last plane, odd and even filter widths, two tap
+# groups, ragged last chunks, images smaller than a chunk, a single column
+DW_SHAPES = [(30, 41, 16, 64, 7, 7), (19, 26, 12, 40, 5, 3), (24, 31, 4, 8, 3, 4), (17, 40, 24, 132, 2, 5),
+             (40, 33, 8, 20, 9, 9), (25, 29, 32, 68, 4, 13), (21, 60, 4, 36, 2, 19), (9, 11, 20, 4, 3, 1),
+             (5, 1, 8, 64, 2, 1)]
+
+
+@pytest.mark.parametrize("clamp", [None, (-0.5, 0.5)])
+@pytest.mark.parametrize("shape", DW_SHAPES)
+def test_dw_against_oracle_and_integers(shape, clamp, monkeypatch):
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    monkeypatch.setenv("FBCORR_F32TC", "force")
+    for kind in ("real", "int"):
+        wl = inputs.random_case(7700, *shape, kind=kind, with_g=True)
+        p = Plan(wl.x.shape, wl.w.shape, "f32", clamp)
+        y = oracle.fwd(wl.x, wl.w, epilogue=clamp).astype(np.float32)
+        args = (dev(wl.x, torch), dev(wl.w, torch), dev(wl.g, torch), dev(y, torch))
+        dw = p.backward(*args, need_dx=False)[1]
+        assert "f32tc" in p.info()["dw"] and p.device_status() == 0
+        assert torch.equal(dw, p.backward(*args)[1])          # with dL/dx beside it, run to run
+        ref = oracle.bwd_filt(wl.x, wl.g, wl.w.shape, y=y.astype(np.float64), epilogue=clamp)
+        if kind == "int":
+            assert np.array_equal(host(dw), ref)
+        else:
+            mag = oracle.bwd_filt(np.abs(wl.x), np.abs(wl.g), wl.w.shape)
+            _within(host(dw), ref, mag, shape[0] * shape[1] // 96 + 64)
+
+
+@pytest.mark.parametrize("what", ["inf", "nan", "tiny_g", "tiny_x"])
+def test_dw_values_outside_the_split(what, monkeypatch):
+    """They come from the FMA kernel, as a plan without the tensor-core kernel computes them."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    wl = inputs.random_case(7800, 30, 41, 16, 64, 5, 5, with_g=True)
+    x, g = wl.x.copy(), wl.g.copy()
+    if what == "inf":
+        x[7, 40, 3] = np.inf            # a column that the last output columns alone read
+    elif what == "nan":
+        g[3, 4, 5] = np.nan
+    elif what == "tiny_g":
+        g *= np.float32(1e-34)
+    else:
+        x[2, 3, 4] = 1e-33
+    out = []
+    for sw in ("force", "0"):
+        monkeypatch.setenv("FBCORR_F32TC", sw)
+        p = Plan(x.shape, wl.w.shape)
+        out.append(p.backward(dev(x, torch), dev(wl.w, torch), dev(g, torch), need_dx=False)[1].cpu().numpy())
+        assert ("f32tc" in p.info()["dw"]) == (sw == "force")
+    assert np.array_equal(out[0], out[1], equal_nan=True)
+
+
 def _special(shape):
     """Inputs the BF16 split cannot carry: non-finite, at the range's ends, denormal."""
     wl = inputs.random_case(7300, *shape)
