@@ -21,6 +21,9 @@ Clamp = Optional[Tuple[float, float]]
 
 
 def _check_tensor(t: torch.Tensor, name: str, shape=None) -> None:
+    if (isinstance(t, torch.Tensor) and t.is_cuda and t.dtype is torch.float32 and t.is_contiguous()
+            and (shape is None or t.shape == shape)):
+        return
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name} must be a torch.Tensor")
     if not t.is_cuda:
@@ -42,13 +45,20 @@ def _check_host_tensor(t: torch.Tensor, name: str, shape) -> None:
         raise ValueError(f"{name} has shape {tuple(t.shape)}, expected {tuple(shape)}")
 
 
-def _vp(t: Optional[torch.Tensor]) -> ctypes.c_void_p:
-    return ctypes.c_void_p(t.data_ptr() if t is not None else 0)
+def _vp(t: Optional[torch.Tensor]) -> Optional[int]:
+    return t.data_ptr() if t is not None else None
 
 
-def _stream_handle(stream: Optional[torch.cuda.Stream]) -> ctypes.c_void_p:
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+# what torch.cuda.current_stream().cuda_stream returns, without the stream object (2 us a call)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+
+
+def _stream_handle(stream: Optional[torch.cuda.Stream]) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 class Plan:
@@ -376,6 +386,7 @@ class FBCorr(torch.autograd.Function):
     def forward(ctx, x, w, dtype="f32", clamp=None):
         plan = get_plan(x.shape, w.shape, dtype, clamp, x.device)
         y = plan.forward(x.contiguous(), w.contiguous())
+        ctx.plan = plan if dtype == "f32" else None     # the gradients' plan is the FP32 one
         ctx.clamp = clamp
         ctx.save_for_backward(x, w, y)
         return y
@@ -383,7 +394,7 @@ class FBCorr(torch.autograd.Function):
     @staticmethod
     def backward(ctx, gy):
         x, w, y = ctx.saved_tensors
-        plan = get_plan(x.shape, w.shape, "f32", ctx.clamp, x.device)
+        plan = ctx.plan or get_plan(x.shape, w.shape, "f32", ctx.clamp, x.device)
         dx, dw = plan.backward(x.contiguous(), w.contiguous(), gy.contiguous(),
                                y if ctx.clamp is not None else None,
                                need_dx=ctx.needs_input_grad[0], need_dw=ctx.needs_input_grad[1])

@@ -674,8 +674,14 @@ fbcorr_status_t fbcorr_backward(fbcorr_plan_t p, const float* x, const float* w,
     const float* m = clamp ? y : nullptr;
     // both gradients: dL/dw on the side stream, forked after the work already on
     // `s` and joined back before anything queued on `s` after this call, so the two
-    // gradients' kernels fill each other's idle SMs
-    const bool fork = dx && dw && p->bwd_side;
+    // gradients' kernels fill each other's idle SMs.  Not when both run on the tensor
+    // cores: each fills every SM, and the fork costs the host four event calls
+    // (autograd step 256x256x16 * 64x7x7, bound by the host: 261 to 207 us together
+    // with the lighter Python calls)
+    const bool f3_dx = dx && p->dx_kind == VarKind::F32tc && ws && aligned16(ws) &&
+                       ws_bytes >= dx_scratch_offset(p) + p->dx_f3.ws_bytes;
+    const bool f3_dw = dw && p->dw_f3.parts && ws_bytes >= dw_scratch_offset(p) + p->dw_f3.ws_bytes;
+    const bool fork = dx && dw && p->bwd_side && !(f3_dx && f3_dw);
     cudaStream_t sw = fork ? p->bwd_side : s;
     if (fork) {
         FBC_CUDA(cudaEventRecord(p->bwd_fork, s));
@@ -687,7 +693,7 @@ fbcorr_status_t fbcorr_backward(fbcorr_plan_t p, const float* x, const float* w,
         // for inputs that it flags (non-finite or tiny values)
         const float* part3 = nullptr;
         const int* flags = nullptr;
-        if (p->dw_f3.parts && ws_bytes >= dw_scratch_offset(p) + p->dw_f3.ws_bytes)
+        if (f3_dw)
             FBC_TRY(f3dw_run(p->dw_f3, dw_problem(p), x, g, m ? m : g, (uint8_t*)ws + dw_scratch_offset(p), p->epi.lo,
                              p->epi.hi, p->err_dev, &part3, &flags, sw));
         if (p->dw_kind == VarKind::Direct) {
@@ -710,9 +716,8 @@ fbcorr_status_t fbcorr_backward(fbcorr_plan_t p, const float* x, const float* w,
     fbcorr_status_t st = FBCORR_OK;
     if (dx) {
         const DirectProblem pr = dx_problem(p);
-        const size_t off = dx_scratch_offset(p);
-        const bool f3 = p->dx_kind == VarKind::F32tc && ws && aligned16(ws) && ws_bytes >= off + p->dx_f3.ws_bytes;
-        st = f3 ? f3_run(p->dx_f3, pr, g, m, w, dx, (uint8_t*)ws + off, p->epi.lo, p->epi.hi, p->err_dev, s)
+        st = f3_dx ? f3_run(p->dx_f3, pr, g, m, w, dx, (uint8_t*)ws + dx_scratch_offset(p), p->epi.lo, p->epi.hi,
+                            p->err_dev, s)
              : p->dx_kind != VarKind::Default
                  ? run_direct(p->dx_kernel, pr, p->dx_tile, g, m, w, dx, p->epi.lo, p->epi.hi, s)
                  : run_default(pr, g, m, w, dx, p->epi.lo, p->epi.hi, s);

@@ -162,8 +162,8 @@ std::vector<F3Tile> f3_ranked(const DirectProblem& pr, int sm_count, double* bes
 }
 
 // The line between the two FP32 kernels: the model's cycles and the bank split's
-// launch (about 9000 cycles, 5 us) against the FMA kernels at the 0.65 of their
-// peak that they reach at size.  Measured (us, FMA kernel / this one): 128x128x8 *
+// launch (about 9000 cycles, 5 us) against the FMA kernels at 0.55 of their peak (the
+// forward; 0.65 at size, in a batch) or 0.35 (dL/dx of the untuned tiles).  Measured (us, FMA kernel / this one): 128x128x8 *
 // 16x9x9 (0.3 GFLOP) 11 / 19, 187x233x12 * 40x5x3 (0.6) 20 / 20, 256x256x8 *
 // 64x9x9 (5.1) 115 / 35, 2048x2048x4 * 4x8x8 (8.5) 180 / 100, 512x512x32 *
 // 256x5x5 (106) 1937 / 394.
@@ -176,7 +176,8 @@ bool f3_wins(const DirectProblem& pr, int sm_count, F3Tile* t, bool shared) {
     if (r.empty()) return false;
     *t = r.front();
     const double flops = 2.0 * pr.out_h * pr.out_w * pr.nf * pr.fh * pr.fw * pr.c;
-    return sw == "force" || cycles + (shared ? 0 : 9000) < 0.9 * (flops / (sm_count * 256 * 0.65) + (shared ? 0 : 4000));
+    const double eff = shared ? 0.65 : pr.flip ? 0.35 : 0.55;
+    return sw == "force" || cycles + (shared ? 0 : 9000) < 0.9 * (flops / (sm_count * 256 * eff) + (shared ? 0 : 4000));
 }
 
 size_t f3_ws_bytes(const DirectProblem& pr, const F3Tile& t) {
