@@ -102,6 +102,42 @@ std::string heuristic_spec(const DirectProblem& pr, const DeviceInfo& dev) {
     return direct_tile_spec(direct_heuristic(pr, smem_limit(dev), dev.sm_count));
 }
 
+// BF16 modes: the packed kernel with tile t instead of the plan's own tensor-core kernel.
+int plan_orders(const fbcorr_plan* p) { return p->dtype == FBCORR_F32 ? 3 : p->dtype == FBCORR_BF16X3 ? 2 : 1; }
+
+fbcorr_status_t set_packed(fbcorr_plan* p, const F3Tile& t, const char* source) {
+    const DirectProblem pr = fwd_problem(p);
+    if (f3_ws_bytes(pr, t) > p->ws_fwd)
+        return set_error(FBCORR_ERR_UNSUPPORTED, "variant %s needs more workspace than the plan's", f3_spec(t).c_str());
+    F3Launch l;
+    FBC_TRY(f3_build(pr, t, p->dev.sm_count, &l));
+    p->fwd_f3 = l;
+    p->tc_packed = true;
+    p->fwd_source = source;
+    return FBCORR_OK;
+}
+
+// Select the forward variant of a BF16 or split-BF16 plan from a spec string.
+fbcorr_status_t set_tc_spec(fbcorr_plan* p, const std::string& spec, const char* source) {
+    F3Tile t;
+    if (f3_parse_spec(spec, &t, plan_orders(p))) return set_packed(p, t, source);
+    FBC_TRY(tc_set_spec(p->tc, spec));
+    p->tc_packed = false;
+    p->fwd_source = source;
+    return FBCORR_OK;
+}
+
+// The variant of an untuned BF16 or split-BF16 plan, whose tc is at its default.
+fbcorr_status_t set_tc_heuristic(fbcorr_plan* p) {
+    p->tc_packed = false;
+    p->fwd_source = "heuristic";
+    F3Tile t;
+    if (f3_wins_bf16(fwd_problem(p), p->dev.sm_count, plan_orders(p), p->ws_fwd, &t) &&
+        set_packed(p, t, "heuristic") != FBCORR_OK)
+        logf("packed tensor-core kernel not usable (%s)", last_error_message());
+    return FBCORR_OK;
+}
+
 // Select the forward variant of an F32 plan from a spec string.
 fbcorr_status_t set_fwd_spec(fbcorr_plan* p, const std::string& spec, const char* source) {
     if (spec == "default" && !p->snippet.empty())
@@ -439,15 +475,12 @@ fbcorr_status_t plan_create(fbcorr_plan_t* out, const int64_t in_shape[3], const
                                p->epi.kind == FBCORR_EPI_CLAMP ? 1 : 0, p->epi.lo, p->epi.hi, p->snippet, dev);
             if (s == FBCORR_OK) {
                 p->ws_fwd = tc_workspace_bytes(p->tc);
-                p->fwd_source = "heuristic";
                 std::string spec = env_str("FBCORR_VARIANT", "");
-                if (!spec.empty() && tc_set_spec(p->tc, spec) == FBCORR_OK) {
-                    p->fwd_source = "env";
-                } else if (tune_lookup(tune_key(p->dev, shape_key(p, "fwd")), &spec) &&
-                           tc_set_spec(p->tc, spec) == FBCORR_OK) {
-                    p->fwd_source = "cache";
-                }
-                clear_error();
+                if ((spec.empty() || set_tc_spec(p, spec, "env") != FBCORR_OK) &&
+                    (!tune_lookup(tune_key(p->dev, shape_key(p, "fwd")), &spec) ||
+                     set_tc_spec(p, spec, "cache") != FBCORR_OK))
+                    s = set_tc_heuristic(p);
+                if (s == FBCORR_OK) clear_error();
             }
         }
     }
@@ -646,6 +679,12 @@ fbcorr_status_t fbcorr_forward(fbcorr_plan_t p, const float* x, const float* w, 
             if (e1 && st == FBCORR_OK) FBC_CUDA(cudaEventRecord(e1, s));
             return st;
         case VarKind::Tensor:
+            if (p->tc_packed) {
+                if (e0) FBC_CUDA(cudaEventRecord(e0, s));
+                st = f3_run(p->fwd_f3, fwd_problem(p), x, nullptr, w, y, ws, p->epi.lo, p->epi.hi, p->err_dev, s);
+                if (e1 && st == FBCORR_OK) FBC_CUDA(cudaEventRecord(e1, s));
+                return st;
+            }
             return tc_forward(p->tc, x, w, y, ws, p->err_dev, s, e0, e1);
     }
     return set_error(FBCORR_ERR_INTERNAL, "bad variant kind");
@@ -733,13 +772,9 @@ fbcorr_status_t fbcorr_plan_set_variant(fbcorr_plan_t p, const char* spec) {
     const std::string s = spec;
     if (p->dtype != FBCORR_F32) {
         if (s == "tuned") return fbcorr_autotune(p, nullptr);
-        if (s == "heuristic") {
-            FBC_TRY(tc_set_spec(p->tc, tc_candidates(p->tc).front()));
-        } else {
-            FBC_TRY(tc_set_spec(p->tc, s));
-        }
-        p->fwd_source = s == "heuristic" ? "heuristic" : "forced";
-        return FBCORR_OK;
+        if (s != "heuristic") return set_tc_spec(p, s, "forced");
+        FBC_TRY(tc_set_spec(p->tc, tc_candidates(p->tc).front()));
+        return set_tc_heuristic(p);
     }
     if (s == "heuristic") return set_fwd_spec(p, heuristic_spec(fwd_problem(p), p->dev), "heuristic");
     if (s == "tuned") return fbcorr_autotune(p, nullptr);
@@ -818,6 +853,7 @@ static fbcorr_status_t autotune_tc(fbcorr_plan_t p, fbcorr_stream_t stream) {
     cudaStream_t s = (cudaStream_t)stream;
     const std::vector<std::string> specs = tc_candidates(p->tc);
     const std::string old = tc_spec(p->tc);
+    p->tc_packed = false;   // the candidates below are the plan's own kernel
     float *x = nullptr, *w = nullptr, *y = nullptr;
     void* ws = nullptr;
     const size_t xb = (size_t)p->H * p->W * p->D * 4, wb = (size_t)p->N * p->fh * p->fw * p->D * 4,
@@ -900,8 +936,14 @@ static fbcorr_status_t autotune_tc(fbcorr_plan_t p, fbcorr_stream_t stream) {
         tc_set_spec(p->tc, old);
         return status != FBCORR_OK ? status : set_error(FBCORR_ERR_INTERNAL, "no variant ran");
     }
-    FBC_TRY(tc_set_spec(p->tc, best));
-    p->fwd_source = "tuned";
+    FBC_TRY(set_tc_spec(p, best, "tuned"));
+    float packed_ms = 0.f;
+    std::string packed;
+    FBC_TRY(f3_tune(p->dev, fwd_problem(p), s, p->err_dev, &packed_ms, &packed, plan_orders(p), p->ws_fwd));
+    if (!packed.empty() && packed_ms < best_ms && set_tc_spec(p, packed, "tuned") == FBCORR_OK) {
+        best = packed;
+        best_ms = packed_ms;
+    }
     tune_store(tune_key(p->dev, shape_key(p, "fwd")), best);
     logf("autotune picked %s (%.4f ms)", best.c_str(), best_ms);
     return FBCORR_OK;
@@ -926,6 +968,12 @@ fbcorr_status_t fbcorr_plan_info(fbcorr_plan_t p, char* buf, size_t cap) {
           << hex64(p->fwd_f3.kernel.src_hash) << "\"";
     } else if (p->fwd_kind == VarKind::Default) {
         o << ",\"spec\":\"default\"";
+    } else if (p->tc_packed) {
+        o << ",\"spec\":\"" << f3_spec(p->fwd_f3.tile) << "\",\"detail\":{\"precision\":\""
+          << (p->dtype == FBCORR_BF16X3 ? "bf16x3" : "bf16") << "\",\"filter_tiles\":" << p->fwd_f3.filter_tiles
+          << ",\"tail_half_tiles\":0,\"smem\":" << p->fwd_f3.kernel.smem << ",\"grid\":" << p->fwd_f3.grid
+          << ",\"threads\":" << p->fwd_f3.kernel.threads << ",\"kernel\":\"" << p->fwd_f3.kernel.name
+          << "\",\"source_hash\":\"" << hex64(p->fwd_f3.kernel.src_hash) << "\"}";
     } else if (p->tc) {
         o << ",\"spec\":\"" << tc_spec(p->tc) << "\",\"detail\":" << tc_describe(p->tc);
     }

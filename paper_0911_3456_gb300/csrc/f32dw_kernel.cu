@@ -96,7 +96,12 @@ bool f3dw_wins(const DirectProblem& pr, int sm_count, F3DwTile* out) {
     if (best < 0) return false;
     *out = t;
     const double flops = 2.0 * pr.out_h * pr.out_w * pr.nf * pr.fh * pr.fw * pr.c;
-    return sw == "force" || best + 5000 < 0.9 * (flops / (sm_count * 256 * 0.45) + 4000);
+    // the FMA kernel's CTA has a thread per channel and 4 or 8 filters: a few threads
+    // where both are few (2048x2048x4 * 4x8x8: four, 0.04 of the peak)
+    const int tn = pr.c <= 64 && !pr.mask ? 8 : 4;
+    const int threads = pr.c * std::max(1, std::min((tn == 8 ? 128 : 256) / pr.c, (pr.nf + tn - 1) / tn));
+    const double eff = 0.45 * std::min(1.0, threads / 64.0);
+    return sw == "force" || best + 5000 < 0.9 * (flops / (sm_count * 256 * eff) + 4000);
 }
 
 fbcorr_status_t f3dw_build(const DirectProblem& pr, const F3DwTile& t, F3DwLaunch* out) {

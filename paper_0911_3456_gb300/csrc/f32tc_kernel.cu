@@ -3,6 +3,7 @@
 // per call (the split of the bank, and the correlation as its programmatic
 // dependent); the forward and dL/dx are both DirectProblems.
 #include <algorithm>
+#include <cmath>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -38,9 +39,9 @@ Geometry geometry(const DirectProblem& pr, const F3Tile& t) {
     g.nu = (g.rows + t.ru - 1) / t.ru * g.ncg * g.ntg;
     g.ls = pack ? 128 + (2 * g.s - 1) * g.pp : 128 + t.jt - 1;
     const int lp = g.pl == 4 ? (g.ls + 5) / 8 * 8 + 2 : g.pl == 2 ? (g.ls + 3) / 8 * 8 + 4 : g.ls;
-    g.aslot = ((size_t)t.ru * 3 * g.pl * lp * 16 + 127) / 128 * 128;
-    g.bstage = (size_t)(t.nt >= 48 ? 2 : t.nt >= 32 ? 4 : 8) * 96 * t.nt;
-    g.bunit = (size_t)t.ru * g.s * 96 * t.nt;
+    g.aslot = ((size_t)t.ru * t.ord * g.pl * lp * 16 + 127) / 128 * 128;
+    g.bstage = (size_t)(t.ord * t.nt >= 144 ? 2 : t.ord * t.nt >= 96 ? 4 : 8) * 32 * t.ord * t.nt;
+    g.bunit = (size_t)t.ru * g.s * 32 * t.ord * t.nt;
     const bool va = pr.c % 4 == 0;
     const int items = t.ru * (va && g.pp == 2 ? g.ls + 1 : g.ls) * (!va ? g.pl : g.pp == 2 ? 1 : t.gc / 4);
     g.ka = (items + 32 * FBC_F3_CONV_WARPS - 1) / (32 * FBC_F3_CONV_WARPS);
@@ -60,7 +61,7 @@ long long pixel_tiles(const DirectProblem& pr, const F3Tile& t) {
 // Ring depths: three to six A slots, and two B rings of the stages that then fit, up
 // to 8 each (at least 3: a copy takes about 1 us).
 bool layout(const DirectProblem& pr, const F3Tile& t, int* na, int* nb, size_t* smem) {
-    if (t.nt < 16 || t.nt > 80 || t.nt % 16 || t.r < 1 || t.ru < 1 || t.jt < 1 || t.jt > pr.fw)
+    if (t.ord < 1 || t.ord > 3 || t.nt < 16 || t.nt > (t.ord == 3 ? 80 : 96) || t.nt % 16 || t.r < 1 || t.ru < 1 || t.jt < 1 || t.jt > pr.fw)
         return false;
     if (t.gc != 8 && t.gc != 16 && t.gc != 32) return false;
     if (t.gc > 8 && pr.c <= 4) return false;
@@ -85,14 +86,20 @@ bool layout(const DirectProblem& pr, const F3Tile& t, int* na, int* nb, size_t* 
 // Cycles of a launch, to rank tiles.  A K = 16 step takes 3 NT cycles of the tensor
 // core, or longer at narrow tiles (measured alone: 123, 144, 168, 204, 244 cycles
 // at NT = 16 .. 80); a unit measured 600 to 900 cycles more (barriers, commits, the
-// drain that is not hidden).
+// drain that is not hidden).  The converters take about 250 cycles for each pass
+// over their threads, and the latency of a load where a unit's values leave no
+// registers for the next one's.
 // shared: the launch runs beside others that fill the SMs its last round leaves idle.
 double model_cycles(const DirectProblem& pr, const F3Tile& t, int sm_count, bool shared) {
     const Geometry g = geometry(pr, t);
-    const double step = std::max(102.0 + 1.2 * t.nt, 3.06 * t.nt);
+    // (an MMA of N columns alone: the longer of N / 2 and 32 + N / 4 cycles)
+    auto mma_cycles = [](int n) { return std::max(n / 2.0, 32 + n / 4.0); };
+    const double step = t.ord == 3   ? std::max(102.0 + 1.2 * t.nt, 3.06 * t.nt)
+                        : t.ord == 2 ? mma_cycles(2 * t.nt) + mma_cycles(t.nt)
+                                     : mma_cycles(t.nt);
     const long long items = pixel_tiles(pr, t) * filter_tiles(pr, t);
     const double rounds = shared ? (double)items / sm_count : (double)((items + sm_count - 1) / sm_count);
-    const double mma = t.ru * g.s * step + 700, conv = 90.0 * g.ka + 300, drain = 400.0 + 8 * t.nt;
+    const double mma = t.ru * g.s * step + 700, conv = 250.0 * g.ka + (g.ka > 9 ? 1400 : 300), drain = 400.0 + 8 * t.nt;
     return rounds * g.nu * std::max(std::max(mma, conv), drain) + 4000;
 }
 
@@ -105,28 +112,32 @@ constexpr int kChunkSteps = 16;
 
 std::string f3_spec(const F3Tile& t) {
     char b[96];
-    snprintf(b, sizeof b, "f32tc:nt=%d,r=%d,gc=%d,jt=%d,ru=%d", t.nt, t.r, t.gc, t.jt, t.ru);
+    snprintf(b, sizeof b, "%s:nt=%d,r=%d,gc=%d,jt=%d,ru=%d", t.ord == 3 ? "f32tc" : "tcpack", t.nt, t.r, t.gc, t.jt, t.ru);
     return b;
 }
 
-bool f3_parse_spec(const std::string& s, F3Tile* t) {
+bool f3_parse_spec(const std::string& s, F3Tile* t, int ord) {
     F3Tile v;
+    v.ord = ord;
     int used = 0;
-    if (sscanf(s.c_str(), "f32tc:nt=%d,r=%d,gc=%d,jt=%d,ru=%d%n", &v.nt, &v.r, &v.gc, &v.jt, &v.ru, &used) != 5 ||
+    if (sscanf(s.c_str(), ord == 3 ? "f32tc:nt=%d,r=%d,gc=%d,jt=%d,ru=%d%n" : "tcpack:nt=%d,r=%d,gc=%d,jt=%d,ru=%d%n", &v.nt, &v.r, &v.gc, &v.jt, &v.ru, &used) != 5 ||
         used != (int)s.size())
         return false;
     *t = v;
     return true;
 }
 
-std::vector<F3Tile> f3_ranked(const DirectProblem& pr, int sm_count, double* best_cycles, bool shared) {
+std::vector<F3Tile> f3_ranked(const DirectProblem& pr, int sm_count, double* best_cycles, bool shared, int ord) {
+    const int chunk_steps = ord == 3 ? kChunkSteps : 2 * kChunkSteps;   // the BF16 modes never added up in between
+    const int widest = ord == 3 ? 80 : 96;
     std::vector<std::pair<double, F3Tile>> all;
     const int npad = (pr.nf + 15) / 16 * 16;
     for (int fold = 1; fold <= std::min(16, pr.out_h); ++fold) {
-        if (fold > 1 && fold * pr.nf > 80) break;
+        if (fold > 1 && fold * pr.nf > widest) break;
         F3Tile t;
+        t.ord = ord;
         t.r = fold;
-        const int ntn = (npad + 79) / 80;
+        const int ntn = (npad + widest - 1) / widest;
         t.nt = fold > 1 ? (fold * pr.nf + 15) / 16 * 16 : ((npad + ntn - 1) / ntn + 15) / 16 * 16;
         for (int gc : {32, 16, 8}) {   // no whole group of padding
             if (gc > 8 && (pr.c <= 4 || pr.c <= gc / 2)) continue;
@@ -137,12 +148,12 @@ std::vector<F3Tile> f3_ranked(const DirectProblem& pr, int sm_count, double* bes
                 jt = t.jt;
                 t.ru = 1;
                 const Geometry g = geometry(pr, t);
-                if (g.s > kChunkSteps) continue;
+                if (g.s > chunk_steps) continue;
                 // slab rows per unit, evenly, within the chunk length and half of it
-                for (int steps : {kChunkSteps, kChunkSteps / 2}) {
+                for (int steps : {chunk_steps, chunk_steps / 2}) {
                     const int most = std::max(1, std::min(g.rows, steps / g.s)), units = (g.rows + most - 1) / most;
                     const int ru = (g.rows + units - 1) / units;
-                    if (steps != kChunkSteps && ru == t.ru) break;
+                    if (steps != chunk_steps && ru == t.ru) break;
                     t.ru = ru;
                     int na, nb;
                     size_t smem;
@@ -180,6 +191,28 @@ bool f3_wins(const DirectProblem& pr, int sm_count, F3Tile* t, bool shared) {
     return sw == "force" || cycles + (shared ? 0 : 9000) < 0.9 * (flops / (sm_count * 256 * eff) + (shared ? 0 : 4000));
 }
 
+// The BF16 modes' own kernel (rtcg_tc.cuh) measured 1.35 of its MMAs' time and about
+// 1400 cycles per filter row and 128-pixel tile: far from the tensor rate where the
+// rows are short (narrow banks, shallow or ragged depths, which it pads to 16).
+// Measured untuned (GB300, us, that kernel / this one, split BF16): 244x244x32 *
+// 16x3x3 21 / 10, 256x256x8 * 64x9x9 60 / 26, 248x248x64 * 32x5x5 62 / 33, 300x500x32
+// * 64x7x7 124 / 77, 512x512x4 * 32x13x13 361 / 38, 2048x2048x4 * 4x8x8 2287 / 74; at
+// 128 filters 46 / 47 (200x300x32 * 128x5x5), at 256 theirs.
+bool f3_wins_bf16(const DirectProblem& pr, int sm_count, int ord, size_t ws_limit, F3Tile* t) {
+    if (env_str("FBCORR_TCPACK", "1") == "0" || fault_injected("tcdrop")) return false;
+    double cycles = 0;
+    const std::vector<F3Tile> r = f3_ranked(pr, sm_count, &cycles, false, ord);
+    if (r.empty() || f3_ws_bytes(pr, r.front()) > ws_limit) return false;
+    *t = r.front();
+    const int npad = (pr.nf + 15) / 16 * 16, ntn = (npad + 255) / 256, nt = ((npad + ntn - 1) / ntn + 15) / 16 * 16;
+    const double tiles = ((double)pr.out_h * pr.in_w / 128 + 1) * ntn;
+    const double rounds = std::max(1.0, tiles > 4 * sm_count ? tiles / sm_count : std::ceil(tiles / sm_count));
+    const double mma = (double)pr.fw * ((pr.c + 15) / 16) * (ord == 2 ? 3 : 1) * std::max(nt / 2.0, 32 + nt / 4.0);
+    const double tc = rounds * pr.fh * (1.35 * mma + 1400) + 4000;
+    // plain BF16, bound by the converters here: 301x419x24 * 96x7x5 54 / 53
+    return cycles + 2000 < (ord == 1 ? 0.75 : 0.85) * tc;
+}
+
 size_t f3_ws_bytes(const DirectProblem& pr, const F3Tile& t) {
     int na, nb;
     size_t smem;
@@ -191,7 +224,7 @@ size_t f3_ws_bytes(const DirectProblem& pr, const F3Tile& t) {
 
 std::string f3_kernel_name(const DirectProblem& pr, const F3Tile& t) {
     char b[160];
-    snprintf(b, sizeof b, "fbc_f32tc_f%dx%d_c%d_n%d_fl%d_e%d_m%d_t%d_%d_%d_%d_%d", pr.fh, pr.fw, pr.c, pr.nf, pr.flip,
+    snprintf(b, sizeof b, "%s_f%dx%d_c%d_n%d_fl%d_e%d_m%d_t%d_%d_%d_%d_%d", t.ord == 3 ? "fbc_f32tc" : t.ord == 2 ? "fbc_tcpack2" : "fbc_tcpack1", pr.fh, pr.fw, pr.c, pr.nf, pr.flip,
              pr.epi, pr.mask, t.nt, t.r, t.gc, t.jt, t.ru);
     const std::string name = b;
     return pr.epi == 2 ? name + "_u" + snippet_tag(pr.snippet) : name;
@@ -206,7 +239,7 @@ std::string f3_kernel_source(const DirectProblem& pr, const F3Tile& t, const std
     const Geometry g = geometry(pr, t);
     o << "typedef FbcF3Cfg<" << pr.fh << "," << pr.fw << "," << pr.c << "," << pr.nf << "," << pr.flip << "," << pr.epi
       << "," << pr.mask << "," << t.nt << "," << t.r << "," << t.gc << "," << t.jt << "," << t.ru
-      << "> FbcF3;\nstatic_assert(FbcF3::ASLOT == " << g.aslot << " && FbcF3::BSTAGE == " << g.bstage
+      << "," << t.ord << "> FbcF3;\nstatic_assert(FbcF3::ASLOT == " << g.aslot << " && FbcF3::BSTAGE == " << g.bstage
       << " && FbcF3::NU == " << g.nu << ", \"host and device disagree on the geometry\");\n";
     o << "extern \"C\" __global__ void __launch_bounds__(" << FBC_F3_THREADS << ", 1) " << name
       << "(const __grid_constant__ FbcF3Params P) {\n"
@@ -278,10 +311,12 @@ fbcorr_status_t f3_run(const F3Launch& l, const DirectProblem& pr, const float* 
 }
 
 fbcorr_status_t f3_tune(const DeviceInfo& dev, const DirectProblem& pr, cudaStream_t s, int* err_word, float* ms,
-                        std::string* spec) {
+                        std::string* spec, int ord, size_t ws_limit) {
     spec->clear();
-    std::vector<F3Tile> tiles = f3_ranked(pr, dev.sm_count, nullptr, false);
-    if (env_str("FBCORR_F32TC", "1") == "0" || tiles.empty()) return FBCORR_OK;
+    std::vector<F3Tile> tiles = f3_ranked(pr, dev.sm_count, nullptr, false, ord);
+    tiles.erase(std::remove_if(tiles.begin(), tiles.end(), [&](const F3Tile& t) { return f3_ws_bytes(pr, t) > ws_limit; }),
+                tiles.end());
+    if (env_str(ord == 3 ? "FBCORR_F32TC" : "FBCORR_TCPACK", "1") == "0" || tiles.empty()) return FBCORR_OK;
     tiles.resize(std::min<size_t>(tiles.size(), 8));
     std::vector<std::string> srcs;
     for (const F3Tile& t : tiles) srcs.push_back(f3_kernel_source(pr, t, f3_kernel_name(pr, t)));

@@ -242,6 +242,7 @@ struct F3Tile {
     int gc = 16;   // channels per unit: 8 (packed), 16 or 32
     int jt = 1;    // filter taps per unit
     int ru = 1;    // slab rows per unit (a unit is one accumulation chunk)
+    int ord = 3;   // orders of the split: 3 FP32, 2 split BF16, 1 BF16
 };
 struct F3Launch {
     F3Tile tile;
@@ -251,14 +252,17 @@ struct F3Launch {
     size_t ws_bytes = 0;       // scratch of one call: the split bank and its flags
 };
 std::string f3_spec(const F3Tile& t);
-bool f3_parse_spec(const std::string& s, F3Tile* t);
+bool f3_parse_spec(const std::string& s, F3Tile* t, int ord = 3);
 // Every tile the kernel takes the problem with (none: it does not), by the cost model, best first.
-std::vector<F3Tile> f3_ranked(const DirectProblem& pr, int sm_count, double* best_cycles, bool shared = false);
+std::vector<F3Tile> f3_ranked(const DirectProblem& pr, int sm_count, double* best_cycles, bool shared = false,
+                              int ord = 3);
 // Time the model's first tiles on patterned buffers; *spec is empty when there are none.
 fbcorr_status_t f3_tune(const DeviceInfo& dev, const DirectProblem& pr, cudaStream_t s, int* err_word, float* ms,
-                        std::string* spec);
+                        std::string* spec, int ord = 3, size_t ws_limit = ~(size_t)0);
 // The best rated tile, and whether the model expects it to be faster than the FP32 FMA kernels.
 bool f3_wins(const DirectProblem& pr, int sm_count, F3Tile* t, bool shared = false);
+// The same against the tensor-core kernel of the BF16 modes, within ws_limit bytes of workspace.
+bool f3_wins_bf16(const DirectProblem& pr, int sm_count, int ord, size_t ws_limit, F3Tile* t);
 size_t f3_ws_bytes(const DirectProblem& pr, const F3Tile& t);
 std::string f3_kernel_source(const DirectProblem& pr, const F3Tile& t, const std::string& name);   // + name "_bank"
 std::string f3_kernel_name(const DirectProblem& pr, const F3Tile& t);
@@ -319,6 +323,7 @@ struct fbcorr_plan {
     std::string fwd_source;        // "heuristic", "tuned", "cache", "env", "forced"
     fbc::TcPlan* tc = nullptr;
     fbc::F3Launch fwd_f3;
+    bool tc_packed = false;        // BF16 modes: fwd_f3 runs instead of tc
     std::string snippet;           // user epilogue expression (epi.kind == FBCORR_EPI_SNIPPET)
 
     // backward (F32 always)

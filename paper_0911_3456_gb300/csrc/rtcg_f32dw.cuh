@@ -163,7 +163,7 @@ __device__ __forceinline__ void fbc_f32dw_body(const FbcF3DwParams& P) {
             for (int k = 0; k < G::KG; ++k) {
                 const int it = ct + k * G::NCT;
                 const int px = it / G::QG, q = it % G::QG;
-                if (px < G::KPX)
+                if ((k + 1) * G::NCT <= G::KPX * G::QG || px < G::KPX)
                     fbc_f3_put(gb[k], gd + (fbc_u32)(q >> 1) * G::GPLANE + (fbc_u32)px * 16u + (fbc_u32)(q & 1) * 8u,
                                (G::NB / 8) * G::GPLANE, tiny);
             }
@@ -171,7 +171,7 @@ __device__ __forceinline__ void fbc_f32dw_body(const FbcF3DwParams& P) {
             for (int k = 0; k < G::KX; ++k) {
                 const int it = ct + k * G::NCT;
                 const int px = it / G::QX, q = it % G::QX;
-                if (px < G::LS)
+                if ((k + 1) * G::NCT <= G::LS * G::QX || px < G::LS)
                     fbc_f3_put(xb[k], xd + (fbc_u32)(q >> 1) * G::XPLANE + (fbc_u32)px * 16u + (fbc_u32)(q & 1) * 8u, G::XORD,
                                tiny);
             }

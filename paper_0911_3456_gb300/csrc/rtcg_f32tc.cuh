@@ -14,6 +14,10 @@
 // sums are added to FP32 registers with ordinary rounding.  Measured error
 // against 64 bits: at or below that of the FP32 FMA kernels it stands in for.
 //
+// ORD is the number of orders: 3 for FP32.  The BF16 modes run the same kernel with
+// fewer where their own one (rtcg_tc.cuh) is far from the tensor rate: ORD = 2 is
+// split BF16 (x1 w1, x1 w2 + x2 w1), ORD = 1 plain BF16.
+//
 // Layout.  As in the BF16 kernels, an A tile is 128 consecutive pixels of the
 // image laid out with the virtual row width vw = out_w + FW - 1 (columns past
 // out_w are computed and dropped), and one slab of pixels serves every filter
@@ -75,10 +79,10 @@ __device__ __forceinline__ void fbc_umma_lo(fbc_u32 d, fbc_u32 alo, fbc_u32 ahi,
 __device__ float fbc_user_epi(float y, int n, float lo, float hi);
 
 template <int FH_, int FW_, int C_, int NF_, int FLIP_, int EPI_, int MASK_, int NT_, int R_, int GC_,
-          int JT_, int RU_>
+          int JT_, int RU_, int ORD_ = 3>
 struct FbcF3Cfg {
     static constexpr int FH = FH_, FW = FW_, C = C_, NF = NF_, FLIP = FLIP_, EPI = EPI_, MASK = MASK_;
-    static constexpr int NT = NT_, R = R_, GC = GC_, JT = JT_, RU = RU_;
+    static constexpr int NT = NT_, R = R_, GC = GC_, JT = JT_, RU = RU_, ORD = ORD_;
     static constexpr bool PACK = GC == 8;
     static constexpr int PP = !PACK ? 1 : C <= 1 ? 8 : C <= 2 ? 4 : C <= 4 ? 2 : 1;   // pixels per chunk
     static constexpr int CP = 8 / PP;                                                // channels per pixel in it
@@ -94,14 +98,14 @@ struct FbcF3Cfg {
     static constexpr int LP = PL == 4 ? (LS + 5) / 8 * 8 + 2 : PL == 2 ? (LS + 3) / 8 * 8 + 4 : LS;
     static constexpr unsigned PLANE = LP * 16;
     static constexpr unsigned AORD = PL * PLANE;                                     // bytes of one order of a slab
-    static constexpr unsigned SLAB = 3 * AORD;
+    static constexpr unsigned SLAB = ORD * AORD;
     static constexpr unsigned ASLOT = (RU * SLAB + 127) / 128 * 128;
-    static constexpr unsigned BCH = 3 * NT * 16;             // bytes per chunk of B
+    static constexpr unsigned BCH = ORD * NT * 16;             // bytes per chunk of B
     static constexpr unsigned BSTEP = 2 * BCH;
     static constexpr int STEPS = RU * S;                     // steps of a unit
     // a B stage holds BS steps, about 12 KB (one copy at the copy unit's full rate):
     // refills start, and are waited for, in small pieces
-    static constexpr int BS = NT >= 48 ? 2 : NT >= 32 ? 4 : 8;
+    static constexpr int BS = ORD * NT >= 144 ? 2 : ORD * NT >= 96 ? 4 : 8;
     static constexpr int NST = (STEPS + BS - 1) / BS;        // stages of a unit
     static constexpr unsigned BSTAGE = BS * BSTEP;
     static constexpr unsigned BUNIT = STEPS * BSTEP;         // the unit's image in the split bank
@@ -120,7 +124,8 @@ struct FbcF3Cfg {
     __device__ static __forceinline__ int tap_group(int u) { return NTG > 1 ? u % NTG : 0; }
     __device__ static __forceinline__ int channel_group(int u) { return NCG > 1 ? (u / NTG) % NCG : 0; }
     __device__ static __forceinline__ int row0(int u) { return u / (NTG * NCG) * RU; }
-    static constexpr unsigned TMEM = 6 * NT <= 32 ? 32 : 6 * NT <= 64 ? 64 : 6 * NT <= 128 ? 128 : 6 * NT <= 256 ? 256 : 512;
+    static constexpr int TC = 2 * ORD * NT;                  // columns of the two accumulator sets
+    static constexpr unsigned TMEM = TC <= 32 ? 32 : TC <= 64 ? 64 : TC <= 128 ? 128 : TC <= 256 ? 256 : 512;
 };
 
 // v = h + m + l exactly (finite v in the BF16 range); tiny takes the least of
@@ -139,22 +144,24 @@ __device__ __forceinline__ void fbc_f3_split4(const float (&v)[4], fbc_u32 (&h)[
     fbc_f3_split2(v[2], v[3], h[1], m[1], l[1], tiny);
 }
 
-// The three orders of one chunk (8 values) to shared memory, `ord` bytes apart.
+// The first ORD orders of one chunk (8 values) to shared memory, `ord` bytes apart.
+template <int ORD = 3>
 __device__ __forceinline__ void fbc_f3_put(const float (&v)[8], fbc_u32 dst, fbc_u32 ord, fbc_u32& tiny) {
     fbc_u32 h[4], m[4], l[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) fbc_f3_split2(v[2 * k], v[2 * k + 1], h[k], m[k], l[k], tiny);
     fbc_st_shared_v4(dst, h[0], h[1], h[2], h[3]);
-    fbc_st_shared_v4(dst + ord, m[0], m[1], m[2], m[3]);
-    fbc_st_shared_v4(dst + 2 * ord, l[0], l[1], l[2], l[3]);
+    if (ORD > 1) fbc_st_shared_v4(dst + ord, m[0], m[1], m[2], m[3]);
+    if (ORD > 2) fbc_st_shared_v4(dst + 2 * ord, l[0], l[1], l[2], l[3]);
 }
 
+template <int ORD = 3>
 __device__ __forceinline__ void fbc_f3_put(const float (&v)[4], fbc_u32 dst, fbc_u32 ord, fbc_u32& tiny) {
     fbc_u32 h[2], m[2], l[2];
     fbc_f3_split4(v, h, m, l, tiny);
     fbc_st_shared_v2(dst, h[0], h[1]);
-    fbc_st_shared_v2(dst + ord, m[0], m[1]);
-    fbc_st_shared_v2(dst + 2 * ord, l[0], l[1]);
+    if (ORD > 1) fbc_st_shared_v2(dst + ord, m[0], m[1]);
+    if (ORD > 2) fbc_st_shared_v2(dst + 2 * ord, l[0], l[1]);
 }
 
 #define FBC_F3_TINY ((27u << 24) - 1u)   // 2 * bits(2^-100) - 1
@@ -212,7 +219,10 @@ __device__ __forceinline__ void fbc_f3_store8(const FbcF3Params& P, int pg, int 
     }
 }
 
-// Columns [c0, c1) of one pixel recomputed with FP32 FMAs from global memory.
+__device__ __forceinline__ float fbc_f3_bf16(float v) { return __uint_as_float(fbc_pack_bf16x2(v, 0.f) << 16); }
+
+// Columns [c0, c1) of one pixel recomputed with FP32 FMAs from global memory (the
+// BF16 modes: of the rounded values).
 template <class G>
 __device__ __noinline__ void fbc_f3_recompute(const FbcF3Params& P, int pg, int q, int n0, int c0, int c1) {
     for (int col0 = c0; col0 < c1; col0 += 8) {
@@ -239,7 +249,17 @@ __device__ __noinline__ void fbc_f3_recompute(const FbcF3Params& P, int pg, int 
                         const long long wo =
                             G::FLIP ? (((long long)c * G::FH + (G::FH - 1 - i)) * G::FW + (G::FW - 1 - j)) * G::NF + nn[k]
                                     : (((long long)nn[k] * G::FH + i) * G::FW + j) * G::C + c;
-                        acc[k] = fmaf(fbc_f3_masked<G>(__ldg(P.x + xo), P.m + xo, P), __ldg(P.w + wo), acc[k]);
+                        const float xv = fbc_f3_masked<G>(__ldg(P.x + xo), P.m + xo, P), wv = __ldg(P.w + wo);
+                        if constexpr (G::ORD == 3) {
+                            acc[k] = fmaf(xv, wv, acc[k]);
+                        } else {
+                            const float xh = fbc_f3_bf16(xv), wh = fbc_f3_bf16(wv);
+                            if constexpr (G::ORD == 2) {
+                                acc[k] = fmaf(xh, fbc_f3_bf16(wv - wh), acc[k]);
+                                acc[k] = fmaf(fbc_f3_bf16(xv - xh), wh, acc[k]);
+                            }
+                            acc[k] = fmaf(xh, wh, acc[k]);
+                        }
                     }
                 }
             }
@@ -250,16 +270,25 @@ __device__ __noinline__ void fbc_f3_recompute(const FbcF3Params& P, int pg, int 
 // Position in a CTA's sequence of (work item, unit); item = filter tile * mtiles + pixel tile.
 template <class G>
 struct FbcF3Pos {
-    int item, u;
-    __device__ __forceinline__ void start() {
-        item = blockIdx.x;
-        u = 0;
+    int item, u, mt, ft;       // mt, ft: the item's pixel and filter tile, kept without a division
+    __device__ __forceinline__ void wrap(const FbcF3Params& P) {
+        while (mt >= P.mtiles) {
+            mt -= P.mtiles;
+            ++ft;
+        }
+    }
+    __device__ __forceinline__ void start(const FbcF3Params& P) {
+        item = mt = blockIdx.x;
+        u = ft = 0;
+        wrap(P);
     }
     __device__ __forceinline__ bool valid(const FbcF3Params& P) const { return item < P.nitems; }
-    __device__ __forceinline__ void next() {
+    __device__ __forceinline__ void next(const FbcF3Params& P) {
         if (++u < G::NU) return;
         u = 0;
         item += gridDim.x;
+        mt += gridDim.x;
+        wrap(P);
     }
 };
 
@@ -279,12 +308,25 @@ __device__ __forceinline__ void fbc_f3_load_a(const FbcF3Params& P, const FbcF3P
     int k, px, sub;
     fbc_f3_a_item<G>(it, k, px, sub);
     const int ri = G::row0(j.u) + k;
-    const int vp = (j.item % P.mtiles) * 128 + G::tap_group(j.u) * G::JT + px;
+    const int vp = j.mt * 128 + G::tap_group(j.u) * G::JT + px;
+#pragma unroll
+    for (int e = 0; e < G::WA; ++e) v[e] = 0.f;
+    if constexpr (G::VA && G::R == 1 && !G::FLIP) {
+        // no border and one row per tile row: the slab is a run of x itself (past a row's
+        // end it reads the next row, for outputs that are dropped and taps that are zero)
+        const int pix = vp + ri * P.in_w;
+        const int ch = G::PP == 1 ? cg * G::GC + sub * 4 : 0;
+        if (it >= G::NIT || ri >= G::ROWS || pix >= P.in_h * P.in_w || ch >= G::C) return;
+        const float4 f = __ldg(reinterpret_cast<const float4*>(P.x + (unsigned)(pix * G::C + ch)));
+        v[0] = f.x;
+        v[1] = f.y;
+        v[2] = f.z;
+        v[3] = f.w;
+        return;
+    }
     const int pg = fbc_f3_row(vp, P);
     const int col = vp - pg * P.vw - P.pad_x;
     const int row = pg * G::R + ri - P.pad_y;
-#pragma unroll
-    for (int e = 0; e < G::WA; ++e) v[e] = 0.f;
     if (it >= G::NIT || ri >= G::ROWS || row < 0 || row >= P.in_h) return;
     if constexpr (G::VA) {
         const int ch = cg * G::GC + sub * 4;
@@ -314,31 +356,32 @@ __device__ __forceinline__ void fbc_f3_load_a(const FbcF3Params& P, const FbcF3P
     }
 }
 
-// Item `it` of a unit into the A slot at dst.
+// Item `it` of a unit into the A slot at dst; `all`: every thread has one in this pass
+// (no branch: the conversions of several passes interleave).
 template <class G>
-__device__ __forceinline__ void fbc_f3_put_a(int it, const float (&v)[G::WA], fbc_u32 dst, fbc_u32& tiny) {
-    if (it >= G::NIT) return;
+__device__ __forceinline__ void fbc_f3_put_a(int it, bool all, const float (&v)[G::WA], fbc_u32 dst, fbc_u32& tiny) {
+    if (!all && it >= G::NIT) return;
     int k, px, sub;
     fbc_f3_a_item<G>(it, k, px, sub);
     const fbc_u32 d = dst + (fbc_u32)k * G::SLAB + (fbc_u32)px * 16u;
     if constexpr (!G::VA) {
-        fbc_f3_put(v, d + (fbc_u32)sub * G::PLANE, G::AORD, tiny);
+        fbc_f3_put<G::ORD>(v, d + (fbc_u32)sub * G::PLANE, G::AORD, tiny);
     } else if constexpr (G::PP == 2) {
         // a pixel of 4 channels: first half of chunk px and second half of chunk px - 1
         fbc_u32 h[2], m[2], l[2];
         fbc_f3_split4(v, h, m, l, tiny);
         if (px < G::LS) {
             fbc_st_shared_v2(d, h[0], h[1]);
-            fbc_st_shared_v2(d + G::AORD, m[0], m[1]);
-            fbc_st_shared_v2(d + 2 * G::AORD, l[0], l[1]);
+            if (G::ORD > 1) fbc_st_shared_v2(d + G::AORD, m[0], m[1]);
+            if (G::ORD > 2) fbc_st_shared_v2(d + 2 * G::AORD, l[0], l[1]);
         }
         if (px > 0) {
             fbc_st_shared_v2(d - 8u, h[0], h[1]);
-            fbc_st_shared_v2(d - 8u + G::AORD, m[0], m[1]);
-            fbc_st_shared_v2(d - 8u + 2 * G::AORD, l[0], l[1]);
+            if (G::ORD > 1) fbc_st_shared_v2(d - 8u + G::AORD, m[0], m[1]);
+            if (G::ORD > 2) fbc_st_shared_v2(d - 8u + 2 * G::AORD, l[0], l[1]);
         }
     } else {
-        fbc_f3_put(v, d + (fbc_u32)(sub >> 1) * G::PLANE + (fbc_u32)(sub & 1) * 8u, G::AORD, tiny);
+        fbc_f3_put<G::ORD>(v, d + (fbc_u32)(sub >> 1) * G::PLANE + (fbc_u32)(sub & 1) * 8u, G::AORD, tiny);
     }
 }
 
@@ -379,10 +422,10 @@ __device__ __forceinline__ void fbc_f32tc_bank_body(const FbcF3Params& P) {
         for (int k = 0; k < 4; ++k) fbc_f3_split2(v[2 * k], v[2 * k + 1], h[k], m[k], l[k], tiny);
         unsigned char* dst = P.bank + ((long long)blockIdx.y * G::NU + u) * G::BUNIT + (it / G::NT) * G::BCH + col * 16;
         *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
-        *reinterpret_cast<uint4*>(dst + G::NT * 16) = make_uint4(m[0], m[1], m[2], m[3]);
-        *reinterpret_cast<uint4*>(dst + 2 * G::NT * 16) = make_uint4(l[0], l[1], l[2], l[3]);
+        if (G::ORD > 1) *reinterpret_cast<uint4*>(dst + G::NT * 16) = make_uint4(m[0], m[1], m[2], m[3]);
+        if (G::ORD > 2) *reinterpret_cast<uint4*>(dst + 2 * G::NT * 16) = make_uint4(l[0], l[1], l[2], l[3]);
     }
-    const int any = __syncthreads_or(tiny < FBC_F3_TINY);
+    const int any = __syncthreads_or(G::ORD == 3 && tiny < FBC_F3_TINY);
     if (threadIdx.x == 0) P.flags[blockIdx.y * P.bank_blocks + blockIdx.x] = any;
 }
 
@@ -440,14 +483,14 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
         // ------------------------------------------------------------ converters
         const int ct = threadIdx.x - 8 * 32;
         FbcF3Pos<G> ja, jn;      // unit being written, unit being loaded
-        ja.start();
+        ja.start(P);
         jn = ja;
         float abuf[G::PA][G::KA][G::WA];
         auto load_a = [&](float (&buf)[G::KA][G::WA]) {
             if (!jn.valid(P)) return;
 #pragma unroll
             for (int k = 0; k < G::KA; ++k) fbc_f3_load_a<G>(P, jn, ct + k * G::NCT, buf[k]);
-            jn.next();
+            jn.next(P);
         };
 #pragma unroll
         for (int s = 0; s < G::PA; ++s) load_a(abuf[s]);
@@ -466,14 +509,15 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
                 const fbc_u32 dst = sbase + (fbc_u32)as * G::ASLOT;
                 fbc_u32 tiny = 0xFFFFFFFFu;
 #pragma unroll
-                for (int k = 0; k < G::KA; ++k) fbc_f3_put_a<G>(ct + k * G::NCT, abuf[s][k], dst, tiny);
-                if (tiny < FBC_F3_TINY) *(volatile int*)&s_tiny[ord & 15] = ja.item + 1;
+                for (int k = 0; k < G::KA; ++k) 
+                    fbc_f3_put_a<G>(ct + k * G::NCT, (k + 1) * G::NCT <= G::NIT, abuf[s][k], dst, tiny);
+                if (G::ORD == 3 && tiny < FBC_F3_TINY) *(volatile int*)&s_tiny[ord & 15] = ja.item + 1;
                 fbc_fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) fbc_mbar_arrive(a_full0 + 8u * as);
                 if (++as == P.na) { as = 0; aph ^= 1; }
                 load_a(abuf[s]);
-                ja.next();
+                ja.next(P);
             }
         }
     } else if (warp == 13) {
@@ -487,8 +531,8 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
             } q[2];
 #pragma unroll
             for (int r = 0; r < 2; ++r) {
-                q[r].j.start();
-                if (r == 1) q[r].j.next();
+                q[r].j.start(P);
+                if (r == 1) q[r].j.next(P);
                 q[r].st = q[r].bs = 0;
                 q[r].ph = q[r].it = 0;
             }
@@ -507,14 +551,14 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
                     const fbc_u32 bytes = min(G::BSTAGE, G::BUNIT - off);
                     fbc_mbar_expect_tx(b_full0 + 8u * slot, bytes);
                     fbc_bulk_g2s(sbase + P.b_off + (fbc_u32)slot * G::BSTAGE,
-                                 P.bank + ((long long)(q[r].j.item / P.mtiles) * G::NU + q[r].j.u) * G::BUNIT + off, bytes,
+                                 P.bank + ((long long)q[r].j.ft * G::NU + q[r].j.u) * G::BUNIT + off, bytes,
                                  b_full0 + 8u * slot);
                     ++q[r].it;
                     if (++q[r].bs == P.nb) { q[r].bs = 0; q[r].ph ^= 1; }
                     if (++q[r].st == G::NST) {
                         q[r].st = 0;
-                        q[r].j.next();
-                        q[r].j.next();
+                        q[r].j.next(P);
+                        q[r].j.next(P);
                     }
                 }
                 if (moved) {
@@ -551,6 +595,7 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
             const fbc_u32 id3 = idesc0 | ((3u * G::NT >> 3) << 17);
             const fbc_u32 id2 = idesc0 | ((2u * G::NT >> 3) << 17);
             const fbc_u32 id1 = idesc0 | ((1u * G::NT >> 3) << 17);
+            const fbc_u32 idn[3] = {G::ORD == 3 ? id3 : G::ORD == 2 ? id2 : id1, G::ORD == 3 ? id2 : id1, id1};
             // descriptors: the start address (16-byte units) sits in the low bits of the
             // low word and never carries out of its field; the high word is constant
             const fbc_u64 adesc0 = fbc_smem_desc(sbase, G::PACK ? 16u * G::PP : G::PLANE, 128);
@@ -558,13 +603,13 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
             const fbc_u64 bdesc0 = fbc_smem_desc(sbase + P.b_off + ring * G::BSTAGE, G::BCH, 128);
             const fbc_u32 ahi = (fbc_u32)(adesc0 >> 32), bhi = (fbc_u32)(bdesc0 >> 32);
             const int acc = warp - 14;         // this thread's accumulator set
-            const fbc_u32 d = tmem + (fbc_u32)(acc * 3 * G::NT);
+            const fbc_u32 d = tmem + (fbc_u32)(acc * G::ORD * G::NT);
             int as = 0, bs = 0;
             fbc_u32 aph = 0, bph = 0, accph = 0;
             int turn = 0;
             bool ok = true, issued = false;
             FbcF3Pos<G> j;
-            for (j.start(); j.valid(P); j.next(), turn ^= 1) {
+            for (j.start(P); j.valid(P); j.next(P), turn ^= 1) {
                 if (turn == acc) {
                     if (!(ok = fbc_wait(acc_empty0 + 8u * acc, accph ^ 1, P, abort_flag, FBC_F3_ERR_WAIT))) break;
                     if (!(ok = fbc_wait(a_full0 + 8u * as, aph, P, abort_flag, FBC_F3_ERR_WAIT))) break;
@@ -584,9 +629,11 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
                             const fbc_u32 ao = k * G::SLAB + (G::PACK ? 2u * s * G::PP * 16u
                                                                       : (s % (G::GC / 16)) * 2u * G::PLANE + (s / (G::GC / 16)) * 16u);
                             const fbc_u32 a1 = alo + (ao >> 4), b = blo + (q * G::BSTEP >> 4);
-                            fbc_umma_lo(d, a1, ahi, b, bhi, id3, e > 0 ? 1u : 0u);
-                            fbc_umma_lo(d + G::NT, a1 + (G::AORD >> 4), ahi, b, bhi, id2, 1u);
-                            fbc_umma_lo(d + 2 * G::NT, a1 + (2 * G::AORD >> 4), ahi, b, bhi, id1, 1u);
+                            // order o of x with the first ORD - o of w
+                            fbc_umma_lo(d, a1, ahi, b, bhi, idn[0], e > 0 ? 1u : 0u);
+                            if constexpr (G::ORD > 1) fbc_umma_lo(d + G::NT, a1 + (G::AORD >> 4), ahi, b, bhi, idn[1], 1u);
+                            if constexpr (G::ORD > 2)
+                                fbc_umma_lo(d + 2 * G::NT, a1 + (2 * G::AORD >> 4), ahi, b, bhi, idn[2], 1u);
                         }
                         fbc_umma_commit<1>(b_empty0 + 8u * (ring + bs));
                         if (++bs == P.nb) { bs = 0; bph ^= 1; }
@@ -632,7 +679,7 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
         for (int item = blockIdx.x; item < P.nitems && ok; item += gridDim.x, ++ord) {
             const int mt = item % P.mtiles;
             const int n0 = G::R > 1 ? 0 : (item / P.mtiles) * G::NT;
-            if (item / P.mtiles != ftile) {
+            if (G::ORD == 3 && item / P.mtiles != ftile) {
                 ftile = item / P.mtiles;
                 int f = 0;
                 for (int b = lane; b < P.bank_blocks; b += 32) f |= P.flags[ftile * P.bank_blocks + b];
@@ -644,20 +691,24 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
             for (int u = 0; u < G::NU; ++u) {
                 if (!(ok = fbc_wait(acc_full0 + 8u * acc, accph, P, abort_flag, FBC_F3_ERR_WAIT))) break;
                 fbc_tc_fence_after();
-                const fbc_u32 ta = trow + (fbc_u32)(acc * 3 * G::NT);
+                const fbc_u32 ta = trow + (fbc_u32)(acc * G::ORD * G::NT);
 #pragma unroll
                 for (int k = 0; k < HC; k += 8) {
                     fbc_u32 r0[8], r1[8], r2[8];
                     fbc_tmem_ld32x32b_x8_async(ta + k, r0);
-                    fbc_tmem_ld32x32b_x8_async(ta + G::NT + k, r1);
-                    fbc_tmem_ld32x32b_x8_async(ta + 2 * G::NT + k, r2);
+                    if constexpr (G::ORD > 1) fbc_tmem_ld32x32b_x8_async(ta + G::NT + k, r1);
+                    if constexpr (G::ORD > 2) fbc_tmem_ld32x32b_x8_async(ta + 2 * G::NT + k, r2);
                     fbc_tmem_ld_wait();
                     fbc_reg_fence8(r0);
-                    fbc_reg_fence8(r1);
-                    fbc_reg_fence8(r2);
+                    if constexpr (G::ORD > 1) fbc_reg_fence8(r1);
+                    if constexpr (G::ORD > 2) fbc_reg_fence8(r2);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e)
-                        sum[k + e] += __uint_as_float(r0[e]) + (__uint_as_float(r1[e]) + __uint_as_float(r2[e]));
+                    for (int e = 0; e < 8; ++e) {
+                        float s = __uint_as_float(r0[e]);
+                        if constexpr (G::ORD == 2) s += __uint_as_float(r1[e]);
+                        if constexpr (G::ORD == 3) s += __uint_as_float(r1[e]) + __uint_as_float(r2[e]);
+                        sum[k + e] += s;
+                    }
                 }
                 fbc_tc_fence_before();
                 __syncwarp();
@@ -680,7 +731,7 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
                 z += sum[k] - sum[k];
                 out[k] = sum[k];
             }
-            const bool redo = tiny_bank || *(volatile int*)&s_tiny[ord & 15] == item + 1 ||
+            const bool redo = (G::ORD == 3 && (tiny_bank || *(volatile int*)&s_tiny[ord & 15] == item + 1)) ||
                               __any_sync(0xFFFFFFFFu, inside && !(z == 0.f));
             if (redo && inside) fbc_f3_recompute<G>(P, o_pg, o_q, n0, half * HC, half * HC + HC);
             o_next = inside && !redo ? 0 : NG;
