@@ -86,9 +86,11 @@ bool layout(const DirectProblem& pr, const F3Tile& t, int* na, int* nb, size_t* 
 // Cycles of a launch, to rank tiles.  A K = 16 step takes 3 NT cycles of the tensor
 // core, or longer at narrow tiles (measured alone: 123, 144, 168, 204, 244 cycles
 // at NT = 16 .. 80); a unit measured 600 to 900 cycles more (barriers, commits, the
-// drain that is not hidden).  The converters take about 250 cycles for each pass
-// over their threads, and the latency of a load where a unit's values leave no
-// registers for the next one's.
+// drain that is not hidden).  The converters take for each pass
+// over their threads about 170 cycles where a slab is a run of whole pixels, 290 where
+// it takes some channels of deeper ones, 250 where a pixel's row has to be divided out
+// (folded rows, dL/dx).  A finished tile's stores, 45 cycles a column (more where they
+// are narrower than 32 bytes), are spread over a tile's units.
 // shared: the launch runs beside others that fill the SMs its last round leaves idle.
 double model_cycles(const DirectProblem& pr, const F3Tile& t, int sm_count, bool shared) {
     const Geometry g = geometry(pr, t);
@@ -99,7 +101,9 @@ double model_cycles(const DirectProblem& pr, const F3Tile& t, int sm_count, bool
                                      : mma_cycles(t.nt);
     const long long items = pixel_tiles(pr, t) * filter_tiles(pr, t);
     const double rounds = shared ? (double)items / sm_count : (double)((items + sm_count - 1) / sm_count);
-    const double mma = t.ru * g.s * step + 700, conv = 250.0 * g.ka + (g.ka > 9 ? 1400 : 300), drain = 400.0 + 8 * t.nt;
+    const double pass = t.r > 1 || pr.flip ? 250 : t.gc < pr.c ? 290 : 170;
+    const double store = (pr.nf % 8 == 0 ? 45.0 : pr.nf % 4 == 0 ? 90.0 : 180.0) * t.nt / g.nu;
+    const double mma = t.ru * g.s * step + 700, conv = pass * g.ka + 300, drain = 400.0 + 8 * t.nt + store;
     return rounds * g.nu * std::max(std::max(mma, conv), drain) + 4000;
 }
 
@@ -195,9 +199,9 @@ bool f3_wins(const DirectProblem& pr, int sm_count, F3Tile* t, bool shared) {
 // 1400 cycles per filter row and 128-pixel tile: far from the tensor rate where the
 // rows are short (narrow banks, shallow or ragged depths, which it pads to 16).
 // Measured untuned (GB300, us, that kernel / this one, split BF16): 244x244x32 *
-// 16x3x3 21 / 10, 256x256x8 * 64x9x9 60 / 26, 248x248x64 * 32x5x5 62 / 33, 300x500x32
-// * 64x7x7 124 / 77, 512x512x4 * 32x13x13 361 / 38, 2048x2048x4 * 4x8x8 2287 / 74; at
-// 128 filters 46 / 47 (200x300x32 * 128x5x5), at 256 theirs.
+// 16x3x3 21 / 10, 400x400x16 * 128x3x3 33 / 37, 256x256x8 * 64x9x9 60 / 26, 248x248x64 * 32x5x5 62 / 33, 300x500x32
+// * 64x7x7 124 / 77, 512x512x4 * 32x13x13 361 / 38, 2048x2048x4 * 4x8x8 2287 / 74;
+// 200x300x32 * 128x5x5 40 / 44.
 bool f3_wins_bf16(const DirectProblem& pr, int sm_count, int ord, size_t ws_limit, F3Tile* t) {
     if (env_str("FBCORR_TCPACK", "1") == "0" || fault_injected("tcdrop")) return false;
     double cycles = 0;
@@ -209,8 +213,8 @@ bool f3_wins_bf16(const DirectProblem& pr, int sm_count, int ord, size_t ws_limi
     const double rounds = std::max(1.0, tiles > 4 * sm_count ? tiles / sm_count : std::ceil(tiles / sm_count));
     const double mma = (double)pr.fw * ((pr.c + 15) / 16) * (ord == 2 ? 3 : 1) * std::max(nt / 2.0, 32 + nt / 4.0);
     const double tc = rounds * pr.fh * (1.35 * mma + 1400) + 4000;
-    // plain BF16, bound by the converters here: 301x419x24 * 96x7x5 54 / 53
-    return cycles + 2000 < (ord == 1 ? 0.75 : 0.85) * tc;
+    // the margin keeps near ties on their own kernel: BF16 301x419x24 * 96x7x5 47 / 53
+    return cycles + 2000 < 0.75 * tc;
 }
 
 size_t f3_ws_bytes(const DirectProblem& pr, const F3Tile& t) {

@@ -515,6 +515,37 @@ std::vector<TcConfig> tc_candidate_configs(TcPlan* p, bool pairs) {
     return out;
 }
 
+// The configuration of an untuned plan, moved to the front of the candidates: the
+// one that, or a close neighbour of which, the tuner picks at size.  Register
+// conversion (fz = 1) by 8 warps and the most taps per stage; CTA pairs with tiled
+// stores where one 256-wide filter tile covers the bank and the tiles fill the SMs.
+// Measured untuned (GB300, us; the first candidate, raw-ring conversion of single
+// CTAs / this one): 512x512x32 * 256x5x5 split BF16 196 / 158, BF16 118 / 80;
+// 200x300x32 * 128x5x5 split BF16 49 / 41; 400x400x16 * 128x3x3 BF16 37 / 30;
+// 301x419x24 * 96x7x5 BF16 57 / 49; 300x400x16 * 200x5x5 split BF16 53 / 51.
+void default_first(const TcPlan* p, std::vector<TcConfig>* configs) {
+    int nt, ntn;
+    filter_tiles(p->N, 256, &nt, &ntn);
+    const long long mtiles = ((long long)(p->H - p->fh + 1) * p->W + kTileM - 1) / kTileM;
+    const bool pairs = ntn == 1 && nt == 256 && mtiles >= p->sm_count;
+    const int bt = std::min(p->fw, 5);
+    int best = -1, best_score = 0;
+    for (size_t i = 0; i < configs->size(); ++i) {
+        const TcConfig& c = (*configs)[i];
+        if (c.fuse != 1 || c.cw != 8 || c.bt != bt || c.rs || c.sw || c.ntmax != 256 || (c.cg == 2) != pairs) continue;
+        int score = 1;
+        if (pairs ? c.ts == 32 && c.ew == 4 : c.ts == 0 && c.ew == 8) score += 4;
+        if (pairs && c.ts == 0 && c.ew == 8) score += 2;
+        // three A slots where the B ring stays deep beside them
+        if (c.na == (p->split ? 2 : 3) && c.nb >= (p->split ? 2 : 4)) score += 1;
+        if (score > best_score) {
+            best_score = score;
+            best = (int)i;
+        }
+    }
+    if (best > 0) std::rotate(configs->begin(), configs->begin() + best, configs->begin() + best + 1);
+}
+
 // CTA-pair configurations among the tuning candidates (FBCORR_TC_PAIR=0 leaves
 // them out; a pair spec can still be set explicitly).
 bool pairs_offered() { return env_str("FBCORR_TC_PAIR", "1") != "0"; }
@@ -587,7 +618,9 @@ std::string tc_spec(const TcPlan* p) { return format_spec(p->cfg); }
 
 std::vector<std::string> tc_candidates(TcPlan* p) {
     std::vector<std::string> out;
-    for (const auto& c : tc_candidate_configs(p, pairs_offered())) out.push_back(format_spec(c));
+    std::vector<TcConfig> configs = tc_candidate_configs(p, pairs_offered());
+    default_first(p, &configs);
+    for (const auto& c : configs) out.push_back(format_spec(c));
     return out;
 }
 
@@ -639,9 +672,12 @@ fbcorr_status_t tc_plan_create(TcPlan** out, int H, int W, int D, int N, int fh,
         return set_error(FBCORR_ERR_UNSUPPORTED, "shape needs more shared memory than one SM has");
     }
     for (const auto& c : cands) p->ws_bytes = std::max(p->ws_bytes, tc_ws_need(p, c));
-    // default: the first candidate (widest filter tile, raw-ring conversion where
-    // possible, most taps per stage, two A slots, deepest B ring)
-    const fbcorr_status_t s = tc_set_spec(p, format_spec(cands.front()));
+    std::vector<TcConfig> offered = cands;
+    if (!pairs_offered())
+        offered.erase(std::remove_if(offered.begin(), offered.end(), [](const TcConfig& c) { return c.cg != 0; }),
+                      offered.end());
+    default_first(p, &offered);
+    const fbcorr_status_t s = tc_set_spec(p, format_spec(offered.front()));
     if (s != FBCORR_OK) {
         delete p;
         return s;
