@@ -128,7 +128,8 @@ class Plan:
 
     # -- optional scratch of the FP32 tensor-core kernels: from PyTorch's allocator on
     # the call's stream, call by call, so that FP32 calls of one plan may overlap on
-    # several streams and threads
+    # several streams and threads; None where the device has no memory left for it (the
+    # call then runs the FMA kernels, which need none)
     def _scratch_size(self, backward: bool) -> int:
         n = self._scratch.get(backward)
         if n is None:
@@ -139,11 +140,16 @@ class Plan:
         return n
 
     @staticmethod
-    def _scratch_tensor(nbytes: int, device, stream) -> torch.Tensor:
-        if stream is None:
-            return torch.empty(nbytes, dtype=torch.uint8, device=device)
-        with torch.cuda.stream(stream):
-            return torch.empty(nbytes, dtype=torch.uint8, device=device)
+    def _scratch_tensor(nbytes: int, device, stream) -> Optional[torch.Tensor]:
+        try:
+            if stream is None:
+                return torch.empty(nbytes, dtype=torch.uint8, device=device)
+            if not isinstance(stream, torch.cuda.Stream):
+                return None   # a bare handle: the allocator cannot follow its order
+            with torch.cuda.stream(stream):
+                return torch.empty(nbytes, dtype=torch.uint8, device=device)
+        except torch.cuda.OutOfMemoryError:
+            return None
 
     # -- calls
     def forward(self, x: torch.Tensor, w: torch.Tensor, y: Optional[torch.Tensor] = None,
@@ -194,7 +200,7 @@ class Plan:
             scratch = self._scratch_size(True)
             if scratch > self.ws_bwd:
                 ws = self._scratch_tensor(scratch, dev, stream)
-            elif need_dw:
+            if ws is None and need_dw:
                 ws = self.workspace(self.ws_bwd, dev)
         nbytes = ws.numel() * ws.element_size() if ws is not None else 0
         C.call("fbcorr_backward", self._h, _vp(x if need_dw else None), _vp(w if need_dx else None),

@@ -299,7 +299,12 @@ fbcorr_status_t build_f3(fbcorr_batch_plan* b) {
         auto work = [](const DirectProblem& p) { return (double)p.out_h * p.out_w * p.nf * p.fh * p.fw * p.c; };
         return work(a.pr) > work(c.pr);
     });
-    FBC_CUDA(cudaMalloc(&b->f3_ws, bytes));
+    if (cudaMalloc(&b->f3_ws, bytes) != cudaSuccess) {   // no memory: the persistent kernel takes every image
+        cudaGetLastError();
+        b->f3_ws = nullptr;
+        b->f3.clear();
+        return FBCORR_OK;
+    }
     FBC_CUDA(cudaHostAlloc((void**)&b->err_host, sizeof(int), cudaHostAllocMapped));
     FBC_CUDA(cudaHostGetDevicePointer((void**)&b->err_dev, b->err_host, 0));
     *b->err_host = 0;

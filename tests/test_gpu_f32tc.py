@@ -232,3 +232,31 @@ def test_streams_and_capture():
     g.replay()
     torch.cuda.synchronize()
     assert torch.equal(out, y2)
+
+
+def test_no_memory_for_the_scratch_runs_the_fma_kernels(monkeypatch):
+    """The scratch is optional: where the device has no memory for it, the calls give
+    what the FMA kernels give, bit for bit."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    wl = inputs.random_case(7190, 160, 170, 16, 64, 7, 7)
+    x, w = dev(wl.x, torch), dev(wl.w, torch)
+    p = Plan(wl.x.shape, wl.w.shape)
+    g = torch.rand(p.out_shape, device="cuda") - 0.5
+    assert p.info()["fwd"]["spec"].startswith("f32tc:") and p._scratch_size(True) > p.ws_bwd
+    small = torch.empty(16, dtype=torch.uint8, device="cuda")   # too small for any scratch
+    y0 = p.forward(x, w, ws=small)
+    dx0, dw0 = p.backward(x, w, g, ws=p.workspace(p.ws_bwd, x.device))
+    empty = torch.empty
+
+    def full(*size, dtype=None, **kw):
+        if dtype is torch.uint8 and size[0] != p.ws_bwd:
+            raise torch.cuda.OutOfMemoryError("no memory")
+        return empty(*size, dtype=dtype, **kw)
+
+    monkeypatch.setattr(torch, "empty", full)
+    y1 = p.forward(x, w)
+    dx1, dw1 = p.backward(x, w, g)
+    assert torch.equal(y0, y1) and torch.equal(dx0, dx1) and torch.equal(dw0, dw1)
+    dx2, none = p.backward(x, w, g, need_dw=False)
+    assert none is None and torch.equal(dx0, dx2)
