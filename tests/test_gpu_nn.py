@@ -229,3 +229,19 @@ def test_sampled_key_threshold_changes_no_answer(dtype):
             os.environ["FBCORR_NN_PRESCREEN"] = old
     assert np.array_equal(with_thr[0], without[0])
     assert np.array_equal(with_thr[1], without[1])
+
+
+@pytest.mark.parametrize("nt,nn,dim", [(129, 9000, 63), (70, 700, 37), (33, 300, 30), (5, 257, 13), (3, 40, 1)])
+def test_zero_dimensions_change_no_answer(nt, nn, dim):
+    """Rows of a multiple of four dimensions are read by 16-byte loads, others value by
+    value; the sums run in the same order, so with zeros appended up to the next
+    multiple of four the indices and distances are the same bits."""
+    torch = torch_cuda()
+    rng = np.random.default_rng(3500 + nt + nn + dim)
+    t = rng.standard_normal((nt, dim)).astype(np.float32)
+    n = rng.standard_normal((nn, dim)).astype(np.float32)
+    pad = ((0, 0), (0, -dim % 4))
+    idx, dist = _run(torch, t, n)
+    idx4, dist4 = _run(torch, np.pad(t, pad), np.pad(n, pad))
+    assert np.array_equal(idx, idx4) and np.array_equal(dist, dist4)
+    _check(t, n, idx, dist, 4 * 2.0 ** -16, 0.0)
