@@ -65,3 +65,24 @@ def test_packed_non_finite_values(mode):
     a, b = out
     assert np.array_equal(np.isnan(a), np.isnan(b)) and np.array_equal(np.isinf(a), np.isinf(b))
     assert np.array_equal(a[np.isinf(a)], b[np.isinf(b)])
+
+
+@pytest.mark.parametrize("mode", ["bf16", "bf16x3"])
+@pytest.mark.parametrize("shape", [
+    (140, 160, 16, 256, 2, 2),    # one 256-wide filter tile, more pixel tiles than SMs
+    (141, 157, 20, 256, 3, 6),    # the same, ragged: rows no multiple of 32 pixels, taps past a stage
+    (100, 160, 16, 256, 2, 2),    # fewer pixel tiles than SMs
+    (130, 133, 16, 257, 2, 3),    # two filter tiles
+    (20, 41, 33, 96, 3, 7),       # rows too deep for register conversion
+])
+def test_untuned_configuration_is_exact_on_integers(shape, mode, monkeypatch):
+    """An untuned plan starts from the first candidate; integer sums are exact in it."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    monkeypatch.setenv("FBCORR_TCPACK", "0")
+    wl = inputs.random_case(8300, *shape, kind="int")
+    p = Plan(wl.x.shape, wl.w.shape, mode)
+    assert p.info()["fwd"]["spec"] == p.candidates()[0]
+    y = host(p.forward(dev(wl.x, torch), dev(wl.w, torch)))
+    assert p.device_status() == 0
+    assert np.array_equal(y, oracle.fwd(wl.x, wl.w))
