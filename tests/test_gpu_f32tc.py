@@ -260,3 +260,27 @@ def test_no_memory_for_the_scratch_runs_the_fma_kernels(monkeypatch):
     assert torch.equal(y0, y1) and torch.equal(dx0, dx1) and torch.equal(dw0, dw1)
     dx2, none = p.backward(x, w, g, need_dw=False)
     assert none is None and torch.equal(dx0, dx2)
+
+
+@pytest.mark.parametrize("clamp", [None, (-20.0, 25.0)])
+@pytest.mark.parametrize("where", ["g", "w"])
+def test_dx_non_finite_values_against_oracle(where, clamp, monkeypatch):
+    """Infinities and NaN in the gradient or the filters reach the pixels of dL/dx that
+    read them, the border's (where a filter value meets no gradient) as elsewhere, and
+    the finite values are exact on integers."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    monkeypatch.setenv("FBCORR_DX_VARIANT", "f32tc:nt=32,r=1,gc=8,jt=3,ru=2")
+    wl = inputs.random_case(7195, 30, 41, 8, 24, 5, 3, kind="int", with_g=True)
+    p = Plan(wl.x.shape, wl.w.shape, "f32", clamp)
+    y = p.forward(dev(wl.x, torch), dev(wl.w, torch))
+    g, w = wl.g.copy(), wl.w.copy()
+    if where == "g":
+        g[0, 0, 0], g[12, 20, 7], g[25, 38, 23] = np.inf, np.nan, -np.inf
+    else:
+        w[3, 2, 1, 0], w[9, 0, 2, 5], w[20, 4, 0, 7] = np.inf, np.nan, -np.inf
+    dx = p.backward(dev(wl.x, torch), dev(w, torch), dev(g, torch), y=y, need_dw=False)[0].cpu().numpy()
+    assert p.info()["dx"]["spec"].startswith("f32tc") and p.device_status() == 0
+    with np.errstate(all="ignore"):
+        ref = oracle.bwd_input(g, w, wl.x.shape, y=host(y), epilogue=clamp)
+    assert np.array_equal(dx, ref, equal_nan=True)
