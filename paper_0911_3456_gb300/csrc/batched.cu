@@ -57,6 +57,7 @@ struct BatchF3 {
     F3Launch l;
     size_t ws_off = 0;
     cudaGraphNode_t bank_node = nullptr, node = nullptr;
+    bool bank_stale = false, stale = false;   // the node's parameters are older than the plan's pointer table
 };
 
 struct BatchVariant {
@@ -87,6 +88,7 @@ struct fbcorr_batch_plan {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaGraphNode_t knode = nullptr;      // of the persistent kernel (null: no image left for it)
+    bool knode_stale = false;             // its parameters are older than the pointer table
     std::vector<BatchF3> f3;
     unsigned char* f3_ws = nullptr;       // scratch of every tensor-core image
     int* err_host = nullptr;              // bounded-wait failure flag (host-mapped)
@@ -142,13 +144,6 @@ std::string batch_source(const fbcorr_batch_plan* b) {
       << "  }\n"
       << "}\n";
     return o.str();
-}
-
-void write_ptr_entry(std::vector<unsigned char>& args, int k, const void* x, const void* w, void* y) {
-    unsigned char* e = args.data() + kArgsHeader + (size_t)k * kPtrEntry;
-    memcpy(e, &x, 8);
-    memcpy(e + 8, &w, 8);
-    memcpy(e + 16, &y, 8);
 }
 
 void destroy(fbcorr_batch_plan* b) {
@@ -531,31 +526,40 @@ fbcorr_status_t fbcorr_forward_batched(fbcorr_batch_plan_t b, const float* const
         *(volatile int*)b->err_host = 0;
         return set_error(FBCORR_ERR_TIMEOUT, "a kernel of an earlier call gave up a bounded wait");
     }
-    std::vector<char> changed(b->n, 0);
-    bool any = false;
+    // every image is checked before anything is stored: a refused call leaves the plan as it was
     for (int k = 0; k < b->n; ++k) {
         if (!x[k] || !w[k] || !y[k]) return set_error(FBCORR_ERR_INVALID_ARG, "NULL pointer for image %d", k);
         if ((((uintptr_t)x[k]) | ((uintptr_t)w[k]) | ((uintptr_t)y[k])) & 15u)
             return set_error(FBCORR_ERR_ALIGNMENT, "image %d: tensors must be 16-byte aligned", k);
-        const unsigned char* e = b->args.data() + kArgsHeader + (size_t)k * kPtrEntry;
-        const void* old[3];
-        memcpy(old, e, 24);
-        if (old[0] != x[k] || old[1] != w[k] || old[2] != y[k]) {
-            write_ptr_entry(b->args, k, x[k], w[k], y[k]);
-            changed[k] = old[1] != w[k] ? 2 : 1;
-            any = any || b->var_of[k] >= 0;
-        }
     }
-    for (const BatchF3& f : b->f3) {
-        if (!changed[f.image]) continue;
+    // new pointers into the table; a node stays marked until the graph has taken its
+    // new parameters, so a failed update is made up for by the next call
+    auto entry = [b](int k) { return b->args.data() + kArgsHeader + (size_t)k * kPtrEntry; };
+    for (BatchF3& f : b->f3) {
+        const void* now[3] = {x[f.image], w[f.image], y[f.image]};
+        const bool moved = memcmp(entry(f.image), now, kPtrEntry) != 0;
+        f.bank_stale = f.bank_stale || memcmp(entry(f.image) + 8, &now[1], 8) != 0;
+        f.stale = f.stale || moved;
+    }
+    for (int k = 0; k < b->n; ++k) {
+        const void* now[3] = {x[k], w[k], y[k]};
+        if (memcmp(entry(k), now, kPtrEntry) == 0) continue;
+        memcpy(entry(k), now, kPtrEntry);
+        b->knode_stale = b->knode_stale || b->var_of[k] >= 0;
+    }
+    for (BatchF3& f : b->f3) {
+        if (!f.stale && !f.bank_stale) continue;
         FbcF3Params p = image_params(b, f);
         void* kargs[] = {&p};
-        if (changed[f.image] == 2) FBC_TRY(graph_set_kernel(b->exec, f.bank_node, f.l.bank, f3_bank_grid(f.l), kargs));
+        if (f.bank_stale) FBC_TRY(graph_set_kernel(b->exec, f.bank_node, f.l.bank, f3_bank_grid(f.l), kargs));
+        f.bank_stale = false;
         FBC_TRY(graph_set_kernel(b->exec, f.node, f.l.kernel, dim3(f.l.grid), kargs));
+        f.stale = false;
     }
-    if (any) {
+    if (b->knode_stale) {
         void* kargs[] = {b->args.data()};
         FBC_TRY(graph_set_kernel(b->exec, b->knode, b->kern, dim3(b->grid), kargs));
+        b->knode_stale = false;
     }
     FBC_CUDA(cudaGraphLaunch(b->exec, (cudaStream_t)stream));
     return FBCORR_OK;

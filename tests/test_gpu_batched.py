@@ -144,3 +144,32 @@ def test_batched_ksplit_variants(clamp, monkeypatch):
                 assert np.array_equal(host(y), ref), it.name
             else:
                 assert normwise_rel(host(y), ref) <= 1e-5, it.name
+
+
+@pytest.mark.parametrize("f32tc", ["force", "0"], ids=["tensor_cores", "persistent_kernel"])
+def test_batched_refused_call_leaves_the_plan_unharmed(f32tc, monkeypatch):
+    """A call refused for its last image changes nothing: a later call with the pointers
+    that the refused one had for the other images writes to them, not to older tensors."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300._capi import FbcorrError
+    from paper_0911_3456_gb300.api import BatchPlan
+    monkeypatch.setenv("FBCORR_F32TC", f32tc)
+    items = _batch(2500, SHAPES[:4], kind="int")
+    bp = BatchPlan([it.x.shape for it in items], [it.w.shape for it in items])
+    assert (bp.info()["tensor_images"] > 0) == (f32tc == "force")
+    xs, ws = [dev(it.x, torch) for it in items], [dev(it.w, torch) for it in items]
+    old = bp.forward(xs, ws)
+    torch.cuda.synchronize()
+    xs2, ws2 = [2 * x for x in xs], [3 * w for w in ws]
+    new = [torch.zeros_like(y) for y in old]
+    # the last image keeps its first tensors throughout, but for one x four bytes off
+    off = torch.empty(xs[-1].numel() + 4, device="cuda")[1:1 + xs[-1].numel()].view(xs[-1].shape)
+    with pytest.raises(FbcorrError):
+        bp.forward(xs2[:-1] + [off], ws2[:-1] + ws[-1:], new[:-1] + old[-1:])
+    old[-1].zero_()
+    bp.forward(xs2[:-1] + xs[-1:], ws2[:-1] + ws[-1:], new[:-1] + old[-1:])
+    torch.cuda.synchronize()
+    for it, a, b in zip(items[:-1], old, new):
+        ref = oracle.fwd(it.x, it.w)
+        assert np.array_equal(host(a), ref) and np.array_equal(host(b), 6 * ref)
+    assert np.array_equal(host(old[-1]), oracle.fwd(items[-1].x, items[-1].w))
