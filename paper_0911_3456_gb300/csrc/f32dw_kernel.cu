@@ -110,6 +110,7 @@ fbcorr_status_t f3dw_build(const DirectProblem& pr, const F3DwTile& t, F3DwLaunc
     snprintf(name, sizeof name, "fbc_f32dw_f%dx%d_c%d_n%d_m%d_t%d_%d_%d_%d", pr.fh, pr.fw, pr.c, pr.nf, pr.mask, t.nb, t.ncomb,
              t.jt, t.kpx);
     std::ostringstream o;
+    if (fault_injected("f3drop")) o << "#define FBC_F3_DROP 1\n";   // tests: the first chunk is never handed over
     o << rtcg_f32tc_params_source() << "\n" << rtcg_f32dw_params_source() << "\n" << rtcg_ptx_source() << "\n"
       << rtcg_f32tc_source() << "\n" << rtcg_f32dw_source() << "\n";
     o << "static_assert(sizeof(FbcF3DwParams) == " << sizeof(FbcF3DwParams)
@@ -125,6 +126,7 @@ fbcorr_status_t f3dw_build(const DirectProblem& pr, const F3DwTile& t, F3DwLaunc
     l.grid = (int)(combos(pr, t) * t.splits);
     l.parts = t.splits * g.nh;
     l.ws_bytes = f3dw_ws_bytes(pr, t);
+    l.wait_ns = wait_bound_ns();
     *out = l;
     return FBCORR_OK;
 }
@@ -139,9 +141,7 @@ fbcorr_status_t f3dw_run(const F3DwLaunch& l, const DirectProblem& pr, const flo
     const size_t part_bytes = (size_t)l.parts * pr.nf * pr.fh * pr.fw * pr.c * 4;
     k.flags = reinterpret_cast<int*>(static_cast<uint8_t*>(ws) + (part_bytes + 255) / 256 * 256);
     k.err = err_word;
-    static const unsigned long long wait_ns =
-        (unsigned long long)std::max(1LL, atoll(env_str("FBCORR_WAIT_MS", "4000").c_str())) * 1000000ull;
-    k.wait_ns = wait_ns;
+    k.wait_ns = l.wait_ns;
     k.lo = lo; k.hi = hi;
     k.H = pr.in_h; k.W = pr.in_w; k.Ho = pr.out_h; k.Wo = pr.out_w;
     int lg = 0;

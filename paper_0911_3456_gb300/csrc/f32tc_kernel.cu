@@ -236,6 +236,7 @@ std::string f3_kernel_name(const DirectProblem& pr, const F3Tile& t) {
 
 std::string f3_kernel_source(const DirectProblem& pr, const F3Tile& t, const std::string& name) {
     std::ostringstream o;
+    if (fault_injected("f3drop")) o << "#define FBC_F3_DROP 1\n";   // tests: the first bank copy never comes
     o << rtcg_f32tc_params_source() << "\n" << rtcg_ptx_source() << "\n" << rtcg_f32tc_source() << "\n"
       << snippet_definition(pr.epi == 2 ? pr.snippet : "");
     o << "static_assert(sizeof(FbcF3Params) == " << sizeof(FbcF3Params)
@@ -268,6 +269,7 @@ fbcorr_status_t f3_build(const DirectProblem& pr, const F3Tile& t, int sm_count,
     l.grid = (int)std::min<long long>(items, std::max(1, sm_count));
     l.bank_blocks = (int)((g.bank_chunks + FBC_F3_BANK_THREADS - 1) / FBC_F3_BANK_THREADS);
     l.ws_bytes = f3_ws_bytes(pr, t);
+    l.wait_ns = wait_bound_ns();
     *out = l;
     return FBCORR_OK;
 }
@@ -282,9 +284,7 @@ FbcF3Params f3_params(const F3Launch& l, const DirectProblem& pr, const float* x
     k.flags = reinterpret_cast<int*>(k.bank + (size_t)l.filter_tiles * g.nu * g.bunit);
     k.bank_blocks = l.bank_blocks;
     k.err = err_word;
-    static const unsigned long long wait_ns =
-        (unsigned long long)std::max(1LL, atoll(env_str("FBCORR_WAIT_MS", "4000").c_str())) * 1000000ull;
-    k.wait_ns = wait_ns;
+    k.wait_ns = l.wait_ns;
     k.lo = lo; k.hi = hi;
     k.in_h = pr.in_h; k.in_w = pr.in_w; k.out_h = pr.out_h; k.out_w = pr.out_w;
     k.pad_y = pr.pad_y; k.pad_x = pr.pad_x;

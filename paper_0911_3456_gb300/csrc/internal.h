@@ -36,6 +36,7 @@ std::string env_str(const char* name, const char* dflt = "");
 bool log_enabled();
 void logf(const char* fmt, ...);
 bool fault_injected(const char* what);   // FBCORR_FAULT contains `what`
+unsigned long long wait_bound_ns();      // FBCORR_WAIT_MS (4000) in nanoseconds, read at each call
 std::string cache_dir();                  // FBCORR_CACHE_DIR or ~/.cache/fbcorr
 
 // ---- device facts ------------------------------------------------------------
@@ -250,6 +251,7 @@ struct F3Launch {
     int grid = 0, bank_blocks = 0, filter_tiles = 0;
     int na = 0, nb = 0;
     size_t ws_bytes = 0;       // scratch of one call: the split bank and its flags
+    unsigned long long wait_ns = 0;   // bound of every wait in the kernel
 };
 std::string f3_spec(const F3Tile& t);
 bool f3_parse_spec(const std::string& s, F3Tile* t, int ord = 3);
@@ -281,6 +283,7 @@ struct F3DwLaunch {
     int grid = 0;
     int parts = 0;             // partial sums per element
     size_t ws_bytes = 0;       // partial sums and the CTAs' flags
+    unsigned long long wait_ns = 0;   // bound of every wait in the kernel
 };
 bool f3dw_wins(const DirectProblem& pr, int sm_count, F3DwTile* t);
 size_t f3dw_ws_bytes(const DirectProblem& pr, const F3DwTile& t);

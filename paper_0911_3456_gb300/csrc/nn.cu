@@ -719,8 +719,7 @@ fbcorr_status_t fbcorr_nn_plan_create(fbcorr_nn_plan_t* out, int64_t n_targets, 
         delete p;
         return set_error(FBCORR_ERR_CUDA, "shared memory of the exhaustive fallback kernel (%d bytes)", scan_smem);
     }
-    const long long wait_ms = atoll(env_str("FBCORR_WAIT_MS", "4000").c_str());
-    k.wait_ns = (unsigned long long)std::max(1LL, wait_ms) * 1000000ull;
+    k.wait_ns = wait_bound_ns();
     fbcorr_status_t s = FBCORR_OK;
     if (cudaHostAlloc((void**)&p->err_host, sizeof(int), cudaHostAllocMapped) != cudaSuccess ||
         cudaHostGetDevicePointer((void**)&p->err_dev, p->err_host, 0) != cudaSuccess) {

@@ -177,7 +177,7 @@ __device__ __forceinline__ void fbc_f32dw_body(const FbcF3DwParams& P) {
             }
             fbc_fence_proxy_async_smem();
             __syncwarp();
-            if (lane == 0) fbc_mbar_arrive(full0 + 8u * sl);
+            if (lane == 0 && !(FBC_F3_DROP && warp == 8 && c == c0)) fbc_mbar_arrive(full0 + 8u * sl);
             if (++sl == G::NS) { sl = 0; ph ^= 1; }
             if (c + 1 < c1) load(c + 1);
         }

@@ -66,6 +66,11 @@
 
 #define FBC_F3_ERR_WAIT 5
 
+// 1 (tests of the bounded waits): an arrival that the MMA issuers wait for never comes.
+#ifndef FBC_F3_DROP
+#define FBC_F3_DROP 0
+#endif
+
 // tcgen05.mma with the descriptors as low and high words.
 __device__ __forceinline__ void fbc_umma_lo(fbc_u32 d, fbc_u32 alo, fbc_u32 ahi, fbc_u32 blo, fbc_u32 bhi, fbc_u32 idesc,
                                             fbc_u32 accumulate) {
@@ -550,9 +555,10 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
                     const fbc_u32 off = (fbc_u32)q[r].st * G::BSTAGE;
                     const fbc_u32 bytes = min(G::BSTAGE, G::BUNIT - off);
                     fbc_mbar_expect_tx(b_full0 + 8u * slot, bytes);
-                    fbc_bulk_g2s(sbase + P.b_off + (fbc_u32)slot * G::BSTAGE,
-                                 P.bank + ((long long)q[r].j.ft * G::NU + q[r].j.u) * G::BUNIT + off, bytes,
-                                 b_full0 + 8u * slot);
+                    if (!FBC_F3_DROP || r > 0 || q[r].it > 0)
+                        fbc_bulk_g2s(sbase + P.b_off + (fbc_u32)slot * G::BSTAGE,
+                                     P.bank + ((long long)q[r].j.ft * G::NU + q[r].j.u) * G::BUNIT + off, bytes,
+                                     b_full0 + 8u * slot);
                     ++q[r].it;
                     if (++q[r].bs == P.nb) { q[r].bs = 0; q[r].ph ^= 1; }
                     if (++q[r].st == G::NST) {

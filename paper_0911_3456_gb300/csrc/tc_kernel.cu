@@ -662,8 +662,7 @@ fbcorr_status_t tc_plan_create(TcPlan** out, int H, int W, int D, int N, int fh,
     p->split = split; p->epi = epi; p->lo = lo; p->hi = hi;
     p->snippet = snippet;
     p->sm_count = dev.sm_count;
-    const long long wait_ms = atoll(env_str("FBCORR_WAIT_MS", "4000").c_str());
-    p->wait_ns = (unsigned long long)std::max(1LL, wait_ms) * 1000000ull;
+    p->wait_ns = wait_bound_ns();
     p->drop_b = fault_injected("tcdrop") ? 0 : -1;   // the first B stage: every CTA has one
     // the workspace covers every configuration, CTA pairs included
     const std::vector<TcConfig> cands = tc_candidate_configs(p, true);

@@ -12,6 +12,7 @@
 #include <sys/stat.h>
 #include <unistd.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -69,6 +70,10 @@ void logf(const char* fmt, ...) {
 bool fault_injected(const char* what) {
     const std::string v = env_str("FBCORR_FAULT", "");
     return !v.empty() && v.find(what) != std::string::npos;
+}
+
+unsigned long long wait_bound_ns() {
+    return (unsigned long long)std::max(1LL, atoll(env_str("FBCORR_WAIT_MS", "4000").c_str())) * 1000000ull;
 }
 
 std::string cache_dir() {

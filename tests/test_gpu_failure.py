@@ -89,3 +89,52 @@ def test_corrupt_tune_cache_is_ignored(tmp_path):
     assert normwise_rel(y, oracle.fwd(wl.x, wl.w)) <= 1e-5
     text = (tmp_path / "tune.tsv").read_text(errors="replace")
     assert "direct:" in text or "default" in text
+
+
+F3DROP = [("f32", "f32tc:nt=32,r=1,gc=16,jt=3,ru=1"), ("f32", "f32tc:nt=64,r=2,gc=8,jt=3,ru=2"),
+          ("bf16x3", "tcpack:nt=32,r=1,gc=8,jt=3,ru=2"), ("bf16", "tcpack:nt=32,r=1,gc=16,jt=3,ru=3")]
+
+
+@pytest.mark.parametrize("dtype,spec", F3DROP)
+def test_f32tc_dropped_copy_times_out_and_context_survives(dtype, spec):
+    """FBCORR_FAULT=f3drop leaves out the first copy of the bank, for which an issuer of
+    the kernel then waits in vain (here 50 ms): status, drained copies and MMAs, and a
+    context on which the next plan computes."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    wl = inputs.random_case(3300, 60, 150, 16, 32, 3, 3)
+    x, w = dev(wl.x, torch), dev(wl.w, torch)
+    with _env(FBCORR_FAULT="f3drop", FBCORR_WAIT_MS="50"):
+        bad = Plan(wl.x.shape, wl.w.shape, dtype)
+        bad.set_variant(spec)
+    bad.forward(x, w)
+    torch.cuda.synchronize()
+    assert bad.device_status(clear=True) == 9 and bad.device_status() == 0
+    good = Plan(wl.x.shape, wl.w.shape, dtype)
+    good.set_variant(spec)
+    y = host(good.forward(x, w))
+    assert good.device_status() == 0
+    assert normwise_rel(y, oracle.fwd(wl.x, wl.w)) <= (1e-2 if dtype == "bf16" else 2e-5)
+
+
+@pytest.mark.parametrize("shape", [(30, 41, 16, 64, 7, 7), (21, 60, 4, 36, 2, 19)], ids=["two_planes", "tap_groups"])
+def test_gradients_dropped_arrival_times_out_and_context_survives(shape):
+    """The same for both gradients; dL/dw then comes from the FMA kernel behind it."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    wl = inputs.random_case(3400, *shape, kind="int", with_g=True)
+    args = [dev(t, torch) for t in (wl.x, wl.w, wl.g)]
+    with _env(FBCORR_FAULT="f3drop", FBCORR_WAIT_MS="50", FBCORR_F32TC="force"):
+        bad = Plan(wl.x.shape, wl.w.shape)
+        for kw in ({"need_dw": False}, {"need_dx": False}):
+            dw = bad.backward(*args, **kw)[1]
+            torch.cuda.synchronize()
+            assert bad.device_status(clear=True) == 9 and bad.device_status() == 0
+    assert np.array_equal(host(dw), oracle.bwd_filt(wl.x, wl.g, wl.w.shape))
+    with _env(FBCORR_F32TC="force"):
+        good = Plan(wl.x.shape, wl.w.shape)
+        dx, dw = good.backward(*args)
+        info = good.info()
+    assert info["dx"]["kind"] == "f32tc" and "f32tc" in info["dw"] and good.device_status() == 0
+    assert np.array_equal(host(dx), oracle.bwd_input(wl.g, wl.w, wl.x.shape))
+    assert np.array_equal(host(dw), oracle.bwd_filt(wl.x, wl.g, wl.w.shape))
