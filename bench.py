@@ -842,15 +842,14 @@ def secondary(torch, args, world, peaks):
         del td, nd, plan_nn, res
     out["nn_search_4096_patches_8x8"] = nn_rows
 
-    # the 64-image uneven batch: one persistent launch replayed from a CUDA graph
+    # the 64-image uneven batch: one graph launch per call
     out["batch64_uneven"] = measure_batch(torch, world, flush, fp, 20, 3)
     return out
 
 
 def measure_batch(torch, world, flush, fp, steps, warmup):
     """The 64-image uneven batch (per-image tiles auto-tuned on this GPU): one
-    persistent launch per step, replayed from a CUDA graph, L2 flushed between
-    steps."""
+    graph launch per step, L2 flushed between steps."""
     from paper_0911_3456_gb300 import inputs
     from paper_0911_3456_gb300.api import BatchPlan
     bw = inputs.workload_batch()
@@ -879,7 +878,7 @@ def measure_batch(torch, world, flush, fp, steps, warmup):
 
 def batch_only(args):
     """The 64-image uneven batch alone: W warm-up and K timed steps (one
-    persistent launch each); one JSON line."""
+    graph launch each); one JSON line."""
     import torch
     world, rank, local = dist_setup()
     peaks = load_peaks(torch.cuda.get_device_properties(0).multi_processor_count)
@@ -1008,7 +1007,7 @@ def main():
     ap.add_argument("--fwdbwd", action="store_true",
                     help="the differentiation workload alone (forward, dL/dx, dL/dw)")
     ap.add_argument("--batch", action="store_true",
-                    help="the 64-image uneven batch alone (one persistent launch per step)")
+                    help="the 64-image uneven batch alone (one graph launch per step)")
     ap.add_argument("--small", action="store_true",
                     help="the first configuration alone (flushed steps and a stream of forwards)")
     ap.add_argument("--cascade", action="store_true",

@@ -245,8 +245,10 @@ fbcorr_status_t fbcorr_forward_noalloc(fbcorr_plan_t plan, const float* x, const
 /* ---- batches of uneven images ------------------------------------------- */
 
 /* A plan for n independent problems, image k with in_shapes[k] = {H, W, D}
- * and its own bank filt_shapes[k] = {N, fh, fw, D}, all run by ONE persistent
- * kernel launch (replayed from a CUDA graph) over a largest-first tile list. */
+ * and its own bank filt_shapes[k] = {N, fh, fw, D}, run by one CUDA graph launch
+ * per call: the images that the FP32 tensor-core kernel computes faster as
+ * independent branches (two kernels each), the others by ONE persistent kernel
+ * over a largest-first tile list. */
 fbcorr_status_t fbcorr_batch_plan_create(fbcorr_batch_plan_t* out, int n,
                                          const int64_t (*in_shapes)[3],
                                          const int64_t (*filt_shapes)[4], fbcorr_dtype_t dtype,
@@ -261,10 +263,16 @@ fbcorr_status_t fbcorr_batch_plan_workspace_size(fbcorr_batch_plan_t plan, size_
  * variants and their tiles) into buf (NUL-terminated, cap bytes). */
 fbcorr_status_t fbcorr_batch_plan_info(fbcorr_batch_plan_t plan, char* buf, size_t cap);
 
-/* x[k], w[k], y[k]: HOST arrays of n DEVICE pointers (image k's tensors). */
+/* x[k], w[k], y[k]: HOST arrays of n DEVICE pointers (image k's tensors).
+ * Every image is checked before anything is changed or launched.  A kernel that
+ * gives up a bounded wait is reported by fbcorr_batch_plan_device_status, not by
+ * a later call. */
 fbcorr_status_t fbcorr_forward_batched(fbcorr_batch_plan_t plan, const float* const* x,
                                        const float* const* w, float* const* y, void* ws,
                                        size_t ws_bytes, fbcorr_stream_t stream);
+
+/* As fbcorr_plan_device_status, for the kernels of a batch plan. */
+fbcorr_status_t fbcorr_batch_plan_device_status(fbcorr_batch_plan_t plan, int clear);
 
 /* ---- exact nearest-neighbour search -------------------------------------- */
 

@@ -250,7 +250,7 @@ class Plan:
 
 
 class BatchPlan:
-    """Many uneven images in one persistent launch (``fbcorr_batch_plan_create``)."""
+    """Many uneven images in one graph launch (``fbcorr_batch_plan_create``)."""
 
     def __init__(self, in_shapes, filt_shapes, dtype: str = "f32", clamp: Clamp = None):
         if len(in_shapes) != len(filt_shapes) or not in_shapes:
@@ -287,6 +287,10 @@ class BatchPlan:
         buf = ctypes.create_string_buffer(1 << 16)
         C.call("fbcorr_batch_plan_info", self._h, buf, len(buf))
         return json.loads(buf.value.decode())
+
+    def device_status(self, clear: bool = False) -> int:
+        """0, or the FBCORR_ERR_TIMEOUT status once a kernel gave up a bounded wait."""
+        return int(C.load().fbcorr_batch_plan_device_status(self._h, 1 if clear else 0))
 
     def forward(self, xs, ws_, ys=None, stream=None):
         if len(xs) != self.n or len(ws_) != self.n:

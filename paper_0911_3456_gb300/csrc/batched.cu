@@ -1,17 +1,16 @@
-// batched.cu -- many uneven images in one persistent launch, replayed from a
-// CUDA graph.
+// batched.cu -- many uneven images in one call, replayed from a CUDA graph.
 //
 // The paper's point about its vision models is that input shapes vary widely
 // and a different kernel configuration wins for each (Sec. 6.2).  A batch plan
 // therefore specialises one kernel variant per (filter size, depth, filter
 // class) present in the batch -- all compiled together by NVRTC into ONE
 // kernel that switches on the image's variant -- and schedules every output
-// tile of every image through a single launch:
+// tile of the images that stay on the FMA kernels through a single launch:
 //   * the work list (image, tile_x, tile_y, tile_f) is built at plan time and
 //     ordered by tile cost, largest first (longest-processing-time first);
 //   * persistent CTAs (as many as are co-resident) take items from an atomic
 //     counter, so small and large images balance across SMs;
-//   * the launch is a two-node CUDA graph: zero the counter, run the kernel.
+//   * its part of the CUDA graph is two nodes: zero the counter, run the kernel.
 //     Image pointers are kernel parameters; when a call passes different
 //     pointers the instantiated graph's kernel node is updated in place
 //     (launches already enqueued keep their old parameters).
@@ -515,6 +514,16 @@ fbcorr_status_t fbcorr_batch_plan_info(fbcorr_batch_plan_t b, char* buf, size_t 
     return FBCORR_OK;
 }
 
+fbcorr_status_t fbcorr_batch_plan_device_status(fbcorr_batch_plan_t b, int clear) {
+    clear_error();
+    if (!b) return set_error(FBCORR_ERR_INVALID_ARG, "NULL batch plan");
+    if (!b->err_host) return FBCORR_OK;   // no image on the tensor cores: no bounded wait
+    const int v = *(volatile int*)b->err_host;
+    if (clear) *(volatile int*)b->err_host = 0;
+    if (v == 0) return FBCORR_OK;
+    return set_error(FBCORR_ERR_TIMEOUT, "a batch kernel gave up a bounded wait (code %d)", v);
+}
+
 fbcorr_status_t fbcorr_forward_batched(fbcorr_batch_plan_t b, const float* const* x,
                                        const float* const* w, float* const* y, void* ws,
                                        size_t ws_bytes, fbcorr_stream_t stream) {
@@ -522,10 +531,6 @@ fbcorr_status_t fbcorr_forward_batched(fbcorr_batch_plan_t b, const float* const
     (void)ws;
     (void)ws_bytes;
     if (!b || !x || !w || !y) return set_error(FBCORR_ERR_INVALID_ARG, "NULL argument");
-    if (b->err_host && *(volatile int*)b->err_host != 0) {
-        *(volatile int*)b->err_host = 0;
-        return set_error(FBCORR_ERR_TIMEOUT, "a kernel of an earlier call gave up a bounded wait");
-    }
     // every image is checked before anything is stored: a refused call leaves the plan as it was
     for (int k = 0; k < b->n; ++k) {
         if (!x[k] || !w[k] || !y[k]) return set_error(FBCORR_ERR_INVALID_ARG, "NULL pointer for image %d", k);

@@ -138,3 +138,30 @@ def test_gradients_dropped_arrival_times_out_and_context_survives(shape):
     assert info["dx"]["kind"] == "f32tc" and "f32tc" in info["dw"] and good.device_status() == 0
     assert np.array_equal(host(dx), oracle.bwd_input(wl.g, wl.w, wl.x.shape))
     assert np.array_equal(host(dw), oracle.bwd_filt(wl.x, wl.g, wl.w.shape))
+
+
+def test_batch_dropped_copy_is_reported_and_does_not_refuse_the_next_call():
+    """A batch kernel that gave up a wait shows in the plan's device status, which a
+    single or last call can ask for after a synchronise; the next call still runs."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import BatchPlan
+    items = [inputs.random_case(3500 + k, 40, 50 + 30 * k, 8, 16 * (k + 1), 3, 5, kind="int") for k in range(3)]
+    shapes = [it.x.shape for it in items], [it.w.shape for it in items]
+    xs, ws = [dev(it.x, torch) for it in items], [dev(it.w, torch) for it in items]
+    with _env(FBCORR_FAULT="f3drop", FBCORR_WAIT_MS="50", FBCORR_F32TC="force"):
+        bad = BatchPlan(*shapes)
+    assert bad.info()["tensor_images"] == 3 and bad.device_status() == 0
+    bad.forward(xs, ws)
+    torch.cuda.synchronize()
+    assert bad.device_status() == 9
+    bad.forward(xs, ws)                         # not refused for what the call before it met
+    torch.cuda.synchronize()
+    assert bad.device_status(clear=True) == 9 and bad.device_status() == 0
+    for sw in ("force", "0"):
+        with _env(FBCORR_F32TC=sw):
+            good = BatchPlan(*shapes)
+        ys = good.forward(xs, ws)
+        torch.cuda.synchronize()
+        assert good.device_status() == 0
+        for it, y in zip(items, ys):
+            assert np.array_equal(host(y), oracle.fwd(it.x, it.w))
