@@ -222,8 +222,7 @@ size_t f3_ws_bytes(const DirectProblem& pr, const F3Tile& t) {
     size_t smem;
     if (!layout(pr, t, &na, &nb, &smem)) return 0;
     const Geometry g = geometry(pr, t);
-    const long long blocks = (g.bank_chunks + FBC_F3_BANK_THREADS - 1) / FBC_F3_BANK_THREADS;
-    return (size_t)filter_tiles(pr, t) * (g.nu * g.bunit + blocks * sizeof(int));
+    return (size_t)filter_tiles(pr, t) * g.nu * g.bunit;
 }
 
 std::string f3_kernel_name(const DirectProblem& pr, const F3Tile& t) {
@@ -281,8 +280,6 @@ FbcF3Params f3_params(const F3Launch& l, const DirectProblem& pr, const float* x
     memset(&k, 0, sizeof k);
     k.x = x; k.m = m; k.w = w; k.y = y;
     k.bank = static_cast<unsigned char*>(ws);
-    k.flags = reinterpret_cast<int*>(k.bank + (size_t)l.filter_tiles * g.nu * g.bunit);
-    k.bank_blocks = l.bank_blocks;
     k.err = err_word;
     k.wait_ns = l.wait_ns;
     k.lo = lo; k.hi = hi;

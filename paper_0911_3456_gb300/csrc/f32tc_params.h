@@ -16,7 +16,6 @@ struct FbcF3Params {
     const float* w;             // the bank [N][FH][FW][D] (FLIP reads it flipped and transposed)
     float* y;                   // [out_h][out_w][NF]
     unsigned char* bank;        // the split bank: [filter tile][unit][BSTAGE bytes]
-    int* flags;                 // [filter tile][bank_blocks]: 1 where a block of the split met a tiny value
     int* err;                   // host-mapped error word
     unsigned long long wait_ns; // bound of every mbarrier wait
     float lo, hi;
@@ -27,7 +26,6 @@ struct FbcF3Params {
     int vw_shift;
     int mtiles;                 // 128-pixel tiles over ceil(out_h / R) * vw virtual pixels
     int nitems;                 // mtiles x filter tiles
-    int bank_blocks;            // blocks of the bank split per filter tile
     int na, nb;                 // A slots, B stages per issuer
     unsigned int b_off, bar_off;    // B ring and barrier table in shared memory (A ring at 0)
 };

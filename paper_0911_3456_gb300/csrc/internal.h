@@ -250,7 +250,7 @@ struct F3Launch {
     Kernel kernel, bank;       // the correlation, and the split of the bank before it
     int grid = 0, bank_blocks = 0, filter_tiles = 0;
     int na = 0, nb = 0;
-    size_t ws_bytes = 0;       // scratch of one call: the split bank and its flags
+    size_t ws_bytes = 0;       // scratch of one call: the split bank
     unsigned long long wait_ns = 0;   // bound of every wait in the kernel
 };
 std::string f3_spec(const F3Tile& t);

@@ -32,8 +32,11 @@
 // 1, or of D0 and D1): two threads never add to the same accumulator, so the order
 // of the sums is fixed.
 //
-// A tiny value (see the forward) or a non-finite sum sets the CTA's flag, and the
-// FMA kernel launched next, which otherwise returns at once, computes the result.
+// A non-zero |v| < 2^-100, whose third part could fall below the BF16 range, or a
+// non-finite sum sets the CTA's flag, and the FMA kernel launched next, which
+// otherwise returns at once, computes the result.
+
+#define FBC_F3_TINY ((27u << 24) - 1u)   // 2 * bits(2^-100) - 1
 
 template <int FH_, int FW_, int C_, int NF_, int MASK_, int NB_, int NCOMB_, int JT_, int KPX_>
 struct FbcF3DwCfg {
@@ -155,7 +158,12 @@ __device__ __forceinline__ void fbc_f32dw_body(const FbcF3DwParams& P) {
         };
         if (c0 < c1) load(c0);
         int sl = 0;
-        fbc_u32 ph = 0, tiny = 0xFFFFFFFFu;
+        fbc_u32 ph = 0, tiny = 0xFFFFFFFFu;   // the least of 2|v| - 1 as integers (zeros: the largest)
+        auto put = [&](const float (&v)[4], fbc_u32 dst, fbc_u32 ord) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) tiny = min(tiny, __float_as_uint(v[e]) * 2u - 1u);
+            fbc_f3_put(v, dst, ord);
+        };
         for (int c = c0; c < c1; ++c) {
             if (!fbc_wait(empty0 + 8u * sl, ph ^ 1, P, abort_flag, FBC_F3_ERR_WAIT)) break;
             const fbc_u32 gd = sbase + (fbc_u32)sl * G::SLOT, xd = gd + G::GBYTES;
@@ -164,16 +172,15 @@ __device__ __forceinline__ void fbc_f32dw_body(const FbcF3DwParams& P) {
                 const int it = ct + k * G::NCT;
                 const int px = it / G::QG, q = it % G::QG;
                 if ((k + 1) * G::NCT <= G::KPX * G::QG || px < G::KPX)
-                    fbc_f3_put(gb[k], gd + (fbc_u32)(q >> 1) * G::GPLANE + (fbc_u32)px * 16u + (fbc_u32)(q & 1) * 8u,
-                               (G::NB / 8) * G::GPLANE, tiny);
+                    put(gb[k], gd + (fbc_u32)(q >> 1) * G::GPLANE + (fbc_u32)px * 16u + (fbc_u32)(q & 1) * 8u,
+                        (G::NB / 8) * G::GPLANE);
             }
 #pragma unroll
             for (int k = 0; k < G::KX; ++k) {
                 const int it = ct + k * G::NCT;
                 const int px = it / G::QX, q = it % G::QX;
                 if ((k + 1) * G::NCT <= G::LS * G::QX || px < G::LS)
-                    fbc_f3_put(xb[k], xd + (fbc_u32)(q >> 1) * G::XPLANE + (fbc_u32)px * 16u + (fbc_u32)(q & 1) * 8u, G::XORD,
-                               tiny);
+                    put(xb[k], xd + (fbc_u32)(q >> 1) * G::XPLANE + (fbc_u32)px * 16u + (fbc_u32)(q & 1) * 8u, G::XORD);
             }
             fbc_fence_proxy_async_smem();
             __syncwarp();

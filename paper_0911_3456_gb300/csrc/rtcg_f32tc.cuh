@@ -55,10 +55,19 @@
 // have one ring per issuer; A slots, which the converters fill in order, do not need
 // it: an issuer that has seen unit u - 2 filled knows that every earlier one was.)
 //
-// Values the split cannot carry.  Non-finite inputs or overflow give a
-// non-finite sum, and a non-zero |v| < 2^-100 (whose third part could fall below
-// the BF16 range) raises a flag for its work item; the epilogue warps then
-// recompute their outputs with FP32 FMAs straight from global memory.
+// Range.  BF16 has the exponents of FP32, so the third part of a |v| below 2^-110
+// would fall out of its range, and so would products near 2^-126.  FP32 operands are
+// therefore split as 2^16 v (the least bit of any FP32 value, 2^-149, becomes the
+// least one of BF16, 2^-133) and the sums multiplied by 2^-32 at the end, both exact
+// but for results below the normal range: every value splits exactly, and the small
+// orders keep their bits where FP32 keeps those of the result.  Before, one such value
+// sent its tiles (one in the bank: all of them) to the FMAs below: 512x512x32 *
+// 256x5x5 with one tiny weight took 79 ms, now 0.4 as without it (0.7 % more than with
+// the unscaled split; 2048x2048x4 * 4x8x8 9 % less, as nothing is searched for).
+//
+// Values the split cannot carry.  Non-finite inputs, and sums from 2^96, give a
+// non-finite sum; the epilogue warps then recompute their outputs with FP32 FMAs
+// straight from global memory.
 //
 // Every mbarrier wait is bounded in time; on expiry the kernel records an error
 // code in host-mapped memory, stops every role, waits (bounded) for its MMAs in
@@ -133,43 +142,53 @@ struct FbcF3Cfg {
     static constexpr unsigned TMEM = TC <= 32 ? 32 : TC <= 64 ? 64 : TC <= 128 ? 128 : TC <= 256 ? 256 : 512;
 };
 
-// v = h + m + l exactly (finite v in the BF16 range); tiny takes the least of
-// 2|v| - 1 as integers over the values (zeros: the largest integer).
-__device__ __forceinline__ void fbc_f3_split2(float v0, float v1, fbc_u32& h, fbc_u32& m, fbc_u32& l, fbc_u32& tiny) {
+#define FBC_F3_UP 65536.f                      // 2^16, of each operand of the FP32 split
+#define FBC_F3_DOWN 2.3283064365386963e-10f    // 2^-32, of their sums
+
+// v = h + m + l exactly (finite v, 0 or from 2^-110).
+__device__ __forceinline__ void fbc_f3_split2(float v0, float v1, fbc_u32& h, fbc_u32& m, fbc_u32& l) {
     h = fbc_pack_bf16x2(v0, v1);
     const float r0 = v0 - __uint_as_float(h << 16), r1 = v1 - __uint_as_float(h & 0xFFFF0000u);
     m = fbc_pack_bf16x2(r0, r1);
     l = fbc_pack_bf16x2(r0 - __uint_as_float(m << 16), r1 - __uint_as_float(m & 0xFFFF0000u));
-    tiny = min(tiny, min(__float_as_uint(v0) * 2u - 1u, __float_as_uint(v1) * 2u - 1u));
 }
 
-__device__ __forceinline__ void fbc_f3_split4(const float (&v)[4], fbc_u32 (&h)[2], fbc_u32 (&m)[2], fbc_u32 (&l)[2],
-                                              fbc_u32& tiny) {
-    fbc_f3_split2(v[0], v[1], h[0], m[0], l[0], tiny);
-    fbc_f3_split2(v[2], v[3], h[1], m[1], l[1], tiny);
+__device__ __forceinline__ void fbc_f3_split4(const float (&v)[4], fbc_u32 (&h)[2], fbc_u32 (&m)[2], fbc_u32 (&l)[2]) {
+    fbc_f3_split2(v[0], v[1], h[0], m[0], l[0]);
+    fbc_f3_split2(v[2], v[3], h[1], m[1], l[1]);
+}
+
+// FP32 operands into the split's range (packed multiplies: with scalar ones the dense
+// 512x512x32 * 256x5x5 took 429 us instead of 425); the BF16 modes take them as they are.
+template <int ORD, int N>
+__device__ __forceinline__ void fbc_f3_up(float (&v)[N]) {
+    if constexpr (ORD == 3) {
+#pragma unroll
+        for (int k = 0; k < N; k += 2)
+            asm("{\n .reg .b64 t, u;\n mov.b64 t, {%0, %1};\n mov.b64 u, {%2, %2};\n mul.rn.f32x2 t, t, u;\n"
+                " mov.b64 {%0, %1}, t;\n}\n" : "+f"(v[k]), "+f"(v[k + 1]) : "f"(FBC_F3_UP));
+    }
 }
 
 // The first ORD orders of one chunk (8 values) to shared memory, `ord` bytes apart.
 template <int ORD = 3>
-__device__ __forceinline__ void fbc_f3_put(const float (&v)[8], fbc_u32 dst, fbc_u32 ord, fbc_u32& tiny) {
+__device__ __forceinline__ void fbc_f3_put(const float (&v)[8], fbc_u32 dst, fbc_u32 ord) {
     fbc_u32 h[4], m[4], l[4];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) fbc_f3_split2(v[2 * k], v[2 * k + 1], h[k], m[k], l[k], tiny);
+    for (int k = 0; k < 4; ++k) fbc_f3_split2(v[2 * k], v[2 * k + 1], h[k], m[k], l[k]);
     fbc_st_shared_v4(dst, h[0], h[1], h[2], h[3]);
     if (ORD > 1) fbc_st_shared_v4(dst + ord, m[0], m[1], m[2], m[3]);
     if (ORD > 2) fbc_st_shared_v4(dst + 2 * ord, l[0], l[1], l[2], l[3]);
 }
 
 template <int ORD = 3>
-__device__ __forceinline__ void fbc_f3_put(const float (&v)[4], fbc_u32 dst, fbc_u32 ord, fbc_u32& tiny) {
+__device__ __forceinline__ void fbc_f3_put(const float (&v)[4], fbc_u32 dst, fbc_u32 ord) {
     fbc_u32 h[2], m[2], l[2];
-    fbc_f3_split4(v, h, m, l, tiny);
+    fbc_f3_split4(v, h, m, l);
     fbc_st_shared_v2(dst, h[0], h[1]);
     if (ORD > 1) fbc_st_shared_v2(dst + ord, m[0], m[1]);
     if (ORD > 2) fbc_st_shared_v2(dst + 2 * ord, l[0], l[1]);
 }
-
-#define FBC_F3_TINY ((27u << 24) - 1u)   // 2 * bits(2^-100) - 1
 
 __device__ __forceinline__ int fbc_f3_row(int v, const FbcF3Params& P) {
     return P.vw == 1 ? v : (int)(__umulhi((unsigned)v, P.vw_mul) >> P.vw_shift);
@@ -364,17 +383,18 @@ __device__ __forceinline__ void fbc_f3_load_a(const FbcF3Params& P, const FbcF3P
 // Item `it` of a unit into the A slot at dst; `all`: every thread has one in this pass
 // (no branch: the conversions of several passes interleave).
 template <class G>
-__device__ __forceinline__ void fbc_f3_put_a(int it, bool all, const float (&v)[G::WA], fbc_u32 dst, fbc_u32& tiny) {
+__device__ __forceinline__ void fbc_f3_put_a(int it, bool all, float (&v)[G::WA], fbc_u32 dst) {
     if (!all && it >= G::NIT) return;
+    fbc_f3_up<G::ORD>(v);
     int k, px, sub;
     fbc_f3_a_item<G>(it, k, px, sub);
     const fbc_u32 d = dst + (fbc_u32)k * G::SLAB + (fbc_u32)px * 16u;
     if constexpr (!G::VA) {
-        fbc_f3_put<G::ORD>(v, d + (fbc_u32)sub * G::PLANE, G::AORD, tiny);
+        fbc_f3_put<G::ORD>(v, d + (fbc_u32)sub * G::PLANE, G::AORD);
     } else if constexpr (G::PP == 2) {
         // a pixel of 4 channels: first half of chunk px and second half of chunk px - 1
         fbc_u32 h[2], m[2], l[2];
-        fbc_f3_split4(v, h, m, l, tiny);
+        fbc_f3_split4(v, h, m, l);
         if (px < G::LS) {
             fbc_st_shared_v2(d, h[0], h[1]);
             if (G::ORD > 1) fbc_st_shared_v2(d + G::AORD, m[0], m[1]);
@@ -386,19 +406,18 @@ __device__ __forceinline__ void fbc_f3_put_a(int it, bool all, const float (&v)[
             if (G::ORD > 2) fbc_st_shared_v2(d - 8u + 2 * G::AORD, l[0], l[1]);
         }
     } else {
-        fbc_f3_put<G::ORD>(v, d + (fbc_u32)(sub >> 1) * G::PLANE + (fbc_u32)(sub & 1) * 8u, G::AORD, tiny);
+        fbc_f3_put<G::ORD>(v, d + (fbc_u32)(sub >> 1) * G::PLANE + (fbc_u32)(sub & 1) * 8u, G::AORD);
     }
 }
 
 // The bank split: block (b, filter tile) splits chunks 256 b .. of the tile's
 // NU x NBC chunks (unit, slab row, step, half, column), one per thread, columns
-// fastest, into the B stage images; flags say where a tiny value was met.
+// fastest, into the B stage images.
 template <class G>
 __device__ __forceinline__ void fbc_f32tc_bank_body(const FbcF3Params& P) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int id = blockIdx.x * FBC_F3_BANK_THREADS + threadIdx.x;
-    fbc_u32 tiny = 0xFFFFFFFFu;
     if (id < G::NU * G::NBC) {
         const int u = id / G::NBC, it = id % G::NBC;
         const int col = it % G::NT, kq = (it / G::NT) % (2 * G::S), ri = G::row0(u) + it / (G::NT * 2 * G::S);
@@ -422,23 +441,21 @@ __device__ __forceinline__ void fbc_f32tc_bank_body(const FbcF3Params& P) {
                 v[e] = __ldg(P.w + o);
             }
         }
+        fbc_f3_up<G::ORD>(v);
         fbc_u32 h[4], m[4], l[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) fbc_f3_split2(v[2 * k], v[2 * k + 1], h[k], m[k], l[k], tiny);
+        for (int k = 0; k < 4; ++k) fbc_f3_split2(v[2 * k], v[2 * k + 1], h[k], m[k], l[k]);
         unsigned char* dst = P.bank + ((long long)blockIdx.y * G::NU + u) * G::BUNIT + (it / G::NT) * G::BCH + col * 16;
         *reinterpret_cast<uint4*>(dst) = make_uint4(h[0], h[1], h[2], h[3]);
         if (G::ORD > 1) *reinterpret_cast<uint4*>(dst + G::NT * 16) = make_uint4(m[0], m[1], m[2], m[3]);
         if (G::ORD > 2) *reinterpret_cast<uint4*>(dst + 2 * G::NT * 16) = make_uint4(l[0], l[1], l[2], l[3]);
     }
-    const int any = __syncthreads_or(G::ORD == 3 && tiny < FBC_F3_TINY);
-    if (threadIdx.x == 0) P.flags[blockIdx.y * P.bank_blocks + blockIdx.x] = any;
 }
 
 template <class G>
 __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
     __shared__ int s_abort;
     __shared__ fbc_u32 s_tmem;
-    __shared__ int s_tiny[16];       // item + 1 whose inputs need the FP32 path, by item ordinal % 16
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const fbc_u32 sbase = fbc_smem_addr(fbc_tc_smem);
@@ -468,7 +485,6 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_abort = 0;
     }
-    if (threadIdx.x < 16) s_tiny[threadIdx.x] = 0;
     if (warp == 15) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(fbc_smem_addr(&s_tmem)),
                      "n"(G::TMEM));
@@ -499,24 +515,18 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
         };
 #pragma unroll
         for (int s = 0; s < G::PA; ++s) load_a(abuf[s]);
-        int as = 0, ord = 0, item = ja.item;
+        int as = 0;
         fbc_u32 aph = 0;
         bool ok = true;
         while (ok && ja.valid(P)) {
 #pragma unroll
             for (int s = 0; s < G::PA; ++s) {
                 if (!ok || !ja.valid(P)) break;
-                if (ja.item != item) {
-                    item = ja.item;
-                    ++ord;
-                }
                 if (!(ok = fbc_wait(a_empty0 + 8u * as, aph ^ 1, P, abort_flag, FBC_F3_ERR_WAIT))) break;
                 const fbc_u32 dst = sbase + (fbc_u32)as * G::ASLOT;
-                fbc_u32 tiny = 0xFFFFFFFFu;
 #pragma unroll
-                for (int k = 0; k < G::KA; ++k) 
-                    fbc_f3_put_a<G>(ct + k * G::NCT, (k + 1) * G::NCT <= G::NIT, abuf[s][k], dst, tiny);
-                if (G::ORD == 3 && tiny < FBC_F3_TINY) *(volatile int*)&s_tiny[ord & 15] = ja.item + 1;
+                for (int k = 0; k < G::KA; ++k)
+                    fbc_f3_put_a<G>(ct + k * G::NCT, (k + 1) * G::NCT <= G::NIT, abuf[s][k], dst);
                 fbc_fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) fbc_mbar_arrive(a_full0 + 8u * as);
@@ -661,8 +671,7 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
         constexpr int HC = G::NT / 2;          // columns of this warp
         const int lq = warp & 3, half = warp >> 2;
         const fbc_u32 trow = tmem + ((fbc_u32)(lq * 32) << 16) + (fbc_u32)(half * HC);
-        int acc = 0, ord = 0, ftile = -1;
-        bool tiny_bank = false;
+        int acc = 0;
         fbc_u32 accph = 0;
         bool ok = true;
         // A finished tile is stored in pieces between the drains of the next one: storing
@@ -682,15 +691,9 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
                 }
             o_next += count;
         };
-        for (int item = blockIdx.x; item < P.nitems && ok; item += gridDim.x, ++ord) {
+        for (int item = blockIdx.x; item < P.nitems && ok; item += gridDim.x) {
             const int mt = item % P.mtiles;
             const int n0 = G::R > 1 ? 0 : (item / P.mtiles) * G::NT;
-            if (G::ORD == 3 && item / P.mtiles != ftile) {
-                ftile = item / P.mtiles;
-                int f = 0;
-                for (int b = lane; b < P.bank_blocks; b += 32) f |= P.flags[ftile * P.bank_blocks + b];
-                tiny_bank = __any_sync(0xFFFFFFFFu, f != 0);
-            }
             float sum[HC];
 #pragma unroll
             for (int k = 0; k < HC; ++k) sum[k] = 0.f;
@@ -735,10 +738,9 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
 #pragma unroll
             for (int k = 0; k < HC; ++k) {
                 z += sum[k] - sum[k];
-                out[k] = sum[k];
+                out[k] = G::ORD == 3 ? sum[k] * FBC_F3_DOWN : sum[k];
             }
-            const bool redo = (G::ORD == 3 && (tiny_bank || *(volatile int*)&s_tiny[ord & 15] == item + 1)) ||
-                              __any_sync(0xFFFFFFFFu, inside && !(z == 0.f));
+            const bool redo = __any_sync(0xFFFFFFFFu, inside && !(z == 0.f));
             if (redo && inside) fbc_f3_recompute<G>(P, o_pg, o_q, n0, half * HC, half * HC + HC);
             o_next = inside && !redo ? 0 : NG;
             __syncwarp();

@@ -284,3 +284,61 @@ def test_dx_non_finite_values_against_oracle(where, clamp, monkeypatch):
     with np.errstate(all="ignore"):
         ref = oracle.bwd_input(g, w, wl.x.shape, y=host(y), epilogue=clamp)
     assert np.array_equal(dx, ref, equal_nan=True)
+
+
+def _us(torch, f, calls=8, rounds=5):
+    """Least time of a call in back-to-back runs."""
+    best = float("inf")
+    for _ in range(rounds + 1):            # the first round warms up
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(calls):
+            f()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) / calls * 1e3)
+    return best
+
+
+@pytest.mark.parametrize("shape", [(256, 256, 16, 64, 7, 7), (512, 700, 4, 4, 8, 8)])
+def test_tiny_values_do_not_slow_the_calls(shape):
+    """Denormal and tiny weights, pixels and gradients split like any other value: a call
+    with them takes what the call without them takes (it took 10 to 1000 times that)."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    H, W, D, N, fh, fw = shape
+    gen = torch.Generator(device="cuda").manual_seed(7900)
+    x = torch.rand((H, W, D), generator=gen, device="cuda") - 0.5
+    w = torch.randn((N, fh, fw, D), generator=gen, device="cuda")
+    p = Plan(x.shape, w.shape)
+    g = torch.randn(p.out_shape, generator=gen, device="cuda")
+    x1, w1, g1 = x.clone(), w.clone(), g.clone()
+    x1.view(-1)[::997] = 1e-33
+    w1[N // 2, 1, 1, 1] = -1e-38
+    g1.view(-1)[::997] = 1e-40
+    plain = _us(torch, lambda: p.forward(x, w)), _us(torch, lambda: p.backward(x, w, g, need_dw=False))
+    assert p.info()["fwd"]["kind"] == "f32tc" and p.info()["dx"]["kind"] == "f32tc"
+    for a, b in ((x1, w), (x, w1)):
+        assert _us(torch, lambda: p.forward(a, b)) <= 1.5 * plain[0]
+    for b, c in ((w1, g), (w, g1)):
+        assert _us(torch, lambda: p.backward(x, b, c, need_dw=False)) <= 1.5 * plain[1]
+
+
+@pytest.mark.parametrize("ex,ew", [(-70, -70), (-66, -73), (-100, -40), (-126, -14), (-140, 20), (30, -140)])
+def test_small_values_and_products_keep_fp32_accuracy(ex, ew, monkeypatch):
+    """Operands down to the denormal ones, and results near the end of the range: the
+    error is the file's bound with the kernel's one chunk, and one rounding to a
+    multiple of 2^-149 (derived: the sums are held 2^32 times larger)."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    monkeypatch.setenv("FBCORR_DX_VARIANT", "f32tc:nt=16,r=1,gc=16,jt=3,ru=3")
+    wl = inputs.random_case(7950, 20, 40, 8, 16, 3, 3, with_g=True)
+    x, w, g = wl.x * np.float32(2.0 ** ex), wl.w * np.float32(2.0 ** ew), wl.g * np.float32(2.0 ** ex)
+    p = Plan(x.shape, w.shape)
+    p.set_variant("f32tc:nt=32,r=1,gc=8,jt=3,ru=3")
+    y = host(p.forward(dev(x, torch), dev(w, torch)))
+    dx = host(p.backward(dev(x, torch), dev(w, torch), dev(g, torch), need_dw=False)[0])
+    assert p.info()["dx"]["spec"].startswith("f32tc")
+    for got, ref, mag in ((y, oracle.fwd(x, w), oracle.fwd(np.abs(x), np.abs(w))),
+                          (dx, oracle.bwd_input(g, w, x.shape), oracle.bwd_input(np.abs(g), np.abs(w), x.shape))):
+        assert np.all(np.abs(got - ref) <= (16 * 2.0 ** -23 + 5 * 2.0 ** -24) * mag + 2.0 ** -149)
