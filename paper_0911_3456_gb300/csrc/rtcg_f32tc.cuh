@@ -158,16 +158,20 @@ __device__ __forceinline__ void fbc_f3_split4(const float (&v)[4], fbc_u32 (&h)[
     fbc_f3_split2(v[2], v[3], h[1], m[1], l[1]);
 }
 
-// FP32 operands into the split's range (packed multiplies: with scalar ones the dense
-// 512x512x32 * 256x5x5 took 429 us instead of 425); the BF16 modes take them as they are.
+// Packed multiplies: with scalar ones the dense 512x512x32 * 256x5x5 took 429 us
+// instead of 425.
+template <int N>
+__device__ __forceinline__ void fbc_f3_scale(float (&v)[N], float s) {
+#pragma unroll
+    for (int k = 0; k < N; k += 2)
+        asm("{\n .reg .b64 t, u;\n mov.b64 t, {%0, %1};\n mov.b64 u, {%2, %2};\n mul.rn.f32x2 t, t, u;\n"
+            " mov.b64 {%0, %1}, t;\n}\n" : "+f"(v[k]), "+f"(v[k + 1]) : "f"(s));
+}
+
+// FP32 operands into the split's range; the BF16 modes take them as they are.
 template <int ORD, int N>
 __device__ __forceinline__ void fbc_f3_up(float (&v)[N]) {
-    if constexpr (ORD == 3) {
-#pragma unroll
-        for (int k = 0; k < N; k += 2)
-            asm("{\n .reg .b64 t, u;\n mov.b64 t, {%0, %1};\n mov.b64 u, {%2, %2};\n mul.rn.f32x2 t, t, u;\n"
-                " mov.b64 {%0, %1}, t;\n}\n" : "+f"(v[k]), "+f"(v[k + 1]) : "f"(FBC_F3_UP));
-    }
+    if constexpr (ORD == 3) fbc_f3_scale(v, FBC_F3_UP);
 }
 
 // The first ORD orders of one chunk (8 values) to shared memory, `ord` bytes apart.

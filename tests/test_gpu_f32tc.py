@@ -342,3 +342,23 @@ def test_small_values_and_products_keep_fp32_accuracy(ex, ew, monkeypatch):
     for got, ref, mag in ((y, oracle.fwd(x, w), oracle.fwd(np.abs(x), np.abs(w))),
                           (dx, oracle.bwd_input(g, w, x.shape), oracle.bwd_input(np.abs(g), np.abs(w), x.shape))):
         assert np.all(np.abs(got - ref) <= (16 * 2.0 ** -23 + 5 * 2.0 ** -24) * mag + 2.0 ** -149)
+
+
+@pytest.mark.parametrize("ex,eg", [(-70, -70), (-66, -66), (-95, -40), (60, 60)])
+def test_dw_small_products_keep_fp32_accuracy(ex, eg, monkeypatch):
+    """dL/dw near the end of the range (every value of the split's range, sums near
+    2^-130): the bound of one chunk per 96 pixels and partial sum, and one rounding to a
+    multiple of 2^-149 for each of the at most 40 partial sums and their total; and
+    sums that the kernel holds 2^32 times larger than FP32 could: from the FMA kernel."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    monkeypatch.setenv("FBCORR_F32TC", "force")
+    wl = inputs.random_case(7960, 30, 41, 16, 64, 5, 5, with_g=True)
+    least = np.float32(2.0 ** -4)              # no value below the split's range
+    x = np.where(np.abs(wl.x) < least, least, wl.x) * np.float32(2.0 ** ex)
+    g = np.where(np.abs(wl.g) < least, least, wl.g) * np.float32(2.0 ** eg)
+    p = Plan(x.shape, wl.w.shape)
+    dw = host(p.backward(dev(x, torch), dev(wl.w, torch), dev(g, torch), need_dx=False)[1])
+    assert "f32tc" in p.info()["dw"] and p.device_status() == 0
+    ref, mag = oracle.bwd_filt(x, g, wl.w.shape), oracle.bwd_filt(np.abs(x), np.abs(g), wl.w.shape)
+    assert np.all(np.abs(dw - ref) <= (16 * 2.0 ** -23 + 64 * 2.0 ** -24) * mag + 41 * 2.0 ** -150)
