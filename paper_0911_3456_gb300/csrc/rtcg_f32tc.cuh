@@ -66,8 +66,10 @@
 // the unscaled split; 2048x2048x4 * 4x8x8 9 % less, as nothing is searched for).
 //
 // Values the split cannot carry.  Non-finite inputs, and sums from 2^96, give a
-// non-finite sum; the epilogue warps then recompute their outputs with FP32 FMAs
-// straight from global memory.
+// non-finite sum.  The epilogue warps only note where (a call in their loop cost
+// 2048x2048x4 * 4x8x8 a fifth in spilled registers); once the pipeline has ended, all
+// warps of the CTA compute those outputs again, in groups of 8 pixels x 8 columns, with
+// FP32 FMAs straight from global memory (fbc_f3_redo).
 //
 // Every mbarrier wait is bounded in time; on expiry the kernel records an error
 // code in host-mapped memory, stops every role, waits (bounded) for its MMAs in
@@ -249,50 +251,149 @@ __device__ __forceinline__ void fbc_f3_store8(const FbcF3Params& P, int pg, int 
 
 __device__ __forceinline__ float fbc_f3_bf16(float v) { return __uint_as_float(fbc_pack_bf16x2(v, 0.f) << 16); }
 
-// Columns [c0, c1) of one pixel recomputed with FP32 FMAs from global memory (the
-// BF16 modes: of the rounded values).
+// x w added to acc in FP32 (the BF16 modes: the products of the rounded values).
 template <class G>
-__device__ __noinline__ void fbc_f3_recompute(const FbcF3Params& P, int pg, int q, int n0, int c0, int c1) {
-    for (int col0 = c0; col0 < c1; col0 += 8) {
-        float acc[8];
-        int rr[8], nn[8];
-        bool on[8];
+__device__ __forceinline__ float fbc_f3_mac(float x, float w, float acc) {
+    if constexpr (G::ORD == 3) return fmaf(x, w, acc);
+    const float xh = fbc_f3_bf16(x), wh = fbc_f3_bf16(w);
+    if constexpr (G::ORD == 2) {
+        acc = fmaf(xh, fbc_f3_bf16(w - wh), acc);
+        acc = fmaf(fbc_f3_bf16(x - xh), wh, acc);
+    }
+    return fmaf(xh, wh, acc);
+}
+
+// N consecutive floats (N = 4: on a 16-byte boundary).
+template <int N>
+__device__ __forceinline__ void fbc_f3_ldg(const float* p, float (&v)[N]) {
+    if constexpr (N == 4) {
+        const float4 f = __ldg(reinterpret_cast<const float4*>(p));
+        v[0] = f.x;
+        v[1] = f.y;
+        v[2] = f.z;
+        v[3] = f.w;
+    } else {
+        v[0] = __ldg(p);
+    }
+}
+
+// Columns col0 .. col0 + 7 of those of the warp's 32 pixels that `mask` names, again,
+// with FP32 FMAs from global memory.  Bound by the loads: four lanes share the FW C
+// products of a filter row (consecutive floats of x, and of an unflipped bank) and
+// hold four pixels x 8 columns each, so that 12 loads of 16 bytes feed 128 FMAs, with
+// 8 pixels' lines per load of x and one per load of w.  512x512x32 * 256x5x5 with one
+// NaN pixel 0.44 ms, one NaN weight 0.53, NaN all over the image 4.4 (one thread per
+// pixel and whole tiles: 12, 63 and 304; without NaN 0.40; the FMA kernel 1.93).
+template <class G>
+__device__ __forceinline__ void fbc_f3_redo(const FbcF3Params& P, fbc_u32 mask, int pg, int q, int n0, int col0) {
+    if (G::R == 1 ? n0 + col0 >= G::NF : col0 >= G::R * G::NF) return;
+    constexpr int V = G::VA ? 4 : 1;
+    const int part = threadIdx.x & 3, slot = (threadIdx.x & 31) >> 2;
+    int row0[4], col[4];
+    bool on[4];
+    float acc[4][8];
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            acc[k] = 0.f;
-            rr[k] = G::R > 1 ? (col0 + k) / G::NF : 0;
-            nn[k] = G::R > 1 ? (col0 + k) % G::NF : n0 + col0 + k;
-            on[k] = rr[k] < G::R && pg * G::R + rr[k] < P.out_h && nn[k] < G::NF;
-        }
-        for (int i = 0; i < G::FH; ++i)
-            for (int j = 0; j < G::FW; ++j) {
-                const int xc = q + j - P.pad_x;
-                if (xc < 0 || xc >= P.in_w) continue;
-                for (int c = 0; c < G::C; ++c) {
+    for (int t = 0; t < 4; ++t) {
+        row0[t] = __shfl_sync(0xFFFFFFFFu, pg, 8 * t + slot) * G::R - P.pad_y;
+        col[t] = __shfl_sync(0xFFFFFFFFu, q, 8 * t + slot) - P.pad_x;
+        on[t] = (mask >> (8 * t + slot)) & 1u;
 #pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const int xr = pg * G::R + rr[k] + i - P.pad_y;
-                        if (!on[k] || xr < 0 || xr >= P.in_h) continue;
-                        const long long xo = ((long long)xr * P.in_w + xc) * G::C + c;
-                        const long long wo =
-                            G::FLIP ? (((long long)c * G::FH + (G::FH - 1 - i)) * G::FW + (G::FW - 1 - j)) * G::NF + nn[k]
-                                    : (((long long)nn[k] * G::FH + i) * G::FW + j) * G::C + c;
-                        const float xv = fbc_f3_masked<G>(__ldg(P.x + xo), P.m + xo, P), wv = __ldg(P.w + wo);
-                        if constexpr (G::ORD == 3) {
-                            acc[k] = fmaf(xv, wv, acc[k]);
-                        } else {
-                            const float xh = fbc_f3_bf16(xv), wh = fbc_f3_bf16(wv);
-                            if constexpr (G::ORD == 2) {
-                                acc[k] = fmaf(xh, fbc_f3_bf16(wv - wh), acc[k]);
-                                acc[k] = fmaf(fbc_f3_bf16(xv - xh), wh, acc[k]);
-                            }
-                            acc[k] = fmaf(xh, wh, acc[k]);
-                        }
+        for (int k = 0; k < 8; ++k) acc[t][k] = 0.f;
+    }
+    const int r0 = G::R > 1 ? col0 / G::NF : 0, r1 = G::R > 1 ? min(G::R - 1, (col0 + 7) / G::NF) : 0;
+#pragma unroll 1
+    for (int ri = 0; ri < (r1 - r0 + 1) * G::FH; ++ri) {
+        const int r = r0 + ri / G::FH, i = ri % G::FH;
+        const int nb = G::R > 1 ? col0 - r * G::NF : n0 + col0;     // filter of the first column
+#pragma unroll 1
+        for (int e0 = part * V; e0 < G::FW * G::C; e0 += 4 * V) {
+            const int j = e0 / G::C, c = e0 % G::C;
+            // every load before the first FMA, none behind a branch: what takes no part
+            // reads the first pixel or a neighbouring filter and is left out of the sums
+            float xv[4][V], wv[8][V];
+            bool ok[4];
+#pragma unroll
+            for (int t = 0; t < 4; ++t) {
+                const int xr = row0[t] + r + i, xc = col[t] + j;
+                ok[t] = on[t] && xr >= 0 && xr < P.in_h && xc >= 0 && xc < P.in_w;
+                const unsigned o = ok[t] ? ((unsigned)xr * P.in_w + xc) * G::C + c : 0u;
+                fbc_f3_ldg<V>(P.x + o, xv[t]);
+                if constexpr (G::MASK) {
+                    float mv[V];
+                    fbc_f3_ldg<V>(P.m + o, mv);
+#pragma unroll
+                    for (int e = 0; e < V; ++e) xv[t][e] = mv[e] > P.lo && mv[e] < P.hi ? xv[t][e] : 0.f;
+                }
+            }
+            if constexpr (G::FLIP && G::NF % 4 == 0) {
+#pragma unroll
+                for (int k = 0; k < 8; k += 4) {
+                    const int n = min(max(nb + k, 0), G::NF - 4);
+#pragma unroll
+                    for (int e = 0; e < V; ++e) {
+                        float f[4];
+                        fbc_f3_ldg<4>(P.w + (((unsigned)(c + e) * G::FH + (G::FH - 1 - i)) * G::FW + (G::FW - 1 - j)) * G::NF + n, f);
+#pragma unroll
+                        for (int h = 0; h < 4; ++h) wv[k + h][e] = f[h];
+                    }
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int n = min(max(nb + k, 0), G::NF - 1);
+                    if constexpr (!G::FLIP) {
+                        fbc_f3_ldg<V>(P.w + ((unsigned)n * G::FH + i) * (G::FW * G::C) + e0, wv[k]);
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < V; ++e)
+                            fbc_f3_ldg<1>(P.w + (((unsigned)(c + e) * G::FH + (G::FH - 1 - i)) * G::FW + (G::FW - 1 - j)) * G::NF + n,
+                                          reinterpret_cast<float(&)[1]>(wv[k][e]));
                     }
                 }
             }
-        fbc_f3_store8<G>(P, pg, q, n0, col0, acc);
+            // a tap outside the image takes no part (it could be 0 x inf); without a border there is none
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if (G::R == 1 || (nb + k >= 0 && nb + k < G::NF)) {
+#pragma unroll
+                    for (int t = 0; t < 4; ++t)
+#pragma unroll
+                        for (int e = 0; e < V; ++e)
+                            if (!G::FLIP || ok[t]) acc[t][k] = fbc_f3_mac<G>(xv[t][e], wv[k][e], acc[t][k]);
+                }
+        }
     }
+    // the four lanes' sums; each stores one of the four pixels
+    float v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            acc[t][k] += __shfl_xor_sync(0xFFFFFFFFu, acc[t][k], 1);
+            acc[t][k] += __shfl_xor_sync(0xFFFFFFFFu, acc[t][k], 2);
+        }
+        v[k] = part == 0 ? acc[0][k] : part == 1 ? acc[1][k] : part == 2 ? acc[2][k] : acc[3][k];
+    }
+    const int src = 8 * part + slot;
+    pg = __shfl_sync(0xFFFFFFFFu, pg, src);
+    q = __shfl_sync(0xFFFFFFFFu, q, src);
+    if ((mask >> src) & 1u) fbc_f3_store8<G>(P, pg, q, n0, col0, v);
+}
+
+// Notes that warp `warp` met non-finite sums at the lanes of `mask` in its 8 columns g
+// of the CTA's item `ord`: item, warp, group, and which of the lanes' four bytes.  Items
+// for which there is no room are computed again whole, and all after them.
+#define FBC_F3_NOTES 240   // with the rest at most 1 KB of static shared memory
+__device__ __forceinline__ void fbc_f3_note(fbc_u32 mask, int ord, int warp, int g, int lane, fbc_u32* list, int* count, int* from) {
+    if (mask == 0 || lane != 0) return;
+    const int k = ord < (1 << 22) ? atomicAdd(count, 1) : FBC_F3_NOTES;
+    if (k >= FBC_F3_NOTES) {
+        atomicMin(from, ord);
+        return;
+    }
+    fbc_u32 bytes = 0;
+    for (int b = 0; b < 4; ++b) bytes |= (mask >> (8 * b) & 0xFFu) ? 1u << b : 0u;
+    list[k] = (fbc_u32)ord << 10 | (fbc_u32)warp << 7 | (fbc_u32)g << 4 | bytes;
 }
 
 // Position in a CTA's sequence of (work item, unit); item = filter tile * mtiles + pixel tile.
@@ -460,6 +561,8 @@ template <class G>
 __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
     __shared__ int s_abort;
     __shared__ fbc_u32 s_tmem;
+    __shared__ fbc_u32 s_bad[FBC_F3_NOTES];   // groups of outputs with a non-finite sum, and how many
+    __shared__ int s_nbad, s_bad_from;        // (from item s_bad_from on they found no room)
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const fbc_u32 sbase = fbc_smem_addr(fbc_tc_smem);
@@ -488,6 +591,8 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
         fbc_mbar_init(drain_bar + 8u, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         s_abort = 0;
+        s_nbad = 0;
+        s_bad_from = 0x7FFFFFFF;
     }
     if (warp == 15) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(fbc_smem_addr(&s_tmem)),
@@ -675,7 +780,7 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
         constexpr int HC = G::NT / 2;          // columns of this warp
         const int lq = warp & 3, half = warp >> 2;
         const fbc_u32 trow = tmem + ((fbc_u32)(lq * 32) << 16) + (fbc_u32)(half * HC);
-        int acc = 0;
+        int acc = 0, ord = 0;
         fbc_u32 accph = 0;
         bool ok = true;
         // A finished tile is stored in pieces between the drains of the next one: storing
@@ -695,7 +800,7 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
                 }
             o_next += count;
         };
-        for (int item = blockIdx.x; item < P.nitems && ok; item += gridDim.x) {
+        for (int item = blockIdx.x; item < P.nitems && ok; item += gridDim.x, ++ord) {
             const int mt = item % P.mtiles;
             const int n0 = G::R > 1 ? 0 : (item / P.mtiles) * G::NT;
             float sum[HC];
@@ -744,9 +849,16 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
                 z += sum[k] - sum[k];
                 out[k] = G::ORD == 3 ? sum[k] * FBC_F3_DOWN : sum[k];
             }
-            const bool redo = __any_sync(0xFFFFFFFFu, inside && !(z == 0.f));
-            if (redo && inside) fbc_f3_recompute<G>(P, o_pg, o_q, n0, half * HC, half * HC + HC);
-            o_next = inside && !redo ? 0 : NG;
+            if (__any_sync(0xFFFFFFFFu, inside && !(z == 0.f))) {
+#pragma unroll
+                for (int g = 0; g < NG; ++g) {
+                    z = 0.f;
+#pragma unroll
+                    for (int k = 8 * g; k < 8 * g + 8; ++k) z += out[k] - out[k];
+                    fbc_f3_note(__ballot_sync(0xFFFFFFFFu, inside && !(z == 0.f)), ord, warp, g, lane, s_bad, &s_nbad, &s_bad_from);
+                }
+            }
+            o_next = inside ? 0 : NG;
             __syncwarp();
         }
         if (o_next < NG) store_some(NG);
@@ -757,4 +869,23 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
     fbc_tc_fence_after();
     if (warp == 15)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(G::TMEM));
+    // the noted groups, by every warp: the stores above came before the barrier
+    if (s_abort) return;
+    constexpr int NG = G::NT / 16;
+    const int listed = min(s_nbad, FBC_F3_NOTES), from = s_bad_from;
+    const int items = (P.nitems - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    const long long all = listed + (from < items ? (long long)(items - from) * 8 * NG : 0);
+#pragma unroll 1
+    for (long long k = warp; k < all; k += FBC_F3_THREADS / 32) {
+        const long long past = k - listed;     // beyond the list: every group of the items from `from` on
+        const fbc_u32 n = past < 0 ? s_bad[k] : 0xFu;
+        const int ord = past < 0 ? (int)(n >> 10) : from + (int)(past / (8 * NG));
+        const int wq = past < 0 ? (int)(n >> 7) & 7 : (int)(past / NG) & 7, g = past < 0 ? (int)(n >> 4) & 7 : (int)(past % NG);
+        const int item = blockIdx.x + ord * gridDim.x;
+        const int v = (item % P.mtiles) * 128 + (wq & 3) * 32 + lane;
+        const int pg = fbc_f3_row(v, P), q = v - pg * P.vw;
+        const bool inside = q < P.out_w && pg * G::R < P.out_h && ((n >> (lane >> 3)) & 1u);
+        const fbc_u32 mask = __ballot_sync(0xFFFFFFFFu, inside);
+        fbc_f3_redo<G>(P, mask, pg, q, G::R > 1 ? 0 : item / P.mtiles * G::NT, (wq >> 2) * (G::NT / 2) + 8 * g);
+    }
 }

@@ -362,3 +362,98 @@ def test_dw_small_products_keep_fp32_accuracy(ex, eg, monkeypatch):
     assert "f32tc" in p.info()["dw"] and p.device_status() == 0
     ref, mag = oracle.bwd_filt(x, g, wl.w.shape), oracle.bwd_filt(np.abs(x), np.abs(g), wl.w.shape)
     assert np.all(np.abs(dw - ref) <= (16 * 2.0 ** -23 + 64 * 2.0 ** -24) * mag + 41 * 2.0 ** -150)
+
+
+def _spoiled(t):
+    """Integers with a NaN, an infinity and a value whose sums leave the split's range."""
+    t = t.copy()
+    f = t.reshape(-1)
+    f[f.size // 3], f[f.size // 2], f[2 * f.size // 3] = np.nan, -np.inf, 2.0 ** 100
+    return t
+
+
+def _same_as_oracle(got, ref, mag, terms):
+    """Non-finite values alike, integers equal, and sums with 2^100 in them within the
+    rounding of one FMA per term."""
+    fin = np.isfinite(ref)
+    assert np.array_equal(got[~fin], ref[~fin], equal_nan=True)
+    small = fin & (mag < 2.0 ** 24)
+    assert np.array_equal(got[small], ref[small])
+    assert np.all(np.abs(got[fin] - ref[fin]) <= (terms + 4) * 2.0 ** -24 * mag[fin])
+
+
+@pytest.mark.parametrize("where", ["x", "w"])
+@pytest.mark.parametrize("shape,spec", CASES)
+def test_recomputed_outputs_in_every_layout(shape, spec, where):
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    wl = inputs.random_case(7970, *shape, kind="int")
+    x, w = (_spoiled(wl.x), wl.w) if where == "x" else (wl.x, _spoiled(wl.w))
+    p = Plan(x.shape, w.shape)
+    p.set_variant(spec)
+    y = host(p.forward(dev(x, torch), dev(w, torch)))
+    assert p.device_status() == 0
+    with np.errstate(all="ignore"):
+        _same_as_oracle(y, oracle.fwd(x, w), oracle.fwd(np.abs(x), np.abs(w)), shape[2] * shape[4] * shape[5])
+
+
+@pytest.mark.parametrize("clamp", [None, (-20.5, 20.5)])
+@pytest.mark.parametrize("where", ["g", "w"])
+@pytest.mark.parametrize("shape,spec", [
+    ((20, 23, 16, 64, 7, 7), "f32tc:nt=64,r=4,gc=32,jt=7,ru=1"),
+    ((19, 26, 12, 40, 5, 3), "f32tc:nt=48,r=3,gc=8,jt=3,ru=4"),
+    ((24, 31, 5, 7, 3, 4), "f32tc:nt=16,r=1,gc=8,jt=4,ru=2"),
+    ((17, 40, 33, 3, 2, 5), "f32tc:nt=48,r=1,gc=8,jt=3,ru=1"),
+    ((22, 31, 6, 12, 3, 3), "f32tc:nt=32,r=5,gc=8,jt=3,ru=2"),
+])
+def test_recomputed_gradients_in_every_layout(shape, spec, where, clamp, monkeypatch):
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    monkeypatch.setenv("FBCORR_DX_VARIANT", spec)
+    wl = inputs.random_case(7980, *shape, kind="int", with_g=True)
+    g, w = (_spoiled(wl.g), wl.w) if where == "g" else (wl.g, _spoiled(wl.w))
+    p = Plan(wl.x.shape, w.shape, "f32", clamp)
+    y = oracle.fwd(wl.x, wl.w, epilogue=clamp).astype(np.float32)
+    dx = host(p.backward(dev(wl.x, torch), dev(w, torch), dev(g, torch), dev(y, torch), need_dw=False)[0])
+    assert p.info()["dx"]["spec"] == spec and p.device_status() == 0
+    with np.errstate(all="ignore"):
+        ref = oracle.bwd_input(g, w, wl.x.shape, y=y.astype(np.float64), epilogue=clamp)
+        mag = oracle.bwd_input(np.abs(g), np.abs(w), wl.x.shape, y=y.astype(np.float64), epilogue=clamp)
+    _same_as_oracle(dx, ref, mag, shape[3] * shape[4] * shape[5])
+
+
+def test_more_recomputed_groups_than_a_block_notes():
+    """NaN in most groups of pixels: past its list a block computes whole items again."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    wl = inputs.random_case(7985, 402, 410, 4, 80, 2, 2, kind="int")
+    x = wl.x.copy()
+    x.reshape(-1)[::97] = np.nan
+    p = Plan(x.shape, wl.w.shape)
+    p.set_variant("f32tc:nt=80,r=1,gc=8,jt=2,ru=2")
+    y = host(p.forward(dev(x, torch), dev(wl.w, torch)))
+    assert p.device_status() == 0
+    assert np.array_equal(y, oracle.fwd(x, wl.w), equal_nan=True)
+
+
+@pytest.mark.parametrize("shape", [(256, 256, 16, 64, 7, 7), (512, 700, 4, 4, 8, 8)])
+def test_non_finite_values_cost_no_more_than_a_few_fma_kernels(shape):
+    """A NaN weight, one NaN pixel or one NaN gradient, and NaN everywhere: at most four
+    times what the FMA kernels take for the whole call (it was 20 to 1000 times)."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    H, W, D, N, fh, fw = shape
+    gen = torch.Generator(device="cuda").manual_seed(7990)
+    x = torch.rand((H, W, D), generator=gen, device="cuda") - 0.5
+    w = torch.randn((N, fh, fw, D), generator=gen, device="cuda")
+    p = Plan(x.shape, w.shape)
+    g = torch.randn(p.out_shape, generator=gen, device="cuda")
+    small = torch.empty(16, dtype=torch.uint8, device="cuda")     # no scratch: the FMA kernels
+    x1, x2, w1, g1, g2 = x.clone(), x.clone(), w.clone(), g.clone(), g.clone()
+    x1[H // 2, W // 3, 1] = w1[N // 2, 1, 1, 1] = g1[H // 2, W // 3, 1] = float("nan")
+    x2.view(-1)[::997] = g2.view(-1)[::997] = float("nan")
+    fma = (_us(torch, lambda: p.forward(x, w, ws=small)), _us(torch, lambda: p.backward(x, w, g, need_dw=False, ws=small)))
+    for a, b in ((x1, w), (x2, w), (x, w1)):
+        assert _us(torch, lambda: p.forward(a, b)) <= 4 * fma[0]
+    for b, c in ((w1, g), (w, g1), (w, g2)):
+        assert _us(torch, lambda: p.backward(x, b, c, need_dw=False)) <= 4 * fma[1]
