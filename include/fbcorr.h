@@ -144,8 +144,9 @@ fbcorr_status_t fbcorr_plan_workspace_size(fbcorr_plan_t plan, size_t* fwd_bytes
  * kernels (either pointer may be NULL): at least the sizes above.  FP32 plans
  * need none for the forward, but given this much they may run it -- and, in
  * every plan, dL/dx -- on the tensor cores (each FP32 value split exactly into
- * three BF16 values); with less they run FP32 FMA kernels.  The size may change
- * with fbcorr_autotune and fbcorr_plan_set_variant. */
+ * three BF16 values); with less they run FP32 FMA kernels (the fastest measured,
+ * where the shape has been tuned).  The size may change with fbcorr_autotune and
+ * fbcorr_plan_set_variant. */
 fbcorr_status_t fbcorr_plan_scratch_size(fbcorr_plan_t plan, size_t* fwd_bytes, size_t* bwd_bytes);
 
 /* y = epi(corr(x, w)).  x, w, y: device pointers as above; ws: device
@@ -226,9 +227,10 @@ fbcorr_status_t fbcorr_plan_profile_read(fbcorr_plan_t plan, float* ms, int cap,
  * correlation (no cudaMalloc after start-up in a real-time loop, a plugin host
  * whose allocator belongs to another runtime, a process that budgets all
  * device memory at initialisation).  It runs the same kernels as
- * fbcorr_forward, but the scratch that tensor-core plans need (the BF16 copies
- * of x and w) lives in one 48 MiB array built into the library, which every
- * GPU that loads the library keeps until the process exits.  Plans whose
+ * fbcorr_forward (FP32 plans: as it does without scratch), but the scratch that
+ * tensor-core plans need (the BF16 copies of x and w) lives in one 48 MiB array
+ * built into the library, which every GPU that loads the library keeps until the
+ * process exits.  Plans whose
  * forward workspace (fbcorr_plan_workspace_size) exceeds 48 MiB are rejected
  * with FBCORR_ERR_WORKSPACE; FP32 plans need no scratch.  The first call on a
  * device looks up the array's device address, so make that first call before

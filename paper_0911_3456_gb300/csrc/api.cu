@@ -138,8 +138,30 @@ fbcorr_status_t set_tc_heuristic(fbcorr_plan* p) {
     return FBCORR_OK;
 }
 
-// Select the forward variant of an F32 plan from a spec string.
-fbcorr_status_t set_fwd_spec(fbcorr_plan* p, const std::string& spec, const char* source) {
+// The FMA kernel that calls without scratch run beside a tensor-core one (what: "fwd"
+// or "dx"): the spec `fma`, the tuning cache's, or the heuristic's, whichever is the
+// first to fit.  The prebuilt kernel ("default") is an empty *k.
+fbcorr_status_t build_fma(const fbcorr_plan* p, const char* what, const DirectProblem& pr, std::string fma, DirectTile* t,
+                          Kernel* k) {
+    *k = Kernel{};
+    if (!fma.empty() || tune_lookup(tune_key(p->dev, shape_key(p, what) + "|fma"), &fma)) {
+        if (fma == "default" && p->snippet.empty()) return FBCORR_OK;
+        if (parse_direct_spec(fma, t) && direct_smem_bytes(*t, pr.fh, pr.fw, pr.c) <= smem_limit(p->dev) &&
+            build_direct(pr, *t, k) == FBCORR_OK)
+            return FBCORR_OK;
+        logf("FMA variant '%s' not usable; ignoring it", fma.c_str());
+    }
+    *t = direct_heuristic(pr, smem_limit(p->dev), p->dev.sm_count);
+    return build_direct(pr, *t, k);
+}
+
+fbcorr_status_t run_fma(const Kernel& k, const DirectTile& t, const DirectProblem& pr, const float* x, const float* m,
+                        const float* w, float* y, float lo, float hi, cudaStream_t s) {
+    return k.fn ? run_direct(k, pr, t, x, m, w, y, lo, hi, s) : run_default(pr, x, m, w, y, lo, hi, s);
+}
+
+// Select the forward variant of an F32 plan from a spec string (fma: see build_fma).
+fbcorr_status_t set_fwd_spec(fbcorr_plan* p, const std::string& spec, const char* source, const std::string& fma = "") {
     if (spec == "default" && !p->snippet.empty())
         return set_error(FBCORR_ERR_UNSUPPORTED, "the prebuilt default kernel has no snippet epilogue");
     if (spec == "default") {
@@ -153,10 +175,9 @@ fbcorr_status_t set_fwd_spec(fbcorr_plan* p, const std::string& spec, const char
     if (f3_parse_spec(spec, &f3)) {
         F3Launch l;
         FBC_TRY(f3_build(pr, f3, p->dev.sm_count, &l));
-        // and the FMA kernel that calls without scratch run
-        const DirectTile dt = direct_heuristic(pr, smem_limit(p->dev), p->dev.sm_count);
+        DirectTile dt;
         Kernel k;
-        FBC_TRY(build_direct(pr, dt, &k));
+        FBC_TRY(build_fma(p, "fwd", pr, fma, &dt, &k));
         p->fwd_kind = VarKind::F32tc;
         p->fwd_f3 = l;
         p->fwd_tile = dt;
@@ -256,18 +277,16 @@ fbcorr_status_t prepare_backward(fbcorr_plan* p) {
     DirectTile ct;
     if (parse_direct_spec(spec, &ct) && direct_smem_bytes(ct, pr.fh, pr.fw, pr.c) <= smem_limit(p->dev)) t = ct;
     Kernel k;
-    fbcorr_status_t s = use_default ? FBCORR_ERR_NVRTC : build_direct(pr, t, &k);
+    F3Tile f3;
+    F3Launch l;
+    // with scratch the tensor-core kernel runs, without it the FMA kernel
+    const bool tensor = f3_parse_spec(spec, &f3) && f3_build(pr, f3, p->dev.sm_count, &l) == FBCORR_OK;
+    fbcorr_status_t s = use_default ? FBCORR_ERR_NVRTC : tensor ? build_fma(p, "dx", pr, "", &t, &k) : build_direct(pr, t, &k);
     if (s == FBCORR_OK) {
-        p->dx_kind = VarKind::Direct;
+        p->dx_kind = tensor ? VarKind::F32tc : VarKind::Direct;
         p->dx_tile = t;
         p->dx_kernel = k;
-        F3Tile f3;
-        F3Launch l;
-        // with scratch the tensor-core kernel runs, without it the FMA kernel
-        if (f3_parse_spec(spec, &f3) && f3_build(pr, f3, p->dev.sm_count, &l) == FBCORR_OK) {
-            p->dx_kind = VarKind::F32tc;
-            p->dx_f3 = l;
-        }
+        p->dx_f3 = l;
     } else if (s == FBCORR_ERR_NVRTC) {
         p->dx_kind = VarKind::Default;
     } else {
@@ -675,7 +694,7 @@ fbcorr_status_t fbcorr_forward(fbcorr_plan_t p, const float* x, const float* w, 
             if (e0) FBC_CUDA(cudaEventRecord(e0, s));
             st = ws && aligned16(ws) && ws_bytes >= p->fwd_f3.ws_bytes
                      ? f3_run(p->fwd_f3, fwd_problem(p), x, nullptr, w, y, ws, p->epi.lo, p->epi.hi, p->err_dev, s)
-                     : run_direct(p->fwd_kernel, fwd_problem(p), p->fwd_tile, x, nullptr, w, y, p->epi.lo, p->epi.hi, s);
+                     : run_fma(p->fwd_kernel, p->fwd_tile, fwd_problem(p), x, nullptr, w, y, p->epi.lo, p->epi.hi, s);
             if (e1 && st == FBCORR_OK) FBC_CUDA(cudaEventRecord(e1, s));
             return st;
         case VarKind::Tensor:
@@ -758,7 +777,7 @@ fbcorr_status_t fbcorr_backward(fbcorr_plan_t p, const float* x, const float* w,
         st = f3_dx ? f3_run(p->dx_f3, pr, g, m, w, dx, (uint8_t*)ws + dx_scratch_offset(p), p->epi.lo, p->epi.hi,
                             p->err_dev, s)
              : p->dx_kind != VarKind::Default
-                 ? run_direct(p->dx_kernel, pr, p->dx_tile, g, m, w, dx, p->epi.lo, p->epi.hi, s)
+                 ? run_fma(p->dx_kernel, p->dx_tile, pr, g, m, w, dx, p->epi.lo, p->epi.hi, s)
                  : run_default(pr, g, m, w, dx, p->epi.lo, p->epi.hi, s);
     }
     // the join even when dL/dx failed to launch: nothing on `s` may overtake dL/dw
@@ -802,17 +821,21 @@ fbcorr_status_t fbcorr_autotune(fbcorr_plan_t p, fbcorr_stream_t stream) {
     float f3_ms = 0.f;
     std::string f3;
     FBC_TRY(f3_tune(p->dev, fwd_problem(p), s, p->err_dev, &f3_ms, &f3));
+    // the fastest FMA kernel is kept as well, for calls without scratch
+    const std::string fma = best;
+    tune_store(tune_key(p->dev, shape_key(p, "fwd") + "|fma"), fma);
     if (!f3.empty() && f3_ms < ms) {
         best = f3;
         ms = f3_ms;
     }
-    FBC_TRY(set_fwd_spec(p, best, "tuned"));
+    FBC_TRY(set_fwd_spec(p, best, "tuned", fma));
     tune_store(tune_key(p->dev, shape_key(p, "fwd")), best);
     logf("autotune fwd picked %s (%.4f ms)", best.c_str(), ms);
     // dL/dx: the same generated kernel family on the flipped problem
     std::string best_dx;
     FBC_TRY(tune_direct(p, dx_problem(p), s, "dx", &best_dx, &ms));
     FBC_TRY(f3_tune(p->dev, dx_problem(p), s, p->err_dev, &f3_ms, &f3));
+    tune_store(tune_key(p->dev, shape_key(p, "dx") + "|fma"), best_dx);
     if (!f3.empty() && f3_ms < ms) {
         best_dx = f3;
         ms = f3_ms;
@@ -965,7 +988,8 @@ fbcorr_status_t fbcorr_plan_info(fbcorr_plan_t p, char* buf, size_t cap) {
         o << ",\"spec\":\"" << f3_spec(p->fwd_f3.tile) << "\",\"smem\":" << p->fwd_f3.kernel.smem << ",\"threads\":"
           << p->fwd_f3.kernel.threads << ",\"grid\":" << p->fwd_f3.grid << ",\"slots\":[" << p->fwd_f3.na << ","
           << p->fwd_f3.nb << "],\"kernel\":\"" << p->fwd_f3.kernel.name << "\",\"source_hash\":\""
-          << hex64(p->fwd_f3.kernel.src_hash) << "\"";
+          << hex64(p->fwd_f3.kernel.src_hash) << "\",\"fma\":\""
+          << (p->fwd_kernel.fn ? direct_tile_spec(p->fwd_tile) : "default") << "\"";
     } else if (p->fwd_kind == VarKind::Default) {
         o << ",\"spec\":\"default\"";
     } else if (p->tc_packed) {
@@ -981,7 +1005,9 @@ fbcorr_status_t fbcorr_plan_info(fbcorr_plan_t p, char* buf, size_t cap) {
     if (p->bwd_ready) {
         o << ",\"dx\":{\"kind\":\"" << kind_name(p->dx_kind) << "\"";
         if (p->dx_kind == VarKind::Direct) o << ",\"spec\":\"" << direct_tile_spec(p->dx_tile) << "\"";
-        if (p->dx_kind == VarKind::F32tc) o << ",\"spec\":\"" << f3_spec(p->dx_f3.tile) << "\"";
+        if (p->dx_kind == VarKind::F32tc)
+            o << ",\"spec\":\"" << f3_spec(p->dx_f3.tile) << "\",\"fma\":\""
+              << (p->dx_kernel.fn ? direct_tile_spec(p->dx_tile) : "default") << "\"";
         o << "},\"dw\":{\"kind\":\"" << kind_name(p->dw_kind) << "\",\"threads\":" << p->D * p->dw_ng
           << ",\"filters_per_cta\":" << p->dw_tn * p->dw_ng << ",\"packed_pairs\":" << p->dw_pk << ",\"min_blocks\":" << p->dw_mb
           << ",\"registers\":" << p->dw_regs << ",\"tile\":[" << p->dw_tn << "," << p->dw_ng << "," << p->dw_qb << "]"

@@ -457,3 +457,36 @@ def test_non_finite_values_cost_no_more_than_a_few_fma_kernels(shape):
         assert _us(torch, lambda: p.forward(a, b)) <= 4 * fma[0]
     for b, c in ((w1, g), (w, g1), (w, g2)):
         assert _us(torch, lambda: p.backward(x, b, c, need_dw=False)) <= 4 * fma[1]
+
+
+def test_calls_without_scratch_run_the_tuned_fma_kernels(tmp_path, monkeypatch):
+    """Where the tuner picks the tensor-core kernel, the plan, and plans made from the
+    cache, keep the FMA kernel that it measured fastest for calls without scratch."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    monkeypatch.setenv("FBCORR_CACHE_DIR", str(tmp_path))
+    monkeypatch.setenv("FBCORR_TUNE_TOPK", "2")
+    wl = inputs.random_case(7995, 200, 230, 8, 64, 7, 7, with_g=True)
+    x, w, g = dev(wl.x, torch), dev(wl.w, torch), dev(wl.g, torch)
+    p = Plan(wl.x.shape, wl.w.shape)
+    p.autotune()
+    p.backward(x, w, g, need_dw=False)
+    assert p.info()["fwd"]["kind"] == "f32tc" and p.info()["dx"]["kind"] == "f32tc"
+    path = tmp_path / "tune.tsv"
+    saved = dict(line.split("\t") for line in path.read_text().splitlines())
+    fwd, dx = (next(k for k in saved if k.endswith("|fma") and f"{what}|x" in k) for what in ("fwd", "dx"))
+    assert p.info()["fwd"]["fma"] == saved[fwd] and p.info()["dx"]["fma"] == saved[dx]
+    # other kernels in the cache are the ones that run: their bits, without scratch
+    small = torch.empty(16, dtype=torch.uint8, device="cuda")
+    for fma in ({fwd: "direct:tr=2,tf=4,wr=4,wf=2,cc=0,pk=1", dx: "direct:tr=2,tf=4,wr=2,wf=2,cc=16,pk=1"},
+                {fwd: "default", dx: "default"}):
+        path.write_text("".join(f"{k}\t{fma.get(k, v)}\n" for k, v in saved.items()))
+        q = Plan(wl.x.shape, wl.w.shape)
+        assert q.info()["fwd"]["source"] == "cache" and q.info()["fwd"]["kind"] == "f32tc"
+        y, gx = q.forward(x, w, ws=small), q.backward(x, w, g, need_dw=False, ws=small)[0]
+        assert q.info()["fwd"]["fma"] == fma[fwd] and q.info()["dx"]["fma"] == fma[dx]
+        monkeypatch.setenv("FBCORR_DX_VARIANT", fma[dx])
+        r = Plan(wl.x.shape, wl.w.shape)
+        r.set_variant(fma[fwd])
+        assert torch.equal(y, r.forward(x, w)) and torch.equal(gx, r.backward(x, w, g, need_dw=False)[0])
+        monkeypatch.delenv("FBCORR_DX_VARIANT")
