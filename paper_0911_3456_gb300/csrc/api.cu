@@ -1112,6 +1112,8 @@ fbcorr_status_t fbcorr_rtcg_check(const int64_t in_shape[3], const int64_t filt_
             if (ranked.empty())
                 return set_error(FBCORR_ERR_UNSUPPORTED, "the FP32 tensor-core kernel does not take this shape");
             const F3Tile ft = pr == &fp && sp != "f32tc" ? f3 : ranked.front();
+            if (f3_ws_bytes(*pr, ft) == 0)     // before anything is derived from the tile
+                return set_error(FBCORR_ERR_UNSUPPORTED, "variant %s does not fit this shape", f3_spec(ft).c_str());
             std::string lg;
             const fbcorr_status_t st = rtcg_compile_only(f3_kernel_source(*pr, ft, f3_kernel_name(*pr, ft)), &lg);
             if (st != FBCORR_OK) {

@@ -65,11 +65,12 @@ bool layout(const DirectProblem& pr, const F3Tile& t, int* na, int* nb, size_t* 
         return false;
     if (t.gc != 8 && t.gc != 16 && t.gc != 32) return false;
     if (t.gc > 8 && pr.c <= 4) return false;
-    if (t.r > 1 && t.r * pr.nf > t.nt) return false;
+    if (t.r > 1 && (long long)t.r * pr.nf > t.nt) return false;
+    if (t.ru > pr.fh + t.r - 1) return false;
     // 32-bit pixel indices, with room for a slab past the last tile
     if ((pixel_tiles(pr, t) + 1) * 128 + 4096 >= (1ll << 31)) return false;
     const Geometry g = geometry(pr, t);
-    if (t.ru > g.rows || g.ka > 18 || g.bank_chunks >= (1ll << 30)) return false;
+    if (g.ka > 18 || g.bank_chunks >= (1ll << 30)) return false;
     for (int want : {4, 3})
         for (int a = 6; a >= 3; --a) {
             const long room = (long)kSmemMax - kBarBytes - (long)(a * g.aslot);

@@ -1,5 +1,8 @@
 """The FP32 tensor-core kernels compile for sm_103a (no GPU)."""
 import ctypes
+import os
+import subprocess
+import sys
 
 import pytest
 
@@ -17,3 +20,20 @@ def test_rtcg_check(shape, spec, ok):
     st = C.load().fbcorr_rtcg_check(C.I64_3(*shape[0]), C.I64_4(*shape[1]), C.epilogue((0.0, 1.0)), spec.encode(), log,
                                     len(log))
     assert (st == 0) == ok, log.value.decode()
+
+
+@pytest.mark.parametrize("fields", ["nt=64,r=4,gc=8,jt=0,ru=2", "nt=64,r=4,gc=8,jt=9,ru=0", "nt=64,r=4,gc=0,jt=9,ru=2",
+                                    "nt=0,r=4,gc=8,jt=9,ru=2", "nt=64,r=0,gc=8,jt=9,ru=2", "nt=-64,r=4,gc=8,jt=9,ru=2",
+                                    "nt=64,r=4,gc=8,jt=-1,ru=2", "nt=64,r=-4,gc=8,jt=9,ru=2", "nt=64,r=4,gc=-8,jt=9,ru=2",
+                                    "nt=64,r=4,gc=8,jt=9,ru=-2", "nt=96,r=4,gc=8,jt=9,ru=2", "nt=72,r=4,gc=8,jt=9,ru=2",
+                                    "nt=64,r=5,gc=8,jt=9,ru=2", "nt=64,r=268435456,gc=8,jt=9,ru=2", "nt=64,r=4,gc=12,jt=9,ru=2",
+                                    "nt=64,r=4,gc=8,jt=10,ru=2", "nt=64,r=4,gc=8,jt=2000000000,ru=2",
+                                    "nt=64,r=4,gc=8,jt=9,ru=13", "nt=64,r=4,gc=8,jt=9,ru=2000000000"])
+def test_rtcg_check_refuses_tiles_that_no_plan_takes(fields):
+    """In a child process: a tile of zeros once divided by zero on the host."""
+    code = ("from paper_0911_3456_gb300 import _capi as C; "
+            "print(C.load().fbcorr_rtcg_check(C.I64_3(128, 128, 8), C.I64_4(16, 9, 9, 8), C.epilogue(None), "
+            f"b'f32tc:{fields}', None, 0))")
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=120,
+                       cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert r.returncode == 0 and r.stdout.strip() == "3", r.stderr       # FBCORR_ERR_UNSUPPORTED
