@@ -355,7 +355,9 @@ fbcorr_status_t fbcorr_fp32_fma_probe(int packed, int iters, double* tflops, dou
  * with the forward tile `spec` ("heuristic" or a "direct:..." spec; a chunked
  * K-split spec -- ks with cc > 0 -- is a dL/dx tile and replaces the dL/dx
  * heuristic instead, FBCORR_ERR_UNSUPPORTED where the shape's dL/dx cannot take
- * it: a clamp epilogue, or a depth or filter count not a multiple of 4); or, for a
+ * it: a clamp epilogue, or a depth or filter count not a multiple of 4); or, for
+ * "f32tc" (the heuristic's tile) or a "f32tc:nt=..,r=..,gc=..,jt=..,ru=.." spec, the
+ * FP32 tensor-core kernels of the three passes; or, for a
  * "tcgen05:na=..,nb=..,nt=..,bt=..,ew=..,fz=.." spec, the tensor-core kernel
  * that spec generates for this depth and filter width, in both BF16 and split
  * BF16 form.  Needs no GPU.  On failure the NVRTC log (or the reason the spec
@@ -372,8 +374,9 @@ fbcorr_status_t fbcorr_snippet_check(const int64_t in_shape[3], const int64_t fi
                                      fbcorr_dtype_t dtype, const char* expr, char* log, size_t cap);
 
 /* The same offline check for a batch plan: generate and compile (without
- * loading) the single persistent kernel that fbcorr_batch_plan_create would
- * build for these n images.  Needs no GPU. */
+ * loading) the tensor-core kernels that fbcorr_batch_plan_create would build for
+ * these n images, and the persistent kernel that takes all of them where there is
+ * no memory for the former's scratch.  Needs no GPU. */
 fbcorr_status_t fbcorr_batch_rtcg_check(int n, const int64_t (*in_shapes)[3],
                                         const int64_t (*filt_shapes)[4], fbcorr_epilogue_t epilogue,
                                         char* log, size_t cap);

@@ -1106,7 +1106,8 @@ fbcorr_status_t fbcorr_rtcg_check(const int64_t in_shape[3], const int64_t filt_
     const DirectProblem fp = fwd_problem(&tmp), bp = dx_problem(&tmp);
     F3Tile f3;
     if (f3_parse_spec(sp, &f3) || sp == "f32tc") {
-        // the FP32 tensor-core kernels of the forward (this tile, or the heuristic's) and of dL/dx
+        // the FP32 tensor-core kernels of the forward (this tile, or the heuristic's), of
+        // dL/dx, and of dL/dw where a plan runs it
         for (const DirectProblem* pr : {&fp, &bp}) {
             const std::vector<F3Tile> ranked = f3_ranked(*pr, 152, nullptr);
             if (ranked.empty())
@@ -1121,7 +1122,12 @@ fbcorr_status_t fbcorr_rtcg_check(const int64_t in_shape[3], const int64_t filt_
                 return st;
             }
         }
-        return FBCORR_OK;
+        F3DwTile dt;
+        if (!f3dw_wins(dw_problem(&tmp), 152, &dt)) return FBCORR_OK;
+        std::string name, lg;
+        const fbcorr_status_t st = rtcg_compile_only(f3dw_kernel_source(dw_problem(&tmp), dt, &name), &lg);
+        if (st != FBCORR_OK && log && cap) snprintf(log, cap, "%s", lg.c_str());
+        return st;
     }
     DirectTile t;
     if (sp == "heuristic")

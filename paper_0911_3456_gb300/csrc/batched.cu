@@ -260,12 +260,11 @@ size_t batch_smem(const fbcorr_batch_plan* b) {
     return smem;
 }
 
-// The images that run on the tensor cores, their kernels (compiled in parallel)
-// and scratch, largest first.
-fbcorr_status_t build_f3(fbcorr_batch_plan* b) {
-    if (env_str("FBCORR_BATCH_KS", "0") == "1") return FBCORR_OK;   // the K-split tiles are asked for
-    const int epi = b->epi.kind == FBCORR_EPI_CLAMP ? 1 : 0;
+// The images that run on the tensor cores, into b->f3, and the sources of their kernels.
+std::vector<std::string> choose_f3(fbcorr_batch_plan* b) {
     std::vector<std::string> srcs;
+    if (env_str("FBCORR_BATCH_KS", "0") == "1") return srcs;   // the K-split tiles are asked for
+    const int epi = b->epi.kind == FBCORR_EPI_CLAMP ? 1 : 0;
     for (int k = 0; k < b->n; ++k) {
         const auto& s = b->shp[k];
         BatchF3 f;
@@ -276,6 +275,12 @@ fbcorr_status_t build_f3(fbcorr_batch_plan* b) {
         srcs.push_back(f3_kernel_source(f.pr, f.l.tile, f3_kernel_name(f.pr, f.l.tile)));
         b->f3.push_back(f);
     }
+    return srcs;
+}
+
+// Their kernels (compiled in parallel) and scratch, largest first.
+fbcorr_status_t build_f3(fbcorr_batch_plan* b) {
+    const std::vector<std::string> srcs = choose_f3(b);
     if (b->f3.empty()) return FBCORR_OK;
     rtcg_precompile(srcs);
     size_t bytes = 0;
@@ -475,11 +480,23 @@ fbcorr_status_t fbcorr_batch_rtcg_check(int n, const int64_t (*in_shapes)[3],
     for (int k = 0; k < n; ++k)
         tmp.shp.push_back({in_shapes[k][0], in_shapes[k][1], in_shapes[k][2], filt_shapes[k][0],
                            filt_shapes[k][1], filt_shapes[k][2]});
+    // the tensor-core images' kernels, and the persistent kernel of every image (which
+    // takes them all where there is no memory for the former's scratch)
+    std::vector<std::string> srcs = choose_f3(&tmp);
+    std::sort(srcs.begin(), srcs.end());
+    srcs.erase(std::unique(srcs.begin(), srcs.end()), srcs.end());
+    tmp.f3.clear();
     FBC_TRY(select_variants(&tmp, false));
-    std::string lg;
-    fbcorr_status_t s = rtcg_compile_only(batch_source(&tmp), &lg);
-    if (s != FBCORR_OK && log && cap) snprintf(log, cap, "%s", lg.c_str());
-    return s;
+    srcs.push_back(batch_source(&tmp));
+    for (const std::string& src : srcs) {
+        std::string lg;
+        const fbcorr_status_t s = rtcg_compile_only(src, &lg);
+        if (s != FBCORR_OK) {
+            if (log && cap) snprintf(log, cap, "%s", lg.c_str());
+            return s;
+        }
+    }
+    return FBCORR_OK;
 }
 
 fbcorr_status_t fbcorr_batch_plan_destroy(fbcorr_batch_plan_t b) {

@@ -104,7 +104,7 @@ bool f3dw_wins(const DirectProblem& pr, int sm_count, F3DwTile* out) {
     return sw == "force" || best + 5000 < 0.9 * (flops / (sm_count * 256 * eff) + 4000);
 }
 
-fbcorr_status_t f3dw_build(const DirectProblem& pr, const F3DwTile& t, F3DwLaunch* out) {
+std::string f3dw_kernel_source(const DirectProblem& pr, const F3DwTile& t, std::string* kname) {
     const DwGeometry g = geometry(pr, t);
     char name[160];
     snprintf(name, sizeof name, "fbc_f32dw_f%dx%d_c%d_n%d_m%d_t%d_%d_%d_%d", pr.fh, pr.fw, pr.c, pr.nf, pr.mask, t.nb, t.ncomb,
@@ -120,9 +120,17 @@ fbcorr_status_t f3dw_build(const DirectProblem& pr, const F3DwTile& t, F3DwLaunc
       << " && FbcF3Dw::NS == " << g.ns << " && 2 * FbcF3Dw::BUF <= 512, \"host and device disagree on the geometry\");\n";
     o << "extern \"C\" __global__ void __launch_bounds__(" << FBC_F3DW_THREADS << ", 1) " << name
       << "(const __grid_constant__ FbcF3DwParams P) {\n  fbc_f32dw_body<FbcF3Dw>(P);\n}\n";
+    *kname = name;
+    return o.str();
+}
+
+fbcorr_status_t f3dw_build(const DirectProblem& pr, const F3DwTile& t, F3DwLaunch* out) {
+    const DwGeometry g = geometry(pr, t);
+    std::string name;
+    const std::string src = f3dw_kernel_source(pr, t, &name);
     F3DwLaunch l;
     l.tile = t;
-    FBC_TRY(rtcg_kernel(o.str(), name, g.ns * g.slot, FBC_F3DW_THREADS, &l.kernel));
+    FBC_TRY(rtcg_kernel(src, name, g.ns * g.slot, FBC_F3DW_THREADS, &l.kernel));
     l.grid = (int)(combos(pr, t) * t.splits);
     l.parts = t.splits * g.nh;
     l.ws_bytes = f3dw_ws_bytes(pr, t);

@@ -287,6 +287,7 @@ struct F3DwLaunch {
 };
 bool f3dw_wins(const DirectProblem& pr, int sm_count, F3DwTile* t);
 size_t f3dw_ws_bytes(const DirectProblem& pr, const F3DwTile& t);
+std::string f3dw_kernel_source(const DirectProblem& pr, const F3DwTile& t, std::string* name);
 fbcorr_status_t f3dw_build(const DirectProblem& pr, const F3DwTile& t, F3DwLaunch* out);
 // *part: l.parts partial sums per element; *flags: l.grid flags, any set where the
 // result has to come from the FMA kernel.

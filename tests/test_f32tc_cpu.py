@@ -37,3 +37,27 @@ def test_rtcg_check_refuses_tiles_that_no_plan_takes(fields):
     r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=120,
                        cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
     assert r.returncode == 0 and r.stdout.strip() == "3", r.stderr       # FBCORR_ERR_UNSUPPORTED
+
+
+def _kernels(directory):
+    text = "".join(f.read_text() for f in directory.iterdir())
+    return {name for name in ("fbc_f32tc_", "fbc_f32dw_", "fbc_batch(") if f") {name}" in text}, text
+
+
+def test_rtcg_check_compiles_the_kernels_of_all_three_passes(tmp_path, monkeypatch):
+    monkeypatch.setenv("FBCORR_DUMP_DIR", str(tmp_path))
+    assert C.load().fbcorr_rtcg_check(C.I64_3(128, 140, 8), C.I64_4(64, 9, 9, 8), C.epilogue((0.0, 1.0)), b"f32tc", None,
+                                      0) == 0
+    names, text = _kernels(tmp_path)
+    assert names == {"fbc_f32tc_", "fbc_f32dw_"} and "fl0_e1_m0" in text and "fl1_e0_m1" in text
+
+
+def test_batch_rtcg_check_compiles_the_tensor_core_kernels(tmp_path, monkeypatch):
+    monkeypatch.setenv("FBCORR_DUMP_DIR", str(tmp_path))
+    shapes = [(200, 210, 8, 64, 7, 7), (12, 12, 3, 5, 2, 2), (200, 210, 8, 64, 7, 7)]
+    ins = (ctypes.c_int64 * 9)(*[v for s in shapes for v in s[:3]])
+    fls = (ctypes.c_int64 * 12)(*[v for s in shapes for v in (s[3], s[4], s[5], s[2])])
+    assert C.load().fbcorr_batch_rtcg_check(3, ins, fls, C.epilogue(None), None, 0) == 0
+    names, text = _kernels(tmp_path)
+    assert names == {"fbc_f32tc_", "fbc_batch("} and len(list(tmp_path.iterdir())) == 2
+    assert text.count("FbcV0") and text.count("FbcV1")     # the persistent kernel holds every image
