@@ -1,10 +1,15 @@
-"""The FP32 tensor-core kernels compile for sm_103a (no GPU)."""
+"""The FP32 tensor-core kernels without a GPU: they compile for sm_103a, and what the
+accuracy tests ask of them is sharp enough."""
 import ctypes
 import os
 import subprocess
 import sys
 
+import numpy as np
 import pytest
+
+import f32split
+import oracle
 
 from paper_0911_3456_gb300 import _capi as C
 
@@ -61,3 +66,34 @@ def test_batch_rtcg_check_compiles_the_tensor_core_kernels(tmp_path, monkeypatch
     names, text = _kernels(tmp_path)
     assert names == {"fbc_f32tc_", "fbc_batch("} and len(list(tmp_path.iterdir())) == 2
     assert text.count("FbcV0") and text.count("FbcV1")     # the persistent kernel holds every image
+
+
+@pytest.mark.parametrize("positive", [False, True])
+@pytest.mark.parametrize("which", ["forward", "dx", "dw"])
+def test_the_accuracy_question_tells_the_three_way_split_from_less(which, positive):
+    """The bound that the GPU tests put on the kernels' errors holds for the six products
+    that they keep and fails for a kernel that leaves the third order out (of random
+    signs: in sums of one sign that order averages out)."""
+    rng = np.random.default_rng(11)
+    for case in {"forward": f32split.FORWARD, "dx": f32split.GRADIENT, "dw": f32split.BANK}[which]:
+        x, w, g = f32split.layer(rng, case if which == "dw" else case[0], positive)
+        op, a, b = {"forward": (oracle.fwd, x, w),
+                    "dx": (lambda u, v: oracle.bwd_input(u, v, x.shape), g, w),
+                    "dw": (lambda u, v: oracle.bwd_filt(u, v, w.shape), x, g)}[which]
+        ref = op(a, b)
+        assert f32split.rel2(f32split.six_products(op, a, b), ref) <= 2.0 ** -24
+        if not positive:
+            assert f32split.rel2(f32split.six_products(op, a, b, 2), ref) > f32split.NORMWISE
+
+
+def test_left_out_products_are_below_two_to_the_minus_24():
+    """x2 w3 and x3 w2 are below 2^-25 of |x w| each, and all three products together
+    below 2^-24 (not 2^-26: x = w = 1.0038986 leaves out 2^-24.01)."""
+    rng = np.random.default_rng(12)
+    x = np.concatenate([rng.uniform(1, 2, 200000).astype(np.float32), np.float32([1.0038986, 1.00390619, 1.0039])])
+    w = np.concatenate([rng.uniform(1, 2, 200000).astype(np.float32), np.float32([1.0038986, 1.00390619, 1.0039])])
+    (_, x2, x3), (_, w2, w3) = ([p.astype(np.float64) for p in f32split.split3(v)] for v in (x, w))
+    xw = x.astype(np.float64) * w
+    assert np.all(np.abs(x2 * w3) < 2.0 ** -25 * xw) and np.all(np.abs(x3 * w2) < 2.0 ** -25 * xw)
+    left = np.abs(x2 * w3 + x3 * w2 + x3 * w3)
+    assert np.all(left < 2.0 ** -24 * xw) and left[-3] > 2.0 ** -24.1 * xw[-3]

@@ -8,6 +8,7 @@ below 2^-26: |error| <= (16 * 2^-23 + (chunks + 4) * 2^-24) * sum |x| |w|.
 import numpy as np
 import pytest
 
+import f32split
 import oracle
 from paper_0911_3456_gb300 import inputs
 from helpers import dev, host, torch_cuda
@@ -490,3 +491,99 @@ def test_calls_without_scratch_run_the_tuned_fma_kernels(tmp_path, monkeypatch):
         r.set_variant(fma[fwd])
         assert torch.equal(y, r.forward(x, w)) and torch.equal(gx, r.backward(x, w, g, need_dw=False)[0])
         monkeypatch.delenv("FBCORR_DX_VARIANT")
+
+
+def _three_passes(torch, which, x, w, g, spec, monkeypatch):
+    """The pass on the tensor cores, the same on the FMA kernel, and the oracle's."""
+    from paper_0911_3456_gb300.api import Plan
+    xd, wd, gd = dev(x, torch), dev(w, torch), dev(g, torch)
+    if which == "forward":
+        p = Plan(x.shape, w.shape)
+        p.set_variant(spec)
+        out = p.forward(xd, wd), p.forward(xd, wd, ws=torch.empty(16, dtype=torch.uint8, device="cuda"))
+        ref = oracle.fwd(x, w)
+    elif which == "dx":
+        monkeypatch.setenv("FBCORR_DX_VARIANT", spec)
+        p = Plan(x.shape, w.shape)
+        out = [p.backward(xd, wd, gd, need_dw=False, ws=ws)[0] for ws in
+               (None, torch.empty(16, dtype=torch.uint8, device="cuda"))]
+        assert p.info()["dx"]["spec"] == spec
+        ref = oracle.bwd_input(g, w, x.shape)
+    else:
+        monkeypatch.setenv("FBCORR_F32TC", "force")
+        p = Plan(x.shape, w.shape)
+        out = [p.backward(xd, wd, gd, need_dx=False, ws=ws)[1] for ws in (None, p.workspace(p.ws_bwd, xd.device))]
+        assert "f32tc" in p.info()["dw"]
+        ref = oracle.bwd_filt(x, g, w.shape)
+    assert p.device_status() == 0
+    return host(out[0]), host(out[1]), ref
+
+
+ACCURACY = ([("forward", s, t) for s, t in f32split.FORWARD] + [("dx", s, t) for s, t in f32split.GRADIENT] +
+            [("dw", s, None) for s in f32split.BANK])
+
+
+@pytest.mark.parametrize("positive", [False, True], ids=["signs", "positive"])
+@pytest.mark.parametrize("which,shape,spec", ACCURACY)
+def test_normwise_error_is_that_of_the_three_way_split(which, shape, spec, positive, monkeypatch):
+    """A bound that a kernel without the third order breaks (tests/test_f32tc_cpu.py), and
+    no more than twice the FMA kernel's error on the same values of random signs (sums of
+    a few products may be exact there: one rounding of 2^-24 beside it).  In sums of one
+    sign the truncations of a chunk do not average out."""
+    torch = torch_cuda()
+    x, w, g = f32split.layer(np.random.default_rng(8000), shape, positive)
+    got, fma, ref = _three_passes(torch, which, x, w, g, spec, monkeypatch)
+    err = f32split.rel2(got, ref)
+    assert err <= f32split.NORMWISE
+    if not positive:
+        assert err <= 2 * f32split.rel2(fma, ref) + 2.0 ** -24
+
+
+@pytest.mark.parametrize("which,shape,spec", ACCURACY)
+def test_24_bit_values_pass_unchanged(which, shape, spec, monkeypatch):
+    """Each sum holds one product with a power of two: every bit of the other factor comes
+    through, whichever operand it is in."""
+    torch = torch_cuda()
+    rng = np.random.default_rng(8100)
+    H, W, D, N, fh, fw = shape
+    x, w, g = f32split.layer(rng, shape)
+
+    def power():
+        return np.float32(2.0 ** rng.integers(-3, 4)) * rng.choice(np.array([-1, 1], np.float32))
+
+    def one_per_sum(op):
+        """One operand with at most one non-zero value in each sum."""
+        if op == "w_forward":                                  # one weight per filter
+            v = np.zeros_like(w)
+            for n in range(N):
+                v[n, rng.integers(fh), rng.integers(fw), rng.integers(D)] = power()
+        elif op == "x_forward":                                # pixels a filter apart
+            v = np.zeros_like(x)
+            for i in range(0, H, fh):
+                for j in range(0, W, fw):
+                    v[i, j, rng.integers(D)] = power()
+        elif op == "w_dx":                                     # one weight per channel
+            v = np.zeros_like(w)
+            for d in range(D):
+                v[rng.integers(N), rng.integers(fh), rng.integers(fw), d] = power()
+        elif op == "g_dx":                                     # gradients a filter apart
+            v = np.zeros_like(g)
+            for i in range(0, g.shape[0], fh):
+                for j in range(0, g.shape[1], fw):
+                    v[i, j, rng.integers(N)] = power()
+        elif op == "x_dw":                                     # one pixel per channel
+            v = np.zeros_like(x)
+            for d in range(D):
+                v[rng.integers(H), rng.integers(W), d] = power()
+        else:                                                  # one gradient per filter
+            v = np.zeros_like(g)
+            for n in range(N):
+                v[rng.integers(g.shape[0]), rng.integers(g.shape[1]), n] = power()
+        return v
+
+    for op in {"forward": ("w_forward", "x_forward"), "dx": ("w_dx", "g_dx"), "dw": ("x_dw", "g_dw")}[which]:
+        args = [one_per_sum(op) if op[0] == name else v for name, v in (("x", x), ("w", w), ("g", g))]
+        got, _, ref = _three_passes(torch, which, *args, spec, monkeypatch)
+        assert np.count_nonzero(ref) > 0
+        # dL/dw adds first and third parts before the second: 25 bits where the first was rounded up
+        assert np.all(np.abs(got - ref) <= 2.0 ** -23 * np.abs(ref)) if op == "x_dw" else np.array_equal(got, ref)
