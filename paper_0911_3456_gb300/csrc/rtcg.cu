@@ -208,18 +208,21 @@ void dump_source(const std::string& src, const std::string& name) {
     fclose(f);
 }
 
-fbcorr_status_t rtcg_compile_only(const std::string& src, std::string* log) {
-    std::vector<char> cubin;
-    dump_source(src, "check_" + std::to_string(fnv1a(src) & 0xffffff));
-    return compile(src, &cubin, log);
-}
-
 namespace {
 uint64_t source_hash(const std::string& src) {
     std::string keysrc = src + "\n//" + kArch + " nvrtc " + nvrtc_version_string();
     for (auto& o : nvrtc_options()) keysrc += " " + o;
     return fnv1a(keysrc);
 }
+}  // namespace
+
+fbcorr_status_t rtcg_compile_only(const std::string& src, std::string* log) {
+    std::vector<char> cubin;
+    dump_source(src, "check_" + hex64(source_hash(src)));
+    return compile(src, &cubin, log);
+}
+
+namespace {
 
 std::string cubin_path(uint64_t h) {
     char hb[32];

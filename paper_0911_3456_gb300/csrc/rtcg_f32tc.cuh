@@ -82,6 +82,36 @@
 #define FBC_F3_DROP 0
 #endif
 
+// The PTX that the FP32 kernels alone use (the rest: rtcg_ptx.cuh, which is part of
+// every kernel's source and of the hash that measured traffic is filed under).
+// mbarrier test of a phase without a wait.
+__device__ __forceinline__ bool fbc_mbar_test(fbc_u32 bar, fbc_u32 parity) {
+    fbc_u32 ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        " selp.b32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
+// tcgen05.ld 32x32b.x8 -- 32 TMEM lanes x 8 columns, one accumulator row per thread.
+__device__ __forceinline__ void fbc_tmem_ld32x32b_x8_async(fbc_u32 taddr, fbc_u32 (&r)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+}
+
+__device__ __forceinline__ void fbc_reg_fence8(fbc_u32 (&r)[8]) {
+    asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]));
+}
+
+// 8-byte shared store.
+__device__ __forceinline__ void fbc_st_shared_v2(fbc_u32 addr, fbc_u32 a, fbc_u32 b) {
+    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
+}
+
 // tcgen05.mma with the descriptors as low and high words.
 __device__ __forceinline__ void fbc_umma_lo(fbc_u32 d, fbc_u32 alo, fbc_u32 ahi, fbc_u32 blo, fbc_u32 bhi, fbc_u32 idesc,
                                             fbc_u32 accumulate) {

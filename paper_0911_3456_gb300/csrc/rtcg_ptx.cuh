@@ -44,18 +44,6 @@ __device__ __forceinline__ bool fbc_mbar_try_wait(fbc_u32 bar, fbc_u32 parity) {
     return ok != 0;
 }
 
-// The same test without a wait.
-__device__ __forceinline__ bool fbc_mbar_test(fbc_u32 bar, fbc_u32 parity) {
-    fbc_u32 ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-        " selp.b32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
 __device__ __forceinline__ void fbc_mbar_arrive(fbc_u32 bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
@@ -177,13 +165,6 @@ __device__ __forceinline__ void fbc_tmem_ld32x32b_x32_async(fbc_u32 taddr, fbc_u
         : "r"(taddr));
 }
 
-// tcgen05.ld 32x32b.x8 -- 32 TMEM lanes x 8 columns, one accumulator row per thread.
-__device__ __forceinline__ void fbc_tmem_ld32x32b_x8_async(fbc_u32 taddr, fbc_u32 (&r)[8]) {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-}
-
 __device__ __forceinline__ void fbc_tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 __device__ __forceinline__ void fbc_reg_fence(fbc_u32 (&r)[32]) {
@@ -191,10 +172,6 @@ __device__ __forceinline__ void fbc_reg_fence(fbc_u32 (&r)[32]) {
     for (int q = 0; q < 4; ++q)
         asm volatile("" : "+r"(r[8 * q]), "+r"(r[8 * q + 1]), "+r"(r[8 * q + 2]), "+r"(r[8 * q + 3]),
                      "+r"(r[8 * q + 4]), "+r"(r[8 * q + 5]), "+r"(r[8 * q + 6]), "+r"(r[8 * q + 7]));
-}
-
-__device__ __forceinline__ void fbc_reg_fence8(fbc_u32 (&r)[8]) {
-    asm volatile("" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]));
 }
 
 // Streaming 8-byte store.
@@ -206,11 +183,6 @@ __device__ __forceinline__ void fbc_st_cs_f2(float* p, float a, float b) {
 __device__ __forceinline__ void fbc_st_shared_v4(fbc_u32 addr, fbc_u32 a, fbc_u32 b, fbc_u32 c, fbc_u32 d) {
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d)
                  : "memory");
-}
-
-// 8-byte shared store.
-__device__ __forceinline__ void fbc_st_shared_v2(fbc_u32 addr, fbc_u32 a, fbc_u32 b) {
-    asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
 
 __device__ __forceinline__ uint4 fbc_ld_shared_v4(fbc_u32 addr) {

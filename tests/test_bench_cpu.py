@@ -60,3 +60,20 @@ def test_cpu_baseline_reports_an_extrapolated_single_core_figure():
     assert one["value"] > 0 and "extrapolated" in one["note"]
     assert abs(one["whole_output_seconds_extrapolated"] - one["seconds"] / one["rows"] * wl.out_shape[0]) < 1e-9
     assert oracle.max_threads() == before          # the oracle's thread count is restored
+
+
+def test_measured_traffic_belongs_to_the_present_kernels(tmp_path, monkeypatch):
+    """Every entry of profiles/traffic.json is filed under the hash of a source that the
+    library generates now, so the bench finds it."""
+    import json
+    from paper_0911_3456_gb300 import _capi as C
+    monkeypatch.setenv("FBCORR_DUMP_DIR", str(tmp_path))
+    with open(os.path.join(ROOT, "profiles", "traffic.json")) as f:
+        entries = json.load(f)
+    for spec in {e["spec"] for e in entries.values()}:
+        assert C.load().fbcorr_rtcg_check(C.I64_3(512, 512, 32), C.I64_4(256, 5, 5, 32), C.epilogue(), spec.encode(), None,
+                                          0) == 0
+    made = {p.stem.removeprefix("check_") for p in tmp_path.iterdir()}
+    assert entries and set(entries) <= made
+    for h, e in entries.items():
+        assert bench.measured_traffic({"fwd": {"source_hash": h}}, e["workload"])[0] == e["dram_bytes_per_launch"]
