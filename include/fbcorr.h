@@ -73,10 +73,12 @@ typedef enum {
  *  F32    : FP32 products and accumulation: FP32 FMAs on the CUDA cores, or, where
  *           it is faster and the caller passes scratch (fbcorr_plan_scratch_size),
  *           the tensor cores on an exact three-way split v = v1 + v2 + v3 into BF16
- *           (24 bits; six of the nine products, the rest below 2^-26 of x w; short
- *           sums in the tensor core added up in FP32).  Its error against 64 bits
- *           is at or below the FMA kernels'; non-finite and out-of-range values give
- *           what the FMA kernels give.
+ *           (24 bits; six of the nine products, the rest together below 2^-24 of
+ *           |x w|; short sums in the tensor core added up in FP32).  Measured error
+ *           against 64 bits on 14 shapes of 12 to 8192 products per sum (2-norm,
+ *           relative; forward and dL/dx): 3.5e-8 to 2.4e-7, the FMA kernels' 6.5e-8
+ *           to 1.6e-6.  Denormal, non-finite and overflowing values give what the
+ *           FMA kernels give, to that error.
  *  BF16   : x and w rounded to BF16 (round-to-nearest-even), BF16 x BF16
  *           products with FP32 accumulation on the tcgen05 tensor cores.
  *  BF16X3 : "split BF16": v = hi + lo with hi = bf16(v), lo = bf16(v - hi);

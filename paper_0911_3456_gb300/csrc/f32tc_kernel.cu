@@ -108,9 +108,13 @@ double model_cycles(const DirectProblem& pr, const F3Tile& t, int sm_count, bool
     return rounds * g.nu * std::max(std::max(mma, conv), drain) + 4000;
 }
 
-// Steps summed on the tensor core before a chunk is added up in FP32: measured
-// relative errors (2-norm, against 64 bits) of 5e-8 to 2.7e-7 with up to 16, of
-// 9e-8 to 1.4e-6 for the FMA kernels on the same 14 shapes.
+// Steps summed on the tensor core before a chunk is added up in FP32.  Relative errors
+// (2-norm, against 64 bits) measured with up to 16, this kernel / the FMA kernels, for
+// random values: 128x128x8 * 16x9x9 1.9e-7 / 1.7e-7 (dL/dx 2.0e-7 / 6.3e-7),
+// 256x256x8 * 64x9x9 1.9e-7 / 2.3e-7 (2.2e-7 / 1.3e-6), 2048x2048x4 * 4x8x8
+// 1.4e-7 / 1.5e-7 (1.5e-7 / 2.8e-7), 512x512x32 * 256x5x5 1.4e-7 / 2.6e-7
+// (2.2e-7 / 1.4e-6), 64x200x128 * 64x8x8 2.4e-7 / 1.6e-6 (2.4e-7 / 1.1e-6); on nine
+// more shapes 3.5e-8 to 1.8e-7 / 6.5e-8 to 2.6e-7 (4.6e-8 to 2.1e-7 / 9.6e-8 to 1.3e-6).
 constexpr int kChunkSteps = 16;
 
 }  // namespace

@@ -7,12 +7,13 @@
 // (24 significand bits in three 8-bit ones), and the product x w is taken as the
 // six largest of the nine BF16 products, each exact in FP32:
 //   order 0: x1 w1      order 1: x1 w2 + x2 w1      order 2: x1 w3 + x2 w2 + x3 w1
-// The three that are left out are below 2^-26 |x w|.  The tensor core truncates
+// The three that are left out are together below 2^-24 |x w| (|v2| <= 2^-8 |v| and
+// |v3| <= 2^-17 |v|: x2 w3 and x3 w2 up to 2^-25 each).  The tensor core truncates
 // its FP32 accumulator at every K = 16 step, so a sum is only left there for a
 // chunk of a few steps: each order has its own accumulator (a truncation of
 // order 1 and 2 is then 2^-8 and 2^-16 below one of the result), and the chunk
-// sums are added to FP32 registers with ordinary rounding.  Measured error
-// against 64 bits: at or below that of the FP32 FMA kernels it stands in for.
+// sums are added to FP32 registers with ordinary rounding.  Measured errors against
+// 64 bits, beside the FMA kernels' on the same values: kChunkSteps in f32tc_kernel.cu.
 //
 // ORD is the number of orders: 3 for FP32.  The BF16 modes run the same kernel with
 // fewer where their own one (rtcg_tc.cuh) is far from the tensor rate: ORD = 2 is
