@@ -876,7 +876,7 @@ static fbcorr_status_t autotune_tc(fbcorr_plan_t p, fbcorr_stream_t stream) {
     cudaStream_t s = (cudaStream_t)stream;
     const std::vector<std::string> specs = tc_candidates(p->tc);
     const std::string old = tc_spec(p->tc);
-    p->tc_packed = false;   // the candidates below are the plan's own kernel
+    const bool packed_before = p->tc_packed;
     float *x = nullptr, *w = nullptr, *y = nullptr;
     void* ws = nullptr;
     const size_t xb = (size_t)p->H * p->W * p->D * 4, wb = (size_t)p->N * p->fh * p->fw * p->D * 4,
@@ -887,6 +887,7 @@ static fbcorr_status_t autotune_tc(fbcorr_plan_t p, fbcorr_stream_t stream) {
         cudaGetLastError();
         return set_error(FBCORR_ERR_OOM, "autotune buffers");
     }
+    p->tc_packed = false;   // the candidates below are the plan's own kernel
     // non-zero operands: the tensor cores draw (and the clocks follow) more power
     // on real data than on zeros, so timings on zeros would favour the wrong spec
     launch_fill_pattern(x, xb / 4, 1.0f, 0x1234u, s);
@@ -957,6 +958,7 @@ static fbcorr_status_t autotune_tc(fbcorr_plan_t p, fbcorr_stream_t stream) {
     cudaFree(x); cudaFree(w); cudaFree(y); cudaFree(ws);
     if (status != FBCORR_OK || best.empty()) {
         tc_set_spec(p->tc, old);
+        p->tc_packed = packed_before;
         return status != FBCORR_OK ? status : set_error(FBCORR_ERR_INTERNAL, "no variant ran");
     }
     FBC_TRY(set_tc_spec(p, best, "tuned"));

@@ -298,9 +298,7 @@ fbcorr_status_t build_f3(fbcorr_batch_plan* b) {
         auto work = [](const DirectProblem& p) { return (double)p.out_h * p.out_w * p.nf * p.fh * p.fw * p.c; };
         return work(a.pr) > work(c.pr);
     });
-    if (cudaMalloc(&b->f3_ws, bytes) != cudaSuccess) {   // no memory: the persistent kernel takes every image
-        cudaGetLastError();
-        b->f3_ws = nullptr;
+    if (scratch_alloc((void**)&b->f3_ws, bytes) != cudaSuccess) {   // no memory: the persistent kernel takes every image
         b->f3.clear();
         return FBCORR_OK;
     }

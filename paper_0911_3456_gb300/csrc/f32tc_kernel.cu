@@ -336,11 +336,11 @@ fbcorr_status_t f3_tune(const DeviceInfo& dev, const DirectProblem& pr, cudaStre
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     fbcorr_status_t status = FBCORR_OK;
     if (cudaMalloc(&x, xn * 4) != cudaSuccess || cudaMalloc(&w, wn * 4) != cudaSuccess ||
-        cudaMalloc(&y, yn * 4) != cudaSuccess || cudaMalloc(&ws, wsn) != cudaSuccess ||
+        cudaMalloc(&y, yn * 4) != cudaSuccess || scratch_alloc(&ws, wsn) != cudaSuccess ||
         (pr.mask && cudaMalloc(&m, xn * 4) != cudaSuccess) || cudaEventCreate(&e0) != cudaSuccess ||
         cudaEventCreate(&e1) != cudaSuccess) {
         cudaGetLastError();
-        status = set_error(FBCORR_ERR_OOM, "autotune buffers");
+        logf("no memory to time the tensor-core tiles: the other variants are left");
     } else {
         launch_fill_pattern(x, xn, 1.0f, 0x1234u, s);
         launch_fill_pattern(w, wn, 0.05f, 0x5678u, s);

@@ -74,10 +74,8 @@ fbcorr_status_t setup(fbcorr_plan_t p, int bands, cudaStream_t s) {
         FBC_TRY(fbcorr_plan_scratch_size(bp, &need, nullptr));
         hp->ws_bytes = std::max(hp->ws_bytes, need);
     }
-    if (hp->ws_bytes && cudaMalloc(&hp->ws, hp->ws_bytes) != cudaSuccess) {
+    if (hp->ws_bytes && scratch_alloc(&hp->ws, hp->ws_bytes) != cudaSuccess) {
         // scratch that the bands can do without (FP32) is left out, a workspace is not
-        cudaGetLastError();
-        hp->ws = nullptr;
         hp->ws_bytes = 0;
         for (auto& kv : hp->plans) hp->ws_bytes = std::max(hp->ws_bytes, kv.second->ws_fwd);
         if (hp->ws_bytes) FBC_CUDA(cudaMalloc(&hp->ws, hp->ws_bytes));

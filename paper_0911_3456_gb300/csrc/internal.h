@@ -36,6 +36,7 @@ std::string env_str(const char* name, const char* dflt = "");
 bool log_enabled();
 void logf(const char* fmt, ...);
 bool fault_injected(const char* what);   // FBCORR_FAULT contains `what`
+cudaError_t scratch_alloc(void** p, size_t bytes);   // cudaMalloc of scratch that the caller can do without
 unsigned long long wait_bound_ns();      // FBCORR_WAIT_MS (4000) in nanoseconds, read at each call
 std::string cache_dir();                  // FBCORR_CACHE_DIR or ~/.cache/fbcorr
 

@@ -72,6 +72,15 @@ bool fault_injected(const char* what) {
     return !v.empty() && v.find(what) != std::string::npos;
 }
 
+// FBCORR_FAULT=scratchmem: as on a device without memory left.
+cudaError_t scratch_alloc(void** p, size_t bytes) {
+    const cudaError_t e = fault_injected("scratchmem") ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+    if (e == cudaSuccess) return e;
+    *p = nullptr;
+    cudaGetLastError();
+    return e;
+}
+
 unsigned long long wait_bound_ns() {
     return (unsigned long long)std::max(1LL, atoll(env_str("FBCORR_WAIT_MS", "4000").c_str())) * 1000000ull;
 }

@@ -165,3 +165,29 @@ def test_batch_dropped_copy_is_reported_and_does_not_refuse_the_next_call():
         assert good.device_status() == 0
         for it, y in zip(items, ys):
             assert np.array_equal(host(y), oracle.fwd(it.x, it.w))
+
+
+def test_no_device_memory_for_optional_scratch(tmp_path):
+    """Where the device has no memory for scratch that a call can do without (a fake of the
+    allocation that fails), tuning, batches and the host-buffer forward still run, on the
+    kernels that need none, as they did before there was such scratch."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import BatchPlan, Plan
+    wl = inputs.random_case(3600, 90, 130, 8, 32, 5, 5, kind="int")
+    x, w, ref = dev(wl.x, torch), dev(wl.w, torch), oracle.fwd(wl.x, wl.w)
+    with _env(FBCORR_FAULT="scratchmem", FBCORR_CACHE_DIR=str(tmp_path), FBCORR_TUNE_TOPK="2", FBCORR_F32TC="force"):
+        p = Plan(wl.x.shape, wl.w.shape)
+        y = p.forward_host(torch.from_numpy(wl.x), torch.from_numpy(wl.w))
+        torch.cuda.synchronize()
+        assert p.info()["fwd"]["kind"] == "f32tc" and np.array_equal(host(y), ref)
+        p.autotune()
+        assert p.info()["fwd"]["source"] == "tuned" and p.info()["fwd"]["kind"] != "f32tc"
+        assert np.array_equal(host(p.forward(x, w)), ref)
+        b = Plan(wl.x.shape, wl.w.shape, "bf16x3")
+        b.autotune()
+        assert b.info()["fwd"]["spec"].startswith("tcgen05:") and np.array_equal(host(b.forward(x, w)), ref)
+        batch = BatchPlan([wl.x.shape] * 2, [wl.w.shape] * 2)
+        assert batch.info()["tensor_images"] == 0
+        ys = batch.forward([x, x], [w, w])
+        torch.cuda.synchronize()
+        assert all(np.array_equal(host(t), ref) for t in ys)
