@@ -70,7 +70,7 @@
 // non-finite sum.  The epilogue warps only note where (a call in their loop cost
 // 2048x2048x4 * 4x8x8 a fifth in spilled registers); once the pipeline has ended, all
 // warps of the CTA compute those outputs again, in groups of 8 pixels x 8 columns, with
-// FP32 FMAs straight from global memory (fbc_f3_redo).
+// FP32 FMAs straight from global memory (fbc_f3_redo_noted).
 //
 // Every mbarrier wait is bounded in time; on expiry the kernel records an error
 // code in host-mapped memory, stops every role, waits (bounded) for its MMAs in
@@ -313,7 +313,7 @@ __device__ __forceinline__ void fbc_f3_ldg(const float* p, float (&v)[N]) {
 // products of a filter row (consecutive floats of x, and of an unflipped bank) and
 // hold four pixels x 8 columns each, so that 12 loads of 16 bytes feed 128 FMAs, with
 // 8 pixels' lines per load of x and one per load of w.  512x512x32 * 256x5x5 with one
-// NaN pixel 0.44 ms, one NaN weight 0.53, NaN all over the image 4.4 (one thread per
+// NaN pixel 0.43 ms, one NaN weight 0.53, NaN all over the image 4.5 (one thread per
 // pixel and whole tiles: 12, 63 and 304; without NaN 0.40; the FMA kernel 1.93).
 template <class G>
 __device__ __forceinline__ void fbc_f3_redo(const FbcF3Params& P, fbc_u32 mask, int pg, int q, int n0, int col0) {
@@ -411,21 +411,12 @@ __device__ __forceinline__ void fbc_f3_redo(const FbcF3Params& P, fbc_u32 mask, 
     if ((mask >> src) & 1u) fbc_f3_store8<G>(P, pg, q, n0, col0, v);
 }
 
-// Notes that warp `warp` met non-finite sums at the lanes of `mask` in its 8 columns g
-// of the CTA's item `ord`: item, warp, group, and which of the lanes' four bytes.  Items
-// for which there is no room are computed again whole, and all after them.
-#define FBC_F3_NOTES 240   // with the rest at most 1 KB of static shared memory
-__device__ __forceinline__ void fbc_f3_note(fbc_u32 mask, int ord, int warp, int g, int lane, fbc_u32* list, int* count, int* from) {
-    if (mask == 0 || lane != 0) return;
-    const int k = ord < (1 << 22) ? atomicAdd(count, 1) : FBC_F3_NOTES;
-    if (k >= FBC_F3_NOTES) {
-        atomicMin(from, ord);
-        return;
-    }
-    fbc_u32 bytes = 0;
-    for (int b = 0; b < 4; ++b) bytes |= (mask >> (8 * b) & 0xFFu) ? 1u << b : 0u;
-    list[k] = (fbc_u32)ord << 10 | (fbc_u32)warp << 7 | (fbc_u32)g << 4 | bytes;
-}
+// A note: the CTA's item and the accumulating warp (low 3 bits) that met non-finite sums,
+// and for each group of 8 columns which of its four groups of 8 pixels hold them.
+struct FbcF3Note {
+    fbc_u32 where, what;
+};
+#define FBC_F3_NOTES 120     // with the rest at most 1 KB of static shared memory
 
 // Position in a CTA's sequence of (work item, unit); item = filter tile * mtiles + pixel tile.
 template <class G>
@@ -588,12 +579,43 @@ __device__ __forceinline__ void fbc_f32tc_bank_body(const FbcF3Params& P) {
     }
 }
 
+// The noted outputs of a CTA, by every one of its warps; the items from `from` on, for
+// which there was no room, whole.  Not inlined: inlined, or noted group by group, it cost
+// the pipeline registers (512x512x32 * 256x5x5 401 instead of 392 us, split BF16
+// 256x256x8 * 64x9x9 24.2 either way, BF16 2048x2048x4 * 4x8x8 62.4 instead of 61.3).
+template <class G>
+__device__ __noinline__ void fbc_f3_redo_noted(const FbcF3Params& P0, const FbcF3Note* list, int noted, int from) {
+    const FbcF3Params P = P0;     // in registers: by reference it took half as long again
+    constexpr int NG = G::NT / 16;
+    const int lane = threadIdx.x & 31;
+    const int items = (P.nitems - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int listed = min(noted, FBC_F3_NOTES);
+    const int count = listed + (from < items ? (items - from) * 8 : 0);
+    // a group of all notes after the other: one bad filter is work for every warp
+    int g = 0, e = threadIdx.x >> 5;
+#pragma unroll 1
+    for (;; e += FBC_F3_THREADS / 32) {
+        for (; e >= count && g < NG; ++g) e -= count;
+        if (g >= NG) break;
+        // beyond the list: every warp's part of an item
+        const fbc_u32 where = e < listed ? list[e].where : (fbc_u32)(from * 8 + e - listed);
+        const fbc_u32 bytes = e < listed ? list[e].what >> (4 * g) & 0xFu : 0xFu;
+        if (bytes == 0) continue;
+        const int item = (int)(blockIdx.x + (where >> 3) * gridDim.x), wq = (int)where & 7;
+        const int v = (item % P.mtiles) * 128 + (wq & 3) * 32 + lane;
+        const int pg = fbc_f3_row(v, P), q = v - pg * P.vw;
+        const bool inside = q < P.out_w && pg * G::R < P.out_h && ((bytes >> (lane >> 3)) & 1u);
+        const fbc_u32 mask = __ballot_sync(0xFFFFFFFFu, inside);
+        fbc_f3_redo<G>(P, mask, pg, q, G::R > 1 ? 0 : item / P.mtiles * G::NT, (wq >> 2) * (G::NT / 2) + 8 * g);
+    }
+}
+
 template <class G>
 __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
     __shared__ int s_abort;
     __shared__ fbc_u32 s_tmem;
-    __shared__ fbc_u32 s_bad[FBC_F3_NOTES];   // groups of outputs with a non-finite sum, and how many
-    __shared__ int s_nbad, s_bad_from;        // (from item s_bad_from on they found no room)
+    __shared__ FbcF3Note s_bad[FBC_F3_NOTES];   // where sums were not finite, and how often that was noted
+    __shared__ int s_nbad, s_bad_from;          // (from item s_bad_from on there was no room)
     const int warp = threadIdx.x >> 5;
     const int lane = threadIdx.x & 31;
     const fbc_u32 sbase = fbc_smem_addr(fbc_tc_smem);
@@ -881,12 +903,19 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
                 out[k] = G::ORD == 3 ? sum[k] * FBC_F3_DOWN : sum[k];
             }
             if (__any_sync(0xFFFFFFFFu, inside && !(z == 0.f))) {
+                fbc_u32 bad = 0;
 #pragma unroll
                 for (int g = 0; g < NG; ++g) {
                     z = 0.f;
 #pragma unroll
                     for (int k = 8 * g; k < 8 * g + 8; ++k) z += out[k] - out[k];
-                    fbc_f3_note(__ballot_sync(0xFFFFFFFFu, inside && !(z == 0.f)), ord, warp, g, lane, s_bad, &s_nbad, &s_bad_from);
+                    bad |= inside && !(z == 0.f) ? 1u << (4 * g) : 0u;
+                }
+                bad = __reduce_or_sync(0xFFFFFFFFu, bad << (lane >> 3));
+                if (lane == 0) {
+                    const int k = atomicAdd(&s_nbad, 1);
+                    if (k < FBC_F3_NOTES) s_bad[k] = FbcF3Note{(fbc_u32)ord << 3 | (fbc_u32)warp, bad};
+                    else atomicMin(&s_bad_from, ord);
                 }
             }
             o_next = inside ? 0 : NG;
@@ -900,23 +929,6 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
     fbc_tc_fence_after();
     if (warp == 15)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(G::TMEM));
-    // the noted groups, by every warp: the stores above came before the barrier
-    if (s_abort) return;
-    constexpr int NG = G::NT / 16;
-    const int listed = min(s_nbad, FBC_F3_NOTES), from = s_bad_from;
-    const int items = (P.nitems - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
-    const long long all = listed + (from < items ? (long long)(items - from) * 8 * NG : 0);
-#pragma unroll 1
-    for (long long k = warp; k < all; k += FBC_F3_THREADS / 32) {
-        const long long past = k - listed;     // beyond the list: every group of the items from `from` on
-        const fbc_u32 n = past < 0 ? s_bad[k] : 0xFu;
-        const int ord = past < 0 ? (int)(n >> 10) : from + (int)(past / (8 * NG));
-        const int wq = past < 0 ? (int)(n >> 7) & 7 : (int)(past / NG) & 7, g = past < 0 ? (int)(n >> 4) & 7 : (int)(past % NG);
-        const int item = blockIdx.x + ord * gridDim.x;
-        const int v = (item % P.mtiles) * 128 + (wq & 3) * 32 + lane;
-        const int pg = fbc_f3_row(v, P), q = v - pg * P.vw;
-        const bool inside = q < P.out_w && pg * G::R < P.out_h && ((n >> (lane >> 3)) & 1u);
-        const fbc_u32 mask = __ballot_sync(0xFFFFFFFFu, inside);
-        fbc_f3_redo<G>(P, mask, pg, q, G::R > 1 ? 0 : item / P.mtiles * G::NT, (wq >> 2) * (G::NT / 2) + 8 * g);
-    }
+    // the noted groups: the stores above came before the barrier
+    if (s_nbad > 0 && s_abort == 0) fbc_f3_redo_noted<G>(P, s_bad, s_nbad, s_bad_from);
 }

@@ -427,11 +427,11 @@ def test_more_recomputed_groups_than_a_block_notes():
     """NaN in most groups of pixels: past its list a block computes whole items again."""
     torch = torch_cuda()
     from paper_0911_3456_gb300.api import Plan
-    wl = inputs.random_case(7985, 402, 410, 4, 80, 2, 2, kind="int")
+    wl = inputs.random_case(7985, 702, 900, 4, 16, 2, 2, kind="int")
     x = wl.x.copy()
     x.reshape(-1)[::97] = np.nan
     p = Plan(x.shape, wl.w.shape)
-    p.set_variant("f32tc:nt=80,r=1,gc=8,jt=2,ru=2")
+    p.set_variant("f32tc:nt=16,r=1,gc=8,jt=2,ru=2")
     y = host(p.forward(dev(x, torch), dev(wl.w, torch)))
     assert p.device_status() == 0
     assert np.array_equal(y, oracle.fwd(x, wl.w), equal_nan=True)
