@@ -125,7 +125,7 @@ __device__ __forceinline__ void fbc_f32dw_body(const FbcF3DwParams& P) {
     if (warp >= 8 && warp < 8 + FBC_F3DW_CONV_WARPS) {
         // ------------------------------------------------------------ converters
         const int ct = threadIdx.x - 8 * 32;
-        float gb[G::KG][4], xb[G::KX][4];
+        float gb[G::KG][4], xb[G::KX][4], mb[G::MASK ? G::KG : 1][4];
         auto load = [&](int c) {
             const int v0 = c * G::KPX;
 #pragma unroll
@@ -141,10 +141,7 @@ __device__ __forceinline__ void fbc_f32dw_body(const FbcF3DwParams& P) {
                     f = __ldg(reinterpret_cast<const float4*>(P.g + o));
                     if constexpr (G::MASK) {
                         const float4 t = __ldg(reinterpret_cast<const float4*>(P.m + o));
-                        if (!(t.x > P.lo && t.x < P.hi)) f.x = 0.f;
-                        if (!(t.y > P.lo && t.y < P.hi)) f.y = 0.f;
-                        if (!(t.z > P.lo && t.z < P.hi)) f.z = 0.f;
-                        if (!(t.w > P.lo && t.w < P.hi)) f.w = 0.f;
+                        mb[k][0] = t.x; mb[k][1] = t.y; mb[k][2] = t.z; mb[k][3] = t.w;
                     }
                 }
                 gb[k][0] = f.x; gb[k][1] = f.y; gb[k][2] = f.z; gb[k][3] = f.w;
@@ -175,6 +172,13 @@ __device__ __forceinline__ void fbc_f32dw_body(const FbcF3DwParams& P) {
                 const int it = ct + k * G::NCT;
                 const int px = it / G::QG, q = it % G::QG;
                 if ((k + 1) * G::NCT <= G::KPX * G::QG || px < G::KPX) {
+                    if constexpr (G::MASK) {
+                        // not as they are loaded: a chunk's loads have the chunk before it to
+                        // land (500x341x16 * 64x5x4, clamped: 284 to 101 us; FMA kernel 227)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            if (!(mb[k][e] > P.lo && mb[k][e] < P.hi)) gb[k][e] = 0.f;
+                    }
                     look(gb[k]);
                     fbc_f3_put(gb[k], gd + (fbc_u32)(q >> 1) * G::GPLANE + (fbc_u32)px * 16u + (fbc_u32)(q & 1) * 8u,
                                (G::NB / 8) * G::GPLANE);

@@ -587,3 +587,23 @@ def test_24_bit_values_pass_unchanged(which, shape, spec, monkeypatch):
         assert np.count_nonzero(ref) > 0
         # dL/dw adds first and third parts before the second: 25 bits where the first was rounded up
         assert np.all(np.abs(got - ref) <= 2.0 ** -23 * np.abs(ref)) if op == "x_dw" else np.array_equal(got, ref)
+
+
+@pytest.mark.parametrize("shape", [(500, 341, 16, 64, 5, 4), (336, 396, 8, 64, 6, 2)])
+def test_clamped_dw_is_not_slower_than_the_fma_kernel(shape):
+    """Where a plan runs the masked dL/dw on the tensor cores (it took 1.2 and 1.5 times
+    the FMA kernel's time here, with every mask value waited for as it was loaded)."""
+    torch = torch_cuda()
+    from paper_0911_3456_gb300.api import Plan
+    H, W, D, N, fh, fw = shape
+    gen = torch.Generator(device="cuda").manual_seed(8200)
+    x = torch.rand((H, W, D), generator=gen, device="cuda")
+    w = torch.randn((N, fh, fw, D), generator=gen, device="cuda") / (fh * fw * D) ** 0.5
+    p = Plan(x.shape, w.shape, clamp=(0.0, 1.0))
+    y = p.forward(x, w)
+    g = torch.randn(p.out_shape, generator=gen, device="cuda")
+    p.backward(x, w, g, y, need_dx=False)
+    assert "f32tc" in p.info()["dw"]
+    fma = p.workspace(p.ws_bwd, x.device)
+    assert (_us(torch, lambda: p.backward(x, w, g, y, need_dx=False)) <=
+            _us(torch, lambda: p.backward(x, w, g, y, need_dx=False, ws=fma)))
