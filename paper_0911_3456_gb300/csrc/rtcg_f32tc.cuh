@@ -166,7 +166,12 @@ struct FbcF3Cfg {
     static constexpr int NPX = VA && PP == 2 ? LS + 1 : LS;         // pixels read per slab
     static constexpr int NIT = RU * NPX * QA;                // items per unit
     static constexpr int KA = (NIT + NCT - 1) / NCT;
-    static constexpr int PA = KA * WA <= 18 ? 4 : KA * WA <= 24 ? 3 : KA * WA <= 36 ? 2 : 1;   // units in registers
+    // Clamp masks stay beside their values until these are written (where both fit):
+    // compared as they were loaded, each load was waited for in turn (dL/dx of
+    // 2048x2048x4 * 4x8x8, clamped: 228 to 104 us; FMA kernel 182).
+    static constexpr bool LATE = MASK && 2 * KA * WA <= 72;
+    static constexpr int RA = KA * WA * (LATE ? 2 : 1);      // registers of a unit
+    static constexpr int PA = RA <= 18 ? 4 : RA <= 24 ? 3 : RA <= 36 ? 2 : 1;   // units in registers
     static constexpr int NBC = RU * S * 2 * NT;              // bank chunks per unit
     __device__ static __forceinline__ int tap_group(int u) { return NTG > 1 ? u % NTG : 0; }
     __device__ static __forceinline__ int channel_group(int u) { return NCG > 1 ? (u / NTG) % NCG : 0; }
@@ -454,7 +459,8 @@ __device__ __forceinline__ void fbc_f3_a_item(int it, int& k, int& px, int& sub)
 }
 
 template <class G>
-__device__ __forceinline__ void fbc_f3_load_a(const FbcF3Params& P, const FbcF3Pos<G>& j, int it, float (&v)[G::WA]) {
+__device__ __forceinline__ void fbc_f3_load_a(const FbcF3Params& P, const FbcF3Pos<G>& j, int it, float (&v)[G::WA],
+                                              float (&mv)[G::LATE ? G::WA : 1]) {
     const int cg = G::channel_group(j.u);
     int k, px, sub;
     fbc_f3_a_item<G>(it, k, px, sub);
@@ -488,7 +494,13 @@ __device__ __forceinline__ void fbc_f3_load_a(const FbcF3Params& P, const FbcF3P
         v[1] = f.y;
         v[2] = f.z;
         v[3] = f.w;
-        if constexpr (G::MASK) {
+        if constexpr (G::LATE) {
+            const float4 g = __ldg(reinterpret_cast<const float4*>(P.m + o));
+            mv[0] = g.x;
+            mv[1] = g.y;
+            mv[2] = g.z;
+            mv[3] = g.w;
+        } else if constexpr (G::MASK) {
             const float4 g = __ldg(reinterpret_cast<const float4*>(P.m + o));
             if (!(g.x > P.lo && g.x < P.hi)) v[0] = 0.f;
             if (!(g.y > P.lo && g.y < P.hi)) v[1] = 0.f;
@@ -502,7 +514,12 @@ __device__ __forceinline__ void fbc_f3_load_a(const FbcF3Params& P, const FbcF3P
             const int cc = col + e / G::CP, c = ch + e % G::CP;
             if (cc < 0 || cc >= P.in_w || c >= G::C) continue;
             const unsigned o = (unsigned)((row * P.in_w + cc) * G::C + c);
-            v[e] = fbc_f3_masked<G>(__ldg(P.x + o), P.m + o, P);
+            if constexpr (G::LATE) {
+                v[e] = __ldg(P.x + o);
+                mv[e] = __ldg(P.m + o);
+            } else {
+                v[e] = fbc_f3_masked<G>(__ldg(P.x + o), P.m + o, P);
+            }
         }
     }
 }
@@ -510,8 +527,14 @@ __device__ __forceinline__ void fbc_f3_load_a(const FbcF3Params& P, const FbcF3P
 // Item `it` of a unit into the A slot at dst; `all`: every thread has one in this pass
 // (no branch: the conversions of several passes interleave).
 template <class G>
-__device__ __forceinline__ void fbc_f3_put_a(int it, bool all, float (&v)[G::WA], fbc_u32 dst) {
+__device__ __forceinline__ void fbc_f3_put_a(const FbcF3Params& P, int it, bool all, float (&v)[G::WA],
+                                             const float (&mv)[G::LATE ? G::WA : 1], fbc_u32 dst) {
     if (!all && it >= G::NIT) return;
+    if constexpr (G::LATE) {
+#pragma unroll
+        for (int e = 0; e < G::WA; ++e)
+            if (!(mv[e] > P.lo && mv[e] < P.hi)) v[e] = 0.f;
+    }
     fbc_f3_up<G::ORD>(v);
     int k, px, sub;
     fbc_f3_a_item<G>(it, k, px, sub);
@@ -668,15 +691,15 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
         FbcF3Pos<G> ja, jn;      // unit being written, unit being loaded
         ja.start(P);
         jn = ja;
-        float abuf[G::PA][G::KA][G::WA];
-        auto load_a = [&](float (&buf)[G::KA][G::WA]) {
+        float abuf[G::PA][G::KA][G::WA], mbuf[G::PA][G::KA][G::LATE ? G::WA : 1];
+        auto load_a = [&](float (&buf)[G::KA][G::WA], float (&mask)[G::KA][G::LATE ? G::WA : 1]) {
             if (!jn.valid(P)) return;
 #pragma unroll
-            for (int k = 0; k < G::KA; ++k) fbc_f3_load_a<G>(P, jn, ct + k * G::NCT, buf[k]);
+            for (int k = 0; k < G::KA; ++k) fbc_f3_load_a<G>(P, jn, ct + k * G::NCT, buf[k], mask[k]);
             jn.next(P);
         };
 #pragma unroll
-        for (int s = 0; s < G::PA; ++s) load_a(abuf[s]);
+        for (int s = 0; s < G::PA; ++s) load_a(abuf[s], mbuf[s]);
         int as = 0;
         fbc_u32 aph = 0;
         bool ok = true;
@@ -688,12 +711,12 @@ __device__ __forceinline__ void fbc_f32tc_body(const FbcF3Params& P) {
                 const fbc_u32 dst = sbase + (fbc_u32)as * G::ASLOT;
 #pragma unroll
                 for (int k = 0; k < G::KA; ++k)
-                    fbc_f3_put_a<G>(ct + k * G::NCT, (k + 1) * G::NCT <= G::NIT, abuf[s][k], dst);
+                    fbc_f3_put_a<G>(P, ct + k * G::NCT, (k + 1) * G::NCT <= G::NIT, abuf[s][k], mbuf[s][k], dst);
                 fbc_fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) fbc_mbar_arrive(a_full0 + 8u * as);
                 if (++as == P.na) { as = 0; aph ^= 1; }
-                load_a(abuf[s]);
+                load_a(abuf[s], mbuf[s]);
                 ja.next(P);
             }
         }
