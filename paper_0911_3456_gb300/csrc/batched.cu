@@ -19,7 +19,7 @@
 // and its correlation, all independent, so that the CTAs of one image fill the SMs
 // that another leaves idle.  The persistent kernel takes the rest.  Measured on 24
 // images (205 GFLOP, GB300): 3750 us with the persistent kernel alone (0.68 of the
-// FP32 FMA peak), 1027 us with every image on the tensor cores.
+// FP32 FMA peak), 1019 us with every image on the tensor cores.
 #include <algorithm>
 #include <array>
 #include <cstdio>

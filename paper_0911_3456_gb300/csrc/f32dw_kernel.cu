@@ -66,9 +66,14 @@ size_t f3dw_ws_bytes(const DirectProblem& pr, const F3DwTile& t) {
 // its peak), and the tile: 64 filters per tile, 32 where the bank is no
 // wider; two planes of x per CTA where their accumulators fit in TMEM twice; as
 // many CTAs as fill whole rounds of the SMs.  Needs 16-byte rows of x and g.
-// Measured (GB300, us, FMA / this): 187x233x12 * 40x5x3 36 / 33, 256x256x8 * 64x9x9
-// 115 / 63, 256x256x16 * 64x7x7 128 / 67, 40x300x64 * 100x3x11 116 / 68, 512x512x32 *
-// 256x5x5 2148 / 1029, 2048x2048x4 * 4x8x8 3228 / 1795.
+// Measured (GB300, us, FMA / this): 187x233x12 * 40x5x3 34 / 28 (not taken; clamped 40 /
+// 31), 256x256x8 * 64x9x9 113 / 56 (137 / 70), 256x256x16 * 64x7x7 125 / 60 (151 / 60),
+// 40x300x64 * 100x3x11 112 / 59 (132 / 75), 512x512x32 * 256x5x5 2141 / 1034 (2597 / 1098),
+// 2048x2048x4 * 4x8x8 3223 / 1796 (7243 / 2016).  Of 130 drawn shapes it takes 82, four of
+// them wrongly, all with at most 16 filters, which fill half of a tile of 32 or less:
+// 756x191x16 * 8x2x7 36.9 / 37.4, 463x114x64 * 16x9x9 clamped 214 / 230, 666x254x16 *
+// 4x9x9 154 / 184, 254x72x16 * 16x11x11 27.5 / 35.6; lines that leave these out lose as
+// much on others (973x135x12 * 16x3x3 46 / 38, 51x1065x12 * 4x3x8 clamped 73 / 26).
 bool f3dw_wins(const DirectProblem& pr, int sm_count, F3DwTile* out) {
     const std::string sw = env_str("FBCORR_F32TC", "1");
     if (sw == "0" || pr.c % 4 || pr.nf % 4 || pr.c > 256) return false;

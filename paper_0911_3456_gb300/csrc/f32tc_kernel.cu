@@ -186,7 +186,7 @@ std::vector<F3Tile> f3_ranked(const DirectProblem& pr, int sm_count, double* bes
 // forward; 0.65 at size, in a batch) or 0.35 (dL/dx of the untuned tiles).  Measured
 // (us, FMA kernel / this one): 128x128x8 * 16x9x9 (0.3 GFLOP) 11 / 19, 187x233x12 *
 // 40x5x3 (0.6) 20 / 20, 256x256x8 * 64x9x9 (5.1) 115 / 34, 2048x2048x4 * 4x8x8 (8.5)
-// 180 / 103, 512x512x32 * 256x5x5 (106) 1935 / 428.
+// 180 / 92, 512x512x32 * 256x5x5 (106) 1935 / 428.
 // Beside other launches (shared) neither the launch nor the last round counts.
 bool f3_wins(const DirectProblem& pr, int sm_count, F3Tile* t, bool shared) {
     const std::string sw = env_str("FBCORR_F32TC", "1");

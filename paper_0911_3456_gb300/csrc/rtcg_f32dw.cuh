@@ -23,7 +23,7 @@
 // reads of A), four of them do 64 x 56 x 16 multiply-adds for a 7-wide filter: 600
 // FLOP per cycle and SM, where the FMA kernel reached 145.  256x256x16 * 64x7x7: 128 us
 // with the FMA kernel, 67 us with this one (reduction and the FMA kernel's empty
-// launch included); 512x512x32 * 256x5x5: 2148 and 1029.
+// launch included); 512x512x32 * 256x5x5: 2148 and 1039.
 //
 // A CTA takes one filter row i, NCOMB planes of x, one tap group, one tile of NB
 // filters and a run of chunks of KPX pixels.  A chunk is one accumulation chunk
