@@ -152,8 +152,9 @@ fbcorr_status_t fbcorr_plan_workspace_size(fbcorr_plan_t plan, size_t* fwd_bytes
 fbcorr_status_t fbcorr_plan_scratch_size(fbcorr_plan_t plan, size_t* fwd_bytes, size_t* bwd_bytes);
 
 /* y = epi(corr(x, w)).  x, w, y: device pointers as above; ws: device
- * workspace of at least the forward size (NULL allowed when it is zero).
- * y must not alias x, w or ws. */
+ * workspace of at least the forward size (NULL allowed when it is zero), which
+ * belongs to the call until it has run: calls that may overlap need one each
+ * (or, FP32 plans, NULL).  y must not alias x, w or ws. */
 fbcorr_status_t fbcorr_forward(fbcorr_plan_t plan, const float* x, const float* w, float* y,
                                void* ws, size_t ws_bytes, fbcorr_stream_t stream);
 
