@@ -1039,6 +1039,9 @@ fbcorr_status_t fbcorr_plan_candidates(fbcorr_plan_t p, char* buf, size_t cap) {
     } else {
         specs = tc_candidates(p->tc);
     }
+    for (const F3Tile& t : f3_candidates(fwd_problem(p), p->dev.sm_count, plan_orders(p),
+                                         p->dtype == FBCORR_F32 ? ~(size_t)0 : p->ws_fwd))
+        specs.push_back(f3_spec(t));
     std::string s;
     for (const auto& sp : specs) s += sp + "\n";
     if (s.size() + 1 > cap) return set_error(FBCORR_ERR_INVALID_ARG, "buffer too small (%zu bytes needed)", s.size() + 1);

@@ -316,14 +316,20 @@ fbcorr_status_t f3_run(const F3Launch& l, const DirectProblem& pr, const float* 
     return launch_dependent(l.kernel, dim3(l.grid), args, s);
 }
 
+std::vector<F3Tile> f3_candidates(const DirectProblem& pr, int sm_count, int ord, size_t ws_limit) {
+    if (env_str(ord == 3 ? "FBCORR_F32TC" : "FBCORR_TCPACK", "1") == "0") return {};
+    std::vector<F3Tile> tiles = f3_ranked(pr, sm_count, nullptr, false, ord);
+    tiles.erase(std::remove_if(tiles.begin(), tiles.end(), [&](const F3Tile& t) { return f3_ws_bytes(pr, t) > ws_limit; }),
+                tiles.end());
+    tiles.resize(std::min<size_t>(tiles.size(), 8));
+    return tiles;
+}
+
 fbcorr_status_t f3_tune(const DeviceInfo& dev, const DirectProblem& pr, cudaStream_t s, int* err_word, float* ms,
                         std::string* spec, int ord, size_t ws_limit) {
     spec->clear();
-    std::vector<F3Tile> tiles = f3_ranked(pr, dev.sm_count, nullptr, false, ord);
-    tiles.erase(std::remove_if(tiles.begin(), tiles.end(), [&](const F3Tile& t) { return f3_ws_bytes(pr, t) > ws_limit; }),
-                tiles.end());
-    if (env_str(ord == 3 ? "FBCORR_F32TC" : "FBCORR_TCPACK", "1") == "0" || tiles.empty()) return FBCORR_OK;
-    tiles.resize(std::min<size_t>(tiles.size(), 8));
+    const std::vector<F3Tile> tiles = f3_candidates(pr, dev.sm_count, ord, ws_limit);
+    if (tiles.empty()) return FBCORR_OK;
     std::vector<std::string> srcs;
     for (const F3Tile& t : tiles) srcs.push_back(f3_kernel_source(pr, t, f3_kernel_name(pr, t)));
     rtcg_precompile(srcs);

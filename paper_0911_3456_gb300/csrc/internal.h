@@ -259,7 +259,9 @@ bool f3_parse_spec(const std::string& s, F3Tile* t, int ord = 3);
 // Every tile the kernel takes the problem with (none: it does not), by the cost model, best first.
 std::vector<F3Tile> f3_ranked(const DirectProblem& pr, int sm_count, double* best_cycles, bool shared = false,
                               int ord = 3);
-// Time the model's first tiles on patterned buffers; *spec is empty when there are none.
+// The tiles that the tuner times, within ws_limit bytes of workspace.
+std::vector<F3Tile> f3_candidates(const DirectProblem& pr, int sm_count, int ord = 3, size_t ws_limit = ~(size_t)0);
+// Time them on patterned buffers; *spec is empty when there are none.
 fbcorr_status_t f3_tune(const DeviceInfo& dev, const DirectProblem& pr, cudaStream_t s, int* err_word, float* ms,
                         std::string* spec, int ord = 3, size_t ws_limit = ~(size_t)0);
 // The best rated tile, and whether the model expects it to be faster than the FP32 FMA kernels.

@@ -5,6 +5,10 @@ FP32 accumulator by at most one unit (2^-23) of the magnitude summed so far at e
 step, the chunk sums are added with ordinary rounding, and the products left out are
 below 2^-26: |error| <= (16 * 2^-23 + (chunks + 4) * 2^-24) * sum |x| |w|.
 """
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -624,3 +628,24 @@ def test_clamped_dx_is_not_slower_than_the_fma_kernel():
     small = torch.empty(16, dtype=torch.uint8, device="cuda")
     assert (_us(torch, lambda: p.backward(x, w, g, y, need_dw=False)) <=
             _us(torch, lambda: p.backward(x, w, g, y, need_dw=False, ws=small)))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16x3", "bf16"])
+def test_candidates_are_what_the_tuner_times(dtype, tmp_path):
+    """In a child process, whose log names every variant that is timed."""
+    torch_cuda()
+    code = ("import sys; from paper_0911_3456_gb300.api import Plan\n"
+            f"p = Plan((70, 90, 8), (16, 5, 5, 8), {dtype!r}); c = p.candidates()\n"
+            "for s in c:\n    if s.startswith(('f32tc', 'tcpack')): p.set_variant(s)\n"
+            "print(\"\\n\".join(c)); p.autotune()")
+    env = dict(os.environ, FBCORR_LOG="1", FBCORR_CACHE_DIR=str(tmp_path), FBCORR_TUNE_TOPK="3")
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=600, env=env,
+                       cwd=os.path.dirname(os.path.dirname(os.path.abspath(__file__))))
+    assert r.returncode == 0, r.stderr[-2000:]
+    names = ("f32tc:", "tcpack:")
+    listed = {s for s in r.stdout.split() if s.startswith(names)}
+    # an FP32 plan tunes dL/dx as well, after the forward's pick is logged
+    log = r.stderr.split("autotune fwd picked" if dtype == "f32" else "autotune picked")[0]
+    timed = {word.rstrip(":") for line in log.splitlines() if "autotune" in line for word in line.split()
+             if word.startswith(names)}
+    assert listed and listed == timed
