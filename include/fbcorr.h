@@ -370,8 +370,9 @@ fbcorr_status_t fbcorr_rtcg_check(const int64_t in_shape[3], const int64_t filt_
                                   size_t cap);
 
 /* Offline check of a snippet epilogue (no GPU): generate and compile the
- * forward kernel that fbcorr_plan_create_snippet would build for this shape and
- * dtype (the heuristic FP32 tile, or the default tcgen05 configuration).
+ * forward kernels that fbcorr_plan_create_snippet may build for this shape and
+ * dtype (the heuristic FP32 tile or the default tcgen05 configuration, and the
+ * f32tc or tcpack kernel where the cost model prefers it).
  * Status and log as fbcorr_rtcg_check. */
 fbcorr_status_t fbcorr_snippet_check(const int64_t in_shape[3], const int64_t filt_shape[4],
                                      fbcorr_dtype_t dtype, const char* expr, char* log, size_t cap);

@@ -559,19 +559,24 @@ fbcorr_status_t fbcorr_snippet_check(const int64_t in_shape[3], const int64_t fi
     FBC_TRY(validate_snippet(expr));
     std::string lg;
     fbcorr_status_t st;
+    fbcorr_plan tmp;
+    tmp.H = in_shape[0]; tmp.W = in_shape[1]; tmp.D = in_shape[2];
+    tmp.N = filt_shape[0]; tmp.fh = filt_shape[1]; tmp.fw = filt_shape[2];
+    tmp.Ho = tmp.H - tmp.fh + 1; tmp.Wo = tmp.W - tmp.fw + 1;
+    tmp.dtype = dtype;
+    tmp.epi = epi;
+    tmp.snippet = expr;
+    const DirectProblem fp = fwd_problem(&tmp);
     if (dtype == FBCORR_F32) {
-        fbcorr_plan tmp;
-        tmp.H = in_shape[0]; tmp.W = in_shape[1]; tmp.D = in_shape[2];
-        tmp.N = filt_shape[0]; tmp.fh = filt_shape[1]; tmp.fw = filt_shape[2];
-        tmp.Ho = tmp.H - tmp.fh + 1; tmp.Wo = tmp.W - tmp.fw + 1;
-        tmp.epi = epi;
-        tmp.snippet = expr;
-        const DirectProblem fp = fwd_problem(&tmp);
         const DirectTile t = direct_heuristic(fp, 200 * 1024, 148);
         st = rtcg_compile_only(direct_kernel_source(fp, t, kname_for("fbc_direct", fp, t)), &lg);
     } else {
         st = tc_snippet_check((int)in_shape[2], (int)filt_shape[2], dtype == FBCORR_BF16X3 ? 1 : 0, expr, &lg);
     }
+    // and the kernel of rtcg_f32tc.cuh where the model prefers it
+    F3Tile f3;
+    if (st == FBCORR_OK && (dtype == FBCORR_F32 ? f3_wins(fp, 152, &f3) : f3_wins_bf16(fp, 152, plan_orders(&tmp), ~(size_t)0, &f3)))
+        st = rtcg_compile_only(f3_kernel_source(fp, f3, f3_kernel_name(fp, f3)), &lg);
     if (st != FBCORR_OK && log && cap) snprintf(log, cap, "%s", lg.empty() ? fbcorr_last_error() : lg.c_str());
     return st;
 }

@@ -97,3 +97,14 @@ def test_left_out_products_are_below_two_to_the_minus_24():
     assert np.all(np.abs(x2 * w3) < 2.0 ** -25 * xw) and np.all(np.abs(x3 * w2) < 2.0 ** -25 * xw)
     left = np.abs(x2 * w3 + x3 * w2 + x3 * w3)
     assert np.all(left < 2.0 ** -24 * xw) and left[-3] > 2.0 ** -24.1 * xw[-3]
+
+
+@pytest.mark.parametrize("dtype,shape", [(0, (128, 140, 8, 64, 9, 9)), (1, (512, 512, 4, 32, 13, 13)),
+                                         (2, (512, 512, 4, 32, 13, 13))])
+def test_snippet_check_compiles_the_packed_kernels(dtype, shape, tmp_path, monkeypatch):
+    monkeypatch.setenv("FBCORR_DUMP_DIR", str(tmp_path))
+    H, W, D, N, fh, fw = shape
+    assert C.load().fbcorr_snippet_check(C.I64_3(H, W, D), C.I64_4(N, fh, fw, D), dtype, b"y > 0.f ? y : lo * y", None,
+                                         0) == 0
+    text = "".join(f.read_text() for f in tmp_path.iterdir())
+    assert len(list(tmp_path.iterdir())) == 2 and ("fbc_f32tc_f", "fbc_tcpack1_f", "fbc_tcpack2_f")[dtype] in text
