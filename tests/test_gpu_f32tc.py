@@ -291,14 +291,19 @@ def test_dx_non_finite_values_against_oracle(where, clamp, monkeypatch):
     assert np.array_equal(dx, ref, equal_nan=True)
 
 
-def _us(torch, f, calls=8, rounds=5):
-    """Least time of a call in back-to-back runs."""
+def _us(torch, f, calls=8, rounds=6):
+    """Least time of a call among others, from a graph: without the host's part."""
+    f()
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        for _ in range(calls):
+            f()
     best = float("inf")
     for _ in range(rounds + 1):            # the first round warms up
         a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         a.record()
-        for _ in range(calls):
-            f()
+        g.replay()
         b.record()
         b.synchronize()
         best = min(best, a.elapsed_time(b) / calls * 1e3)
